@@ -29,6 +29,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "pdd_device.cuh"
 #include "pdd_internal.h"
@@ -166,18 +167,22 @@ __device__ __forceinline__ void start_path(const PathArgs& a, unsigned long long
 #endif
 // Finish test of Algorithm 1: d(X_k) >= -c0 |sigma^T N| sqrt(h).
 template <class P, class T, int D>
-__device__ __forceinline__ bool should_finish(const PathState<T>& s, T thr0) {
+__device__ __forceinline__ bool outside(const T* x, T thr0) {
   T thr = thr0;
-  if (P::kAniso || P::kIsoScaled) thr = mul_rn(thr, P::template exit_scale<T>(s.x[0], s.x[1], s.x[2]));
+  if (P::kAniso || P::kIsoScaled) thr = mul_rn(thr, P::template exit_scale<T>(x[0], x[1], x[2]));
   if (sizeof(T) == 4 && PDD_EXIT_CENTRED) {
     // FP32: the distance to the unit box's faces is 1/2 - max_i |X_i - 1/2|,
     // one instruction fewer than the minimum over the 2D faces
-    T e = fmaxf(fabsf(sub_rn(s.x[0], T(0.5))), fabsf(sub_rn(s.x[1], T(0.5))));
-    if (D == 3) e = fmaxf(e, fabsf(sub_rn(s.x[2], T(0.5))));
+    T e = fmaxf(fabsf(sub_rn(x[0], T(0.5))), fabsf(sub_rn(x[1], T(0.5))));
+    if (D == 3) e = fmaxf(e, fabsf(sub_rn(x[2], T(0.5))));
     return e >= sub_rn(T(0.5), thr);
   }
-  const T m = (D == 3) ? face_distance(s.x[0], s.x[1], s.x[2]) : face_distance(s.x[0], s.x[1]);
+  const T m = (D == 3) ? face_distance(x[0], x[1], x[2]) : face_distance(x[0], x[1]);
   return m <= thr;
+}
+template <class P, class T, int D>
+__device__ __forceinline__ bool should_finish(const PathState<T>& s, T thr0) {
+  return outside<P, T, D>(s.x, thr0);
 }
 
 // Philox block `blk` of the lane's path.
@@ -186,6 +191,59 @@ __device__ __forceinline__ uint4 path_block(const PathArgs& a, uint32_t seg, uin
                                             uint32_t path, uint32_t node) {
   const SegArgs& sg = a.seg[MULTI ? seg : 0];
   return philox4x32_10(make_uint4(blk, path, node, sg.seed_hi), make_uint2(sg.key0, sg.key1));
+}
+
+// Gradient of the control grid at x.
+template <class T, int D>
+__device__ __forceinline__ void grid_gradient(const PathArgs& a, const LaneSeg<T>& ls,
+                                              const T* x, T* gv) {
+  unsigned* err = PDD_DEBUG_BOUNDS ? a.err : nullptr;
+  if (D == 2) {
+    if (UseCells<T, 2>::value)
+      grid_cells_2d<T>((const float4*)ls.grad, ls.gn, x[0], x[1], gv[0], gv[1], err);
+    else
+      grid_grad_2d<T>((const float2*)ls.grad, ls.gn, x[0], x[1], gv[0], gv[1], err);
+  } else {
+    if (UseCells<T, 3>::value)
+      grid_cells_3d<T>((const float4*)ls.grad, ls.gn, x[0], x[1], x[2], gv[0], gv[1], gv[2], err);
+    else
+      grid_grad_3d<T>((const float4*)ls.grad, ls.gn, x[0], x[1], x[2], gv[0], gv[1], gv[2], err);
+  }
+}
+
+// sigma dW.
+template <class P, class T, int D>
+__device__ __forceinline__ void noise(const Coef<T>& o, const T* dW, T* sdW) {
+  const T dW0 = dW[0], dW1 = dW[1];
+  if (P::kAniso) {  // sigma = sqrt(a) [[1, 0], [1/2, sqrt(3)/2]]
+    sdW[0] = mul_rn(o.sa, dW0);
+    sdW[1] = mul_rn(o.sa, fma_rn(T(0.86602540378443864676), dW1, mul_rn(T(0.5), dW0)));
+  } else if (P::kIsoScaled) {  // sigma = sa I
+    sdW[0] = mul_rn(o.sa, dW0);
+    sdW[1] = mul_rn(o.sa, dW1);
+  } else {
+    sdW[0] = dW0;
+    sdW[1] = dW1;
+  }
+  sdW[2] = (D == 3) ? dW[2] : T(0);
+}
+
+// grad v . sigma dW, the integrand of the control variate without its -Y.
+template <class T, int D>
+__device__ __forceinline__ T cv_dot(const T* gv, const T* sdW) {
+  T dot = fma_rn(gv[1], sdW[1], mul_rn(gv[0], sdW[0]));
+  if (D == 3) dot = fma_rn(gv[2], sdW[2], dot);
+  return dot;
+}
+
+// X_{k+1} = X_k + h b + sigma dW.  The drift's step is h b, or (h/2)(2 b) for
+// problems whose eval returns 2 b (the same product: halving h is exact).
+template <class P, class T, int D>
+__device__ __forceinline__ void advance(T* x, T h, const Coef<T>& o, const T* sdW) {
+  const T hb = P::kDriftHalf ? mul_rn(T(0.5), h) : h;
+  x[0] = add_rn(x[0], fma_rn(hb, o.b0, sdW[0]));
+  x[1] = add_rn(x[1], fma_rn(hb, o.b1, sdW[1]));
+  if (D == 3) x[2] = add_rn(x[2], fma_rn(hb, o.b2, sdW[2]));
 }
 
 // One Euler-Maruyama step (eq. F:E_M) with the Feynman-Kac weights and the
@@ -205,57 +263,23 @@ __device__ __forceinline__ void euler_step(const PathArgs& a, PathState<T>& s,
   // The cell-record gather depends only on X_k: it is issued before the
   // coefficients are evaluated, so its latency overlaps their arithmetic.
   T gv[3] = {T(0), T(0), T(0)};
-  if (CV == kCvGrid && use_cv) {
-    if (D == 2) {
-      if (UseCells<T, 2>::value)
-        grid_cells_2d<T>((const float4*)ls.grad, ls.gn, s.x[0], s.x[1], gv[0], gv[1],
-                         PDD_DEBUG_BOUNDS ? a.err : nullptr);
-      else
-        grid_grad_2d<T>((const float2*)ls.grad, ls.gn, s.x[0], s.x[1], gv[0], gv[1],
-                        PDD_DEBUG_BOUNDS ? a.err : nullptr);
-    } else {
-      if (UseCells<T, 3>::value)
-        grid_cells_3d<T>((const float4*)ls.grad, ls.gn, s.x[0], s.x[1], s.x[2], gv[0], gv[1],
-                         gv[2], PDD_DEBUG_BOUNDS ? a.err : nullptr);
-      else
-        grid_grad_3d<T>((const float4*)ls.grad, ls.gn, s.x[0], s.x[1], s.x[2], gv[0], gv[1],
-                        gv[2], PDD_DEBUG_BOUNDS ? a.err : nullptr);
-    }
-  }
+  if (CV == kCvGrid && use_cv) grid_gradient<T, D>(a, ls, s.x, gv);
   Coef<T> o;
   P::template eval<T, CV == kCvExact>(s.x[0], s.x[1], s.x[2], o);
   T sdW[3];
-  const T dW0 = dW[0], dW1 = dW[1];
-  if (P::kAniso) {  // sigma = sqrt(a) [[1, 0], [1/2, sqrt(3)/2]]
-    sdW[0] = mul_rn(o.sa, dW0);
-    sdW[1] = mul_rn(o.sa, fma_rn(T(0.86602540378443864676), dW1, mul_rn(T(0.5), dW0)));
-  } else if (P::kIsoScaled) {  // sigma = sa I
-    sdW[0] = mul_rn(o.sa, dW0);
-    sdW[1] = mul_rn(o.sa, dW1);
-  } else {
-    sdW[0] = dW0;
-    sdW[1] = dW1;
-  }
-  sdW[2] = (D == 3) ? dW[2] : T(0);
+  noise<P, T, D>(o, dW, sdW);
   if (use_cv) {
     if (CV == kCvExact) {
       gv[0] = o.g0;
       gv[1] = o.g1;
       gv[2] = o.g2;
     }
-    T dot = fma_rn(gv[1], sdW[1], mul_rn(gv[0], sdW[0]));
-    if (D == 3) dot = fma_rn(gv[2], sdW[2], dot);
-    kahan_add(s.XI, s.XIc, -s.Y, dot);
+    kahan_add(s.XI, s.XIc, -s.Y, cv_dot<T, D>(gv, sdW));
   }
   // h Y_k serves the Z increment and the Euler rule Y_k (1 - h c) = Y_k - (h Y_k) c
   const T hY = P::kUnitY ? T(0) : mul_rn(h, s.Y);
   if (!P::kUnitY) kahan_add(s.Z, s.Zc, -hY, o.f);
-  // the drift's step: h b, or (h/2)(2 b) for problems whose eval returns 2 b
-  // (the same product: halving h is exact)
-  const T hb = P::kDriftHalf ? mul_rn(T(0.5), h) : h;
-  s.x[0] = add_rn(s.x[0], fma_rn(hb, o.b0, sdW[0]));
-  s.x[1] = add_rn(s.x[1], fma_rn(hb, o.b1, sdW[1]));
-  if (D == 3) s.x[2] = add_rn(s.x[2], fma_rn(hb, o.b2, sdW[2]));
+  advance<P, T, D>(s.x, h, o, sdW);
   if (!P::kUnitY)
     s.Y = (YRULE && a.y_exp) ? mul_rn(s.Y, m_exp(mul_rn(-h, o.c))) : fma_rn(-hY, o.c, s.Y);
   s.k += 1;
@@ -422,11 +446,21 @@ __device__ __forceinline__ bool refill(const PathArgs& a, PathState<T>& s, LaneS
 // runs with all lanes busy instead of one lane at a time while the rest of
 // the warp waits.  Rings follow the record cache in dynamic shared memory.
 constexpr uint32_t kRing = 64;  // entries per warp (>= 2 x 32: a full batch plus one iteration)
+// The ring is two halves of 32 entries, each with its own field arrays, so
+// that the drain can park exits in the first half and work in the second.
 template <class T, int D>
 struct ExitRing {
-  static constexpr size_t kBytes = kRing * ((D + 3) * sizeof(T) + 4 * sizeof(uint32_t));
-  T* f;         // (D + 3) x kRing: X_0 .. X_(D-1), Y, Z, xi
-  uint32_t* u;  // 4 x kRing: k, node, path, segment | truncated << 31
+  static constexpr uint32_t kHalf = 32 * ((D + 3) * sizeof(T) + 4 * sizeof(uint32_t));
+  static constexpr size_t kBytes = 2 * kHalf;
+  char* base;
+  // fields of entry j, 32 apart: X_0 .. X_(D-1), Y, Z, xi
+  __device__ __forceinline__ T* f(uint32_t j) const {
+    return (T*)(base + (j >> 5) * kHalf) + (j & 31u);
+  }
+  // k, node, path, segment | truncated << 31
+  __device__ __forceinline__ uint32_t* u(uint32_t j) const {
+    return (uint32_t*)(base + (j >> 5) * kHalf + 32 * (D + 3) * sizeof(T)) + (j & 31u);
+  }
 };
 
 __host__ __device__ __forceinline__ size_t cache_bytes(uint32_t cache_nodes) {
@@ -436,26 +470,24 @@ __host__ __device__ __forceinline__ size_t cache_bytes(uint32_t cache_nodes) {
 
 template <class T, int D>
 __device__ __forceinline__ ExitRing<T, D> ring_of_warp(const PathArgs& a) {
-  char* base = (char*)s_cache + cache_bytes(a.cache_nodes) +
-               (size_t)(threadIdx.x >> 5) * ExitRing<T, D>::kBytes;
-  ExitRing<T, D> r;
-  r.f = (T*)base;
-  r.u = (uint32_t*)(base + kRing * (D + 3) * sizeof(T));
-  return r;
+  return {(char*)s_cache + cache_bytes(a.cache_nodes) +
+          (size_t)(threadIdx.x >> 5) * ExitRing<T, D>::kBytes};
 }
 
 template <class T, int D>
 __device__ __forceinline__ void ring_put(const ExitRing<T, D>& r, uint32_t j,
                                          const PathState<T>& s, bool trunc) {
+  T* f = r.f(j);
+  uint32_t* u = r.u(j);
 #pragma unroll
-  for (int d = 0; d < D; ++d) r.f[d * kRing + j] = s.x[d];
-  r.f[D * kRing + j] = s.Y;
-  r.f[(D + 1) * kRing + j] = s.Z - s.Zc;
-  r.f[(D + 2) * kRing + j] = s.XI - s.XIc;
-  r.u[j] = (uint32_t)s.k;
-  r.u[kRing + j] = s.node;
-  r.u[2 * kRing + j] = s.path;
-  r.u[3 * kRing + j] = s.seg | (trunc ? 0x80000000u : 0u);
+  for (int d = 0; d < D; ++d) f[d * 32] = s.x[d];
+  f[D * 32] = s.Y;
+  f[(D + 1) * 32] = s.Z - s.Zc;
+  f[(D + 2) * 32] = s.XI - s.XIc;
+  u[0] = (uint32_t)s.k;
+  u[32] = s.node;
+  u[64] = s.path;
+  u[96] = s.seg | (trunc ? 0x80000000u : 0u);
 }
 
 // Score and record `count` (<= 32) parked exits starting at ring slot `first`.
@@ -466,18 +498,20 @@ __device__ __forceinline__ void ring_drain(const PathArgs& a, const ExitRing<T, 
   const uint32_t lane = threadIdx.x & 31u;
   if (lane < count) {
     const uint32_t j = (first + lane) & (kRing - 1);
+    const T* f = r.f(j);
+    const uint32_t* u = r.u(j);
     PathState<T> e;
     e.x[0] = e.x[1] = e.x[2] = T(0);
 #pragma unroll
-    for (int d = 0; d < D; ++d) e.x[d] = r.f[d * kRing + j];
-    e.Y = r.f[D * kRing + j];
-    e.Z = r.f[(D + 1) * kRing + j];
-    e.XI = r.f[(D + 2) * kRing + j];
+    for (int d = 0; d < D; ++d) e.x[d] = f[d * 32];
+    e.Y = f[D * 32];
+    e.Z = f[(D + 1) * 32];
+    e.XI = f[(D + 2) * 32];
     e.Zc = e.XIc = T(0);
-    e.k = (int)r.u[j];
-    e.node = r.u[kRing + j];
-    e.path = r.u[2 * kRing + j];
-    const uint32_t st = r.u[3 * kRing + j];
+    e.k = (int)u[0];
+    e.node = u[32];
+    e.path = u[64];
+    const uint32_t st = u[96];
     e.seg = st & 0x7FFFFFFFu;
     finish_path<P, T, D, MULTI>(a, e, (st >> 31) != 0u);
   }
@@ -520,48 +554,14 @@ __device__ __forceinline__ void init_lane(const PathArgs& a, PathState<T>& s, La
   load_seg<T, D>(a.seg[0], ls);
 }
 
-// One ordinary iteration: STEPS / 2 Philox blocks, two steps each; the exit
-// test precedes every step.  `fin` / `trunc` report a path that ended.
-template <class P, class T, int CV, bool MULTI, int STEPS>
-__device__ __forceinline__ void iteration_2d(const PathArgs& a, PathState<T>& s,
-                                             const LaneSeg<T>& ls, bool active, bool& fin,
-                                             bool& trunc) {
-#pragma unroll
-  for (int half = 0; half < STEPS / 2; ++half) {
-    uint4 w = make_uint4(0, 0, 0, 0);
-    if (active && !fin) fin = should_finish<P, T, 2>(s, ls.thr0);
-    if (active && !fin) {
-      w = path_block<MULTI>(a, s.seg, (uint32_t)(s.k >> 1), s.path, s.node);
-      T n[3];
-      box_muller(w.x, w.y, n[0], n[1], ls.sqh);
-      n[2] = T(0);
-      euler_step<P, T, 2, CV, MULTI>(a, s, ls, n);
-      if (s.k >= ls.max_steps) fin = trunc = true;
-    }
-    if (active && !fin) fin = should_finish<P, T, 2>(s, ls.thr0);
-    if (active && !fin) {
-      T n[3];
-      box_muller(w.z, w.w, n[0], n[1], ls.sqh);
-      n[2] = T(0);
-      euler_step<P, T, 2, CV, MULTI>(a, s, ls, n);
-      if (s.k >= ls.max_steps) fin = trunc = true;
-    }
-  }
-}
-
-// Drain iterations.  Once the launch's cursor is exhausted a warp only
-// finishes the paths it holds; as lanes retire, the launch's time becomes the
-// serial latency of its longest paths, and a lone path spends most of each
-// step drawing its random numbers (Philox rounds, Box-Muller), which do not
-// depend on the path's state.  When at most half the lanes of a warp still
-// run a path, the idle lanes draw them: with A running lanes, every lane L
-// computes Philox block m = L / A of running lane L mod A (counted from that
-// lane's current block) and its four normals, and the running lanes then take
-// 2 * floor(32 / A) steps reading their normals from the helpers with warp
-// shuffles.  The values are the ones a lane would draw itself (same key,
-// same counter, same arithmetic), so results do not change.
-#ifndef PDD_TAIL_COOP
-#define PDD_TAIL_COOP 1
+// Running lanes of a warp at which it goes over to the drain (see Drain): 6,
+// 12, 16 and 20 in 2D took 3.38, 3.00, 2.88 and 3.05 ms on 256 nodes x 1,387
+// paths with the control variate; a 3D batch needs four lanes per path.
+#ifndef PDD_DRAIN_RUN_2D
+#define PDD_DRAIN_RUN_2D 16
+#endif
+#ifndef PDD_DRAIN_RUN_3D
+#define PDD_DRAIN_RUN_3D 8
 #endif
 
 // Position of the q-th (from 0) set bit of m, q < popc(m): the largest p
@@ -574,61 +574,257 @@ __device__ __forceinline__ int nth_set_bit(unsigned m, int q) {
   return p;
 }
 
-// Helper side: this lane's Philox block (block blk + m, m = lane / A, of
-// running lane lane % A, whose current block counter is `blk`) as four scaled
-// normals; lanes with lane / A >= blocks draw none.
-template <class T, bool MULTI>
-__device__ __forceinline__ void coop_draw(const PathArgs& a, const PathState<T>& s,
-                                          const LaneSeg<T>& ls, unsigned runm, int blocks,
-                                          uint32_t blk, T (&nv)[4]) {
-  const int lane = (int)(threadIdx.x & 31u), A = __popc(runm);
-  const int q = lane % A, m = lane / A;
-  const int owner = nth_set_bit(runm, q);
-  const uint32_t o_seg = __shfl_sync(kFull, s.seg, owner);
-  const uint32_t o_path = __shfl_sync(kFull, s.path, owner);
-  const uint32_t o_node = __shfl_sync(kFull, s.node, owner);
-  const uint32_t o_blk = __shfl_sync(kFull, blk, owner);
-  const T o_sqh = __shfl_sync(kFull, ls.sqh, owner);
-  nv[0] = nv[1] = nv[2] = nv[3] = T(0);
-  if (m < blocks) {
-    const uint4 w = path_block<MULTI>(a, o_seg, o_blk + (uint32_t)m, o_path, o_node);
-    box_muller(w.x, w.y, nv[0], nv[1], o_sqh);
-    box_muller(w.z, w.w, nv[2], nv[3], o_sqh);
+// The drain.  Once the launch's cursor is exhausted a warp only finishes the
+// paths it holds, and as lanes retire the launch's time becomes the serial
+// latency of its longest paths.  Of an Euler step only the position's own
+// recurrence (the drift and the noise) has to wait for the previous step;
+// the random numbers depend on the path's key alone, and the exit test, the
+// coefficients c and f and the control variate on one position each.  When at
+// most Drain::kMaxRun lanes of a warp still run a path, the warp takes S steps
+// of its A paths at a time, in four passes over its scratch:
+//   1. every lane draws a Philox block and its four scaled normals;
+//   2. lane q < A advances path q by S positions, without testing for the
+//      exit (what lies past it is not used), one multiply, one SFU call and
+//      two additions deep per step;
+//   3. every lane tests the exit at, and evaluates the coefficients and
+//      grad v . sigma dW of, one or two (path, step) pairs;
+//   4. lane q folds path q's steps up to its exit into Y, Z and xi, in order.
+// Path q and its state move to lane q whenever paths have ended.  Every value
+// comes from the operations of euler_step in their order, so a path's result
+// does not depend on where it ran.
+// What bounds it: alone, the chains of passes 2 and 4 (about 90 cycles a step
+// plain, 105 with the control variate; drawing the random numbers on idle
+// lanes and taking the whole step in order afterwards took 320 and 560);
+// with all of a chip's warps in it, the issue slots, most of which go to the
+// two chains' few lanes.  256 nodes x 1,387 paths at h = 1e-4: 2.95 -> 2.24 ms
+// plain, 4.79 -> 2.96 ms with the control variate; 10 paths per node in 3D,
+// 2.67 -> 1.40 ms.
+template <class T, int D>
+struct Drain {
+  static constexpr int kMaxRun = D == 2 ? PDD_DRAIN_RUN_2D : PDD_DRAIN_RUN_3D;
+  // 2D: a lane's block makes two steps of one path (4 scratch words each)
+  static constexpr int kLanes = ExitRing<T, D>::kHalf / (8 * sizeof(T)) < 32
+                                    ? ExitRing<T, D>::kHalf / (8 * sizeof(T))
+                                    : 32;
+  // Philox blocks and steps per path with A running paths (3D: 3 blocks make
+  // 4 steps, and a lane evaluates one step)
+  __device__ static int blocks(int A) { return D == 2 ? kLanes / A : 3 * (8 / A); }
+  __device__ static int steps(int A) { return D == 2 ? 2 * (kLanes / A) : 4 * (8 / A); }
+};
+static_assert(32 * 6 * sizeof(float) <= ExitRing<float, 3>::kHalf, "3D drain scratch");
+static_assert(32 * 6 * sizeof(double) <= ExitRing<double, 3>::kHalf, "3D drain scratch");
+
+// Scratch vectors of D words: 2D as one 2-word access, 3D A words apart.
+template <class T, int D>
+__device__ __forceinline__ void get_vec(const T* base, int step, int q, int A, T* v) {
+  if (D == 2) {
+    using V = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+    const V w = ((const V*)base)[step * A + q];
+    v[0] = w.x;
+    v[1] = w.y;
+    v[2] = T(0);
+  } else {
+    const T* p = base + 3 * step * A + q;
+    v[0] = p[0];
+    v[1] = p[A];
+    v[2] = p[2 * A];
+  }
+}
+template <class T, int D>
+__device__ __forceinline__ void put_vec(T* base, int step, int q, int A, T v0, T v1, T v2) {
+  if (D == 2) {
+    using V = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+    V w;
+    w.x = v0;
+    w.y = v1;
+    ((V*)base)[step * A + q] = w;
+  } else {
+    T* p = base + 3 * step * A + q;
+    p[0] = v0;
+    p[A] = v1;
+    p[2 * A] = v2;
   }
 }
 
-// 2D: block m of a running lane feeds its steps 2m and 2m + 1 (normals 4m ..
-// 4m + 3), so the lane's counter at the iteration start is even.
-template <class P, class T, int CV, bool MULTI>
-__device__ __forceinline__ void coop_iteration_2d(const PathArgs& a, PathState<T>& s,
-                                                  const LaneSeg<T>& ls, bool active,
-                                                  unsigned runm, bool& fin, bool& trunc) {
-  const unsigned lane = threadIdx.x & 31u;
-  const int A = __popc(runm), blocks = 32 / A;
-  T nv[4];
-  coop_draw<T, MULTI>(a, s, ls, runm, blocks, (uint32_t)s.k >> 1, nv);
-  const int r = __popc(runm & ((1u << lane) - 1u));  // rank among running lanes
-  bool run = active;
-  for (int m = 0; m < blocks; ++m) {
-    const int src = (r + A * m) & 31;
+template <class P, class T, int D, int CV, bool MULTI>
+__device__ __forceinline__ void drain(const PathArgs& a, const ExitRing<T, D> ring, RingCursor rc,
+                                   PathState<T> s, LaneSeg<T> ls, bool active) {
+  constexpr int kFold = 4;  // steps whose terms are read at once in pass 4
+  const int lane = (int)(threadIdx.x & 31u);
+  // the ring's first half parks the exits from here on, its second is scratch
+  if (rc.held > 0u) ring_drain<P, T, D, MULTI>(a, ring, rc.head - rc.held, rc.held);
+  uint32_t held = 0;
+  T* const nrm = (T*)(ring.base + ExitRing<T, D>::kHalf);  // scaled normals, then grad v . sigma dW
+  T* const pos = nrm + (D == 2 ? 4 * Drain<T, D>::kLanes : 96);  // X, then c, f (and the dot in 3D)
+  unsigned runm = __ballot_sync(kFull, active);
+  while (runm != 0u) {
+    // lane L takes path q = L mod A (its state in lanes L < A, its key and
+    // segment in every lane)
+    const int A = __popc(runm), q = lane % A, m = lane / A;
+    const int src = nth_set_bit(runm, q);
+    for (int d = 0; d < D; ++d) s.x[d] = __shfl_sync(kFull, s.x[d], src);
+    s.Y = __shfl_sync(kFull, s.Y, src);
+    s.Z = __shfl_sync(kFull, s.Z, src);
+    s.Zc = __shfl_sync(kFull, s.Zc, src);
+    s.XI = __shfl_sync(kFull, s.XI, src);
+    s.XIc = __shfl_sync(kFull, s.XIc, src);
+    s.k = __shfl_sync(kFull, s.k, src);
+    s.node = __shfl_sync(kFull, s.node, src);
+    s.path = __shfl_sync(kFull, s.path, src);
+    if (MULTI) {
+      s.seg = __shfl_sync(kFull, s.seg, src);
+      load_seg<T, D>(a.seg[s.seg], ls);
+    }
+    const SegArgs& sg = a.seg[MULTI ? s.seg : 0];
+    const uint32_t key0 = sg.key0, key1 = sg.key1, seed_hi = sg.seed_hi;
+    const bool use_cv = CV != kCvNone && (CV != kCvGrid || !MULTI || ls.grad != nullptr);
+    const bool y_exp = MULTI && a.y_exp;
+    const int blocks = Drain<T, D>::blocks(A), S = Drain<T, D>::steps(A);
+    unsigned mine = 0u;  // the lanes of path q
+    for (int l = q; l < 32; l += A) mine |= 1u << l;
+    unsigned endm = 0u;
+    bool trunc = false;
+    do {
+      // 1. random numbers
+      if (m < blocks) {
+        const uint32_t blk0 = D == 2 ? (uint32_t)s.k >> 1 : 3u * ((uint32_t)s.k >> 2);
+        // (the empty asm keeps the ten rounds' keys from living in registers
+        // across the batches: 20 of them with per-lane keys)
+        uint2 key = make_uint2(key0, key1);
+        if (MULTI) asm volatile("" : "+r"(key.x), "+r"(key.y));
+        const uint4 w = philox4x32_10(make_uint4(blk0 + (uint32_t)m, s.path, s.node, seed_hi), key);
+        T n[4];
+        box_muller(w.x, w.y, n[0], n[1], ls.sqh);
+        box_muller(w.z, w.w, n[2], n[3], ls.sqh);
+        if (D == 2) {
+          put_vec<T, D>(nrm, 2 * m, q, A, n[0], n[1], T(0));
+          put_vec<T, D>(nrm, 2 * m + 1, q, A, n[2], n[3], T(0));
+        } else {
 #pragma unroll
-    for (int h2 = 0; h2 < 2; ++h2) {
-      T n[3];
-      n[0] = __shfl_sync(kFull, nv[2 * h2], src);
-      n[1] = __shfl_sync(kFull, nv[2 * h2 + 1], src);
-      n[2] = T(0);
-      if (run) run = !should_finish<P, T, 2>(s, ls.thr0);
-      if (run) {
-        euler_step<P, T, 2, CV, MULTI>(a, s, ls, n);
-        if (s.k >= ls.max_steps) {
-          trunc = true;
-          run = false;
+          for (int c = 0; c < 4; ++c) nrm[(4 * m + c) * A + q] = n[c];
         }
       }
+      __syncwarp();
+      // 2. positions (S is even; the normals are read two steps ahead)
+      if (lane < A) {
+        T dW[2][3], next[2][3];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) get_vec<T, D>(nrm, j, q, A, dW[j]);
+#pragma unroll 1
+        for (int i = 0; i < S; i += 2) {
+          const int ahead = min(i + 2, S - 2);
+#pragma unroll
+          for (int j = 0; j < 2; ++j) get_vec<T, D>(nrm, ahead + j, q, A, next[j]);
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            put_vec<T, D>(pos, i + j, q, A, s.x[0], s.x[1], s.x[2]);
+            Coef<T> o;
+            P::template eval<T, false>(s.x[0], s.x[1], s.x[2], o);
+            T sdW[3];
+            noise<P, T, D>(o, dW[j], sdW);
+            advance<P, T, D>(s.x, ls.h, o, sdW);
+#pragma unroll
+            for (int d = 0; d < D; ++d) dW[j][d] = next[j][d];
+          }
+        }
+      }
+      __syncwarp();
+      // 3. exit tests, then coefficients of the steps before the exit
+      constexpr int kItems = D == 2 ? 2 : 1;  // (path, step) pairs per lane
+      unsigned f[kItems];
+#pragma unroll
+      for (int j = 0; j < kItems; ++j) {
+        const int i = kItems * m + j;
+        bool fin = false;
+        if (i < S) {
+          T x[3];
+          get_vec<T, D>(pos, i, q, A, x);
+          fin = outside<P, T, D>(x, ls.thr0);
+        }
+        f[j] = __ballot_sync(kFull, fin) & mine;
+      }
+      int n = S;  // steps path q takes
+      const unsigned any = f[0] | f[kItems - 1];
+      if (any != 0u) {
+        const int l = __ffs(any) - 1;
+        n = kItems * (l / A) + ((f[0] >> l) & 1u ? 0 : 1);
+      }
+      trunc = n >= ls.max_steps - s.k;
+      if (trunc) n = ls.max_steps - s.k;
+#pragma unroll
+      for (int j = 0; j < kItems; ++j) {
+        const int i = kItems * m + j;
+        if (i < n) {
+          T x[3];
+          get_vec<T, D>(pos, i, q, A, x);
+          T gv[3] = {T(0), T(0), T(0)}, dot = T(0);
+          if (CV == kCvGrid && use_cv) grid_gradient<T, D>(a, ls, x, gv);
+          Coef<T> o;
+          P::template eval<T, CV == kCvExact>(x[0], x[1], x[2], o);
+          if (use_cv) {
+            T dW[3], sdW[3];
+            get_vec<T, D>(nrm, i, q, A, dW);
+            noise<P, T, D>(o, dW, sdW);
+            if (CV == kCvExact) {
+              gv[0] = o.g0;
+              gv[1] = o.g1;
+              gv[2] = o.g2;
+            }
+            dot = cv_dot<T, D>(gv, sdW);
+          }
+          const T c = y_exp ? m_exp(mul_rn(-ls.h, o.c)) : o.c;
+          put_vec<T, D>(pos, i, q, A, c, o.f, dot);
+          if (D == 2 && use_cv) nrm[2 * (i * A + q)] = dot;
+        }
+      }
+      __syncwarp();
+      // 4. Y, Z and xi
+      if (lane < A) {
+        auto fold = [&](const T* v, T dot) {
+          if (use_cv) kahan_add(s.XI, s.XIc, -s.Y, dot);
+          if (!P::kUnitY) {
+            const T hY = mul_rn(ls.h, s.Y);
+            kahan_add(s.Z, s.Zc, -hY, v[1]);
+            s.Y = y_exp ? mul_rn(s.Y, v[0]) : fma_rn(-hY, v[0], s.Y);
+          }
+        };
+        auto read = [&](int i, T* v) {
+          get_vec<T, D>(pos, i, q, A, v);
+          if (D == 2 && use_cv) v[2] = nrm[2 * (i * A + q)];
+        };
+        int i = 0;
+#pragma unroll 1
+        for (; i + kFold <= n; i += kFold) {
+          T v[kFold][3];
+#pragma unroll
+          for (int j = 0; j < kFold; ++j) read(i + j, v[j]);
+#pragma unroll
+          for (int j = 0; j < kFold; ++j) fold(v[j], v[j][2]);
+        }
+#pragma unroll 1
+        for (; i < n; ++i) {
+          T v[3];
+          read(i, v);
+          fold(v, v[2]);
+        }
+        if (n < S) get_vec<T, D>(pos, n, q, A, s.x);  // X at the exit
+      }
+      s.k += n;
+      endm = __ballot_sync(kFull, lane < A && (trunc || n < S));
+      __syncwarp();
+    } while (endm == 0u);
+    // park the exits
+    const uint32_t ended = (uint32_t)__popc(endm);
+    if (held + ended > 32u) {
+      ring_drain<P, T, D, MULTI>(a, ring, 0u, held);
+      held = 0;
     }
-    if (__ballot_sync(kFull, run) == 0u) break;
+    if ((endm >> lane) & 1u)
+      ring_put<T, D>(ring, held + (uint32_t)__popc(endm & ((1u << lane) - 1u)), s, trunc);
+    held += ended;
+    runm = ((1u << A) - 1u) & ~endm;
   }
-  fin = active && !run;
+  if (held > 0u) ring_drain<P, T, D, MULTI>(a, ring, 0u, held);
 }
 
 // The segment-table build keeps per-lane segment parameters in registers; at
@@ -636,8 +832,7 @@ __device__ __forceinline__ void coop_iteration_2d(const PathArgs& a, PathState<T
 // block fits an SM, so it is capped at 64 (two blocks), which measured faster
 // than the uncapped build.
 template <class P, class T, int CV, bool MULTI, int STEPS>
-__global__ void __launch_bounds__(kMaxBlockThreads, (MULTI && sizeof(T) == 4) ? 2
-                                                                               : PDD_MIN_BLOCKS_2D)
+__global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_2D)
     paths_2d(const __grid_constant__ PathArgs a) {
   PathState<T> s;
   LaneSeg<T> ls;
@@ -648,10 +843,9 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (MULTI && sizeof(T) == 4) ? 
   bool active = false, exhausted = false;
   unsigned long long bnext = 0, bend = 0;
   while (refill<T, 2, MULTI>(a, s, ls, active, bnext, bend, exhausted)) {
-    if (PDD_TAIL_COOP && exhausted) break;  // warp-uniform: on to the drain
+    // warp-uniform: few paths left, on to the drain
+    if (exhausted && __popc(__ballot_sync(kFull, active)) <= Drain<T, 2>::kMaxRun) break;
     bool fin = false, trunc = false;
-    // the body of iteration_2d, written out: inlining the function here
-    // changes the compiler's schedule of this loop (measured slower)
 #pragma unroll
     for (int half = 0; half < STEPS / 2; ++half) {
       uint4 w = make_uint4(0, 0, 0, 0);
@@ -676,16 +870,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (MULTI && sizeof(T) == 4) ? 
     ring_exit<P, T, 2, MULTI>(a, ring, rc, s, active && fin, trunc);
     if (fin) active = false;
   }
-  // drain: the cursor is exhausted and the warp finishes the paths it holds
-  while (PDD_TAIL_COOP && exhausted) {
-    const unsigned runm = __ballot_sync(kFull, active);
-    if (runm == 0u) break;
-    bool fin = false, trunc = false;
-    coop_iteration_2d<P, T, CV, MULTI>(a, s, ls, active, runm, fin, trunc);
-    ring_exit<P, T, 2, MULTI>(a, ring, rc, s, active && fin, trunc);
-    if (fin) active = false;
-  }
-  if (rc.held > 0u) ring_drain<P, T, 2, MULTI>(a, ring, rc.head - rc.held, rc.held);
+  drain<P, T, 2, CV, MULTI>(a, ring, rc, s, ls, active);
   cache_flush(a);
 }
 
@@ -694,97 +879,6 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (MULTI && sizeof(T) == 4) ? 
 //   step 0: a0 a1 a2   step 1: a3 b0 b1   step 2: b2 b3 c0   step 3: c1 c2 c3
 // Blocks are drawn only when the path is still running.  STEPS / 4 such
 // groups of four steps run per iteration (between lane refills).
-// One ordinary 3D iteration runs STEPS / 4 such groups; the exit test
-// precedes every step.
-template <class P, class T, int CV, bool MULTI, int STEPS>
-__device__ __forceinline__ void iteration_3d(const PathArgs& a, PathState<T>& s,
-                                             const LaneSeg<T>& ls, bool active, bool& fin,
-                                             bool& trunc) {
-#pragma unroll
-  for (int quad = 0; quad < STEPS / 4; ++quad) {
-    T carry0 = T(0), carry1 = T(0);  // normals left over from the previous block
-    uint4 w = make_uint4(0, 0, 0, 0);
-    const uint32_t blk0 = 3u * ((uint32_t)s.k >> 2);
-    // step 0
-    if (active && !fin) fin = should_finish<P, T, 3>(s, ls.thr0);
-    if (active && !fin) {
-      w = path_block<MULTI>(a, s.seg, blk0, s.path, s.node);
-      T n[3], n3;
-      box_muller(w.x, w.y, n[0], n[1], ls.sqh);
-      box_muller(w.z, w.w, n[2], n3, ls.sqh);
-      carry0 = n3;
-      euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-      if (s.k >= ls.max_steps) fin = trunc = true;
-    }
-    // step 1
-    if (active && !fin) fin = should_finish<P, T, 3>(s, ls.thr0);
-    if (active && !fin) {
-      w = path_block<MULTI>(a, s.seg, blk0 + 1u, s.path, s.node);
-      T n[3];
-      n[0] = carry0;
-      box_muller(w.x, w.y, n[1], n[2], ls.sqh);
-      euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-      if (s.k >= ls.max_steps) fin = trunc = true;
-    }
-    // step 2
-    if (active && !fin) fin = should_finish<P, T, 3>(s, ls.thr0);
-    if (active && !fin) {
-      T n[3];
-      box_muller(w.z, w.w, n[0], n[1], ls.sqh);
-      w = path_block<MULTI>(a, s.seg, blk0 + 2u, s.path, s.node);
-      box_muller(w.x, w.y, n[2], carry1, ls.sqh);
-      euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-      if (s.k >= ls.max_steps) fin = trunc = true;
-    }
-    // step 3
-    if (active && !fin) fin = should_finish<P, T, 3>(s, ls.thr0);
-    if (active && !fin) {
-      T n[3];
-      n[0] = carry1;
-      box_muller(w.z, w.w, n[1], n[2], ls.sqh);
-      euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-      if (s.k >= ls.max_steps) fin = trunc = true;
-    }
-  }
-}
-
-// The 3D drain iteration: a running lane's block counter at the iteration
-// start is 3 k / 4 (k a multiple of four); with A <= 10 running lanes each
-// takes 4 * floor(floor(32 / A) / 3) steps, normal i of a group of four steps
-// coming from helper block i / 4 of that group, word i mod 4.
-template <class P, class T, int CV, bool MULTI>
-__device__ __forceinline__ void coop_iteration_3d(const PathArgs& a, PathState<T>& s,
-                                                  const LaneSeg<T>& ls, bool active,
-                                                  unsigned runm, bool& fin, bool& trunc) {
-  const unsigned lane = threadIdx.x & 31u;
-  const int A = __popc(runm), quads = (32 / A) / 3;
-  T nv[4];
-  coop_draw<T, MULTI>(a, s, ls, runm, 3 * quads, 3u * ((uint32_t)s.k >> 2), nv);
-  const int r = __popc(runm & ((1u << lane) - 1u));
-  bool run = active;
-  for (int j = 0; j < quads; ++j) {
-#pragma unroll
-    for (int st = 0; st < 4; ++st) {
-      T n[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const int i = 3 * st + c;  // normal index within the group of four steps
-        n[c] = __shfl_sync(kFull, nv[i & 3], (r + A * (3 * j + (i >> 2))) & 31);
-      }
-      if (run) run = !should_finish<P, T, 3>(s, ls.thr0);
-      if (run) {
-        euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-        if (s.k >= ls.max_steps) {
-          trunc = true;
-          run = false;
-        }
-      }
-    }
-    if (__ballot_sync(kFull, run) == 0u) break;
-  }
-  fin = active && !run;
-}
-
 template <class P, class T, int CV, bool MULTI, int STEPS>
 __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
     paths_3d(const __grid_constant__ PathArgs a) {
@@ -796,14 +890,9 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
   RingCursor rc;
   bool active = false, exhausted = false;
   unsigned long long bnext = 0, bend = 0;
-  // The ordinary iterations run until the cursor is exhausted and at most
-  // ten lanes of the warp still run a path (warp-uniform); then drain
-  // iterations alternate with the check.
-  for (;;) {
   while (refill<T, 3, MULTI>(a, s, ls, active, bnext, bend, exhausted)) {
-    if (PDD_TAIL_COOP && exhausted && __popc(__ballot_sync(kFull, active)) <= 10) break;
+    if (exhausted && __popc(__ballot_sync(kFull, active)) <= Drain<T, 3>::kMaxRun) break;
     bool fin = false, trunc = false;
-    // the body of iteration_3d, written out (as in paths_2d)
 #pragma unroll
     for (int quad = 0; quad < STEPS / 4; ++quad) {
       T carry0 = T(0), carry1 = T(0);  // normals left over from the previous block
@@ -853,14 +942,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
     ring_exit<P, T, 3, MULTI>(a, ring, rc, s, active && fin, trunc);
     if (fin) active = false;
   }
-  const unsigned runm = __ballot_sync(kFull, active);
-  if (!PDD_TAIL_COOP || runm == 0u) break;
-  bool fin = false, trunc = false;
-  coop_iteration_3d<P, T, CV, MULTI>(a, s, ls, active, runm, fin, trunc);
-  ring_exit<P, T, 3, MULTI>(a, ring, rc, s, active && fin, trunc);
-  if (fin) active = false;
-  }
-  if (rc.held > 0u) ring_drain<P, T, 3, MULTI>(a, ring, rc.head - rc.held, rc.held);
+  drain<P, T, 3, CV, MULTI>(a, ring, rc, s, ls, active);
   cache_flush(a);
 }
 
@@ -1063,7 +1145,12 @@ static size_t plan_cache(PathArgs& b) {
   b.cache_nodes = base;
   return cache_bytes(base);
 }
-constexpr int kCacheBlockThreads = 512;  // default block size of cached launches
+// Default block size of launches with the record cache: large, so that many
+// warps share one copy of the records, and two blocks to an SM where that
+// costs few warps (up to 64 registers a thread: 512 threads, 72: 448, which
+// measured 23.0 -> 16.6 ms on 512 nodes x 10-step paths against one block of
+// 512; the coupled kernels, above 72, are faster with one).
+static int cache_block_threads(int regs) { return regs > 64 && regs <= 72 ? 448 : 512; }
 
 // Persistent launch of `kern` over the flat index space of `a`: occupancy x
 // SM count blocks (at most one warp per 32 paths), with the record cache
@@ -1111,8 +1198,19 @@ static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cud
   PathArgs b = a;
   b.warp_batch = kWarpBatch * (unsigned long long)resolve_claim(a, num_sms);
   const size_t cache = plan_cache(b);
-  const int threads =
-      a.block_threads > 0 ? a.block_threads : (cache > 0 ? kCacheBlockThreads : kBlockThreads);
+  int threads = a.block_threads > 0 ? a.block_threads : kBlockThreads;
+  if (a.block_threads <= 0 && cache > 0) {
+    // occ_cache[0] keeps the kernel's register count (block sizes start at 32)
+    int regs = occ_cache[0].load(std::memory_order_relaxed);
+    if (regs == 0) {
+      cudaFuncAttributes fa;
+      cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+      if (e != cudaSuccess) return e;
+      regs = fa.numRegs > 0 ? fa.numRegs : 1;
+      occ_cache[0].store(regs, std::memory_order_relaxed);
+    }
+    threads = cache_block_threads(regs);
+  }
   if (threads % 32 != 0 || threads > kMaxBlockThreads) return cudaErrorInvalidValue;
   const size_t smem = cache + (size_t)(threads / 32) * ring_per_warp;
   if (smem > 48u * 1024u && (int)smem > attr_set->load(std::memory_order_relaxed)) {

@@ -1,0 +1,57 @@
+"""Paths finished in the drain's batches equal the same paths run in ordinary iterations.
+
+The drain takes a warp's last paths S steps at a time, S depending on how many
+paths the warp still holds, and finds the exits and the truncations afterwards.
+One warp is given every number of paths here, with caps on the steps that fall at the
+start, inside and at the end of a batch; the same paths of a launch of many
+are issued first and run in the ordinary iterations.  Everything is compared
+bit for bit.
+"""
+import numpy as np
+import pytest
+
+from paper_1512_02818_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1512_02818_gb300 import build, pdd
+    build.build()
+    ctx = pdd.Context(0)
+    yield torch, pdd, ctx
+    ctx.close()
+
+
+KINDS = {"cfg0": (0, 129), "aniso": (1, 129), "cube": (2, 33), "harmonic": (3, 129), "paper": (4, 129)}
+
+
+@pytest.mark.parametrize("kind,precision,y_exp,cv", [
+    ("cfg0", 0, 0, "grid"), ("cfg0", 0, 1, "none"), ("cfg0", 1, 0, "grid"), ("aniso", 0, 0, "grid"),
+    ("paper", 0, 1, "grid"), ("harmonic", 0, 0, "exact"), ("cube", 0, 0, "grid"),
+    ("cube", 0, 0, "none"), ("cube", 1, 0, "grid"), ("cfg0", 0, 0, "exact")])
+def test_every_count_and_cap(env, kind, precision, y_exp, cv):
+    torch, pdd, ctx = env
+    k, grid = KINDS[kind]
+    node = np.full((1, 3 if kind == "cube" else 2), 0.5, np.float32)
+    many = 40_000 if precision == 0 else 4_000
+    for cap in (0, 37, 64):
+        prob = pdd.Problem(ctx, k, y_rule=y_exp, precision=precision, max_steps=cap)
+        gid = {"none": pdd.PDD_CV_NONE, "exact": pdd.PDD_CV_EXACT, "grid": 0}[cv]
+        if cv == "grid":
+            prob.set_control_grid(0, W.control_grid(k, grid, 1e-1))
+        big = prob.estimate(node, many, 2e-3, grid_id=gid, emit_paths=True)
+        ctx.set_claim(1)
+        try:
+            for n in (1, 2, 3, 5, 7, 8, 9, 11, 15, 16, 17, 20, 32):
+                small = prob.estimate(node, n, 2e-3, grid_id=gid, emit_paths=True)
+                for f in ("phi", "xi", "steps"):
+                    assert torch.equal(small[f], big[f][:, :n]), (cap, n, f)
+        finally:
+            ctx.set_claim(0)
+        prob.close()
+
