@@ -74,6 +74,8 @@ struct PathArgs {
   int iter_mode;               // Euler steps per iteration: PDD_ITER_AUTO / _SHORT / _LONG
   int claim;                   // paths per lane a warp claims from the cursor at once (0: auto)
   unsigned long long warp_batch;  // path indices a warp claims at once; set by the launcher
+  int one_claim;               // every warp starts one batch of its own (spread launches); set by
+                               // the launcher
   int n_segs;                  // 1 .. kMaxSegments; segments in increasing `begin`
   uint32_t cache_nodes;        // record slots cached in shared memory per block (0: none);
                                // set by the launchers

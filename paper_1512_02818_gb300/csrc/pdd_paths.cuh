@@ -438,6 +438,19 @@ __device__ __forceinline__ bool refill(const PathArgs& a, PathState<T>& s, LaneS
   return __ballot_sync(kFull, active) != 0u;
 }
 
+// Spread launches (see spread_batch): every warp has a batch of its own, and
+// the cursor is past the last path when the warp asks it for more.
+__device__ __forceinline__ void spread_claim(const PathArgs& a, unsigned long long& bnext,
+                                             unsigned long long& bend) {
+  if (a.one_claim == 0) return;
+  // (the shuffle tells the compiler that the batch is the warp's: without it
+  // the kernels take 20 registers more)
+  const unsigned warp = __shfl_sync(kFull, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, 0);
+  bnext = min(warp * a.warp_batch, a.total);
+  bend = min(bnext + a.warp_batch, a.total);
+  if ((threadIdx.x & 31u) == 0u) atomicAdd(a.cursor, a.total);
+}
+
 // Per-warp exit ring.  A lane whose path has ended parks the path's final
 // state (X, Y, Z, xi, k, node, path, segment | truncated) in its warp's ring
 // in shared memory and takes a new path at once; whenever 32 exits are
@@ -842,6 +855,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_2D)
   RingCursor rc;
   bool active = false, exhausted = false;
   unsigned long long bnext = 0, bend = 0;
+  spread_claim(a, bnext, bend);
   while (refill<T, 2, MULTI>(a, s, ls, active, bnext, bend, exhausted)) {
     // warp-uniform: few paths left, on to the drain
     if (exhausted && __popc(__ballot_sync(kFull, active)) <= Drain<T, 2>::kMaxRun) break;
@@ -890,6 +904,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
   RingCursor rc;
   bool active = false, exhausted = false;
   unsigned long long bnext = 0, bend = 0;
+  spread_claim(a, bnext, bend);
   while (refill<T, 3, MULTI>(a, s, ls, active, bnext, bend, exhausted)) {
     if (exhausted && __popc(__ballot_sync(kFull, active)) <= Drain<T, 3>::kMaxRun) break;
     bool fin = false, trunc = false;
@@ -1155,7 +1170,9 @@ static int cache_block_threads(int regs) { return regs > 64 && regs <= 72 ? 448 
 // Persistent launch of `kern` over the flat index space of `a`: occupancy x
 // SM count blocks (at most one warp per 32 paths), with the record cache
 // when the launch's nodes fit it and `ring_per_warp` bytes of exit ring per
-// warp.  `attr_set` / `occ_cache` are the kernel's own (static) state: the
+// warp.  `spread` > 0: that many paths per warp (see spread_batch), in blocks
+// of 128 threads so that the warps cover the SMs evenly.  `attr_set` /
+// `occ_cache` are the kernel's own (static) state: the
 // dynamic shared memory limit set so far and the occupancy per block size
 // without the cache.
 static bool long_iterations(const PathArgs& a) {
@@ -1191,15 +1208,38 @@ static int resolve_claim(const PathArgs& a, int num_sms) {
   return (longer <= kShortWorkShare * all && a.total >= enough) ? kAutoClaim : 1;
 }
 
+// Paths per warp of a launch too small to fill the chip, 0 for the others.
+// Such a launch is over when its longest path is, and a step of a warp's paths
+// takes the less time the fewer paths the warp holds, as the other lanes then
+// work for them (see Drain): 1,024 paths at h = 1e-4 take 830 us as 32 full
+// warps and 330 us as 1,024 warps of one path.  More than about 2.5 warps per
+// scheduler compete for its issue slots instead (5,120 paths: 435 us with 2
+// per warp, 450 with 4, 532 with 8; 20,480 paths: 685 us with 8, 621 with 12,
+// 703 with 16), and from 24 paths per warp on a full chip in ordinary
+// iterations is as fast (102,400 paths: 1,376 us with 24, 1,485 with 32).
+// FP64 paths are bound by the SM's one FP64 pipe, which a warp's instruction
+// holds as long for one lane as for 32: they get one warp per scheduler.
+constexpr int kSpreadMax = 24;
+template <class T>
+static int spread_batch(const PathArgs& a, int num_sms) {
+  const unsigned long long sms = (unsigned long long)num_sms;
+  const unsigned long long want = sizeof(T) == 4 ? 10 * sms : 4 * sms;  // warps
+  const unsigned long long each = (a.total + want - 1) / want;
+  if (a.claim > 0) return 0;  // the caller chose the claim
+  if (each <= (unsigned long long)kSpreadMax) return (int)each;
+  return sizeof(T) == 4 && a.total <= kSpreadMax * 32ull * sms ? kSpreadMax : 0;
+}
+
 template <class K>
 static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cudaStream_t st,
-                                     int* blocks, size_t ring_per_warp,
+                                     int* blocks, size_t ring_per_warp, int spread,
                                      std::atomic<int>* attr_set, std::atomic<int>* occ_cache) {
   PathArgs b = a;
-  b.warp_batch = kWarpBatch * (unsigned long long)resolve_claim(a, num_sms);
+  b.warp_batch = spread > 0 ? (unsigned long long)spread
+                            : kWarpBatch * (unsigned long long)resolve_claim(a, num_sms);
   const size_t cache = plan_cache(b);
   int threads = a.block_threads > 0 ? a.block_threads : kBlockThreads;
-  if (a.block_threads <= 0 && cache > 0) {
+  if (a.block_threads <= 0 && cache > 0 && spread == 0) {
     // occ_cache[0] keeps the kernel's register count (block sizes start at 32)
     int regs = occ_cache[0].load(std::memory_order_relaxed);
     if (regs == 0) {
@@ -1210,6 +1250,12 @@ static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cud
       occ_cache[0].store(regs, std::memory_order_relaxed);
     }
     threads = cache_block_threads(regs);
+    // a launch that does not fill the chip: as many warps on every SM
+    const unsigned long long per_sm =
+        ((a.total + b.warp_batch - 1ull) / b.warp_batch + num_sms - 1) / num_sms;
+    const unsigned long long full = (unsigned long long)threads / 32;
+    if (per_sm <= full) threads = 32 * (int)per_sm;
+    else if (per_sm <= 2 * full) threads = 32 * (int)((per_sm + 1) / 2);
   }
   if (threads % 32 != 0 || threads > kMaxBlockThreads) return cudaErrorInvalidValue;
   const size_t smem = cache + (size_t)(threads / 32) * ring_per_warp;
@@ -1234,9 +1280,11 @@ static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cud
   const unsigned long long blocks_needed =
       (warps_needed + (threads / 32) - 1) / (threads / 32);
   unsigned long long nb = (unsigned long long)occ * (unsigned long long)num_sms;
+  if (spread > 0 && nb < blocks_needed) nb = blocks_needed;
   if (a.max_blocks > 0 && nb > (unsigned long long)a.max_blocks) nb = a.max_blocks;
   if (nb > blocks_needed) nb = blocks_needed;
   if (nb < 1) nb = 1;
+  b.one_claim = spread > 0 && nb == blocks_needed;  // the warps' single batches cover every path
   *blocks = (int)nb;
   kern<<<(unsigned)nb, (unsigned)threads, smem, st>>>(b);
   return cudaGetLastError();
@@ -1248,27 +1296,28 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, i
   // FP64 paths: the step dominates, they always take the short iteration
   const bool longer = sizeof(T) == 4 && (a.iter_mode == PDD_ITER_LONG ||
                                          (a.iter_mode == PDD_ITER_AUTO && long_iterations(a)));
+  const int spread = spread_batch<T>(a, num_sms);
   if constexpr (P::kDim == 3) {
     if (longer) {
       static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
       static std::atomic<int> attr{0};
       return launch_persistent(paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>, a, num_sms,
-                               st, blocks, ExitRing<T, 3>::kBytes, &attr, per_sm);
+                               st, blocks, ExitRing<T, 3>::kBytes, spread, &attr, per_sm);
     }
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_3d<P, T, CV, MULTI, 4>, a, num_sms, st, blocks,
-                             ExitRing<T, 3>::kBytes, &attr, per_sm);
+                             ExitRing<T, 3>::kBytes, spread, &attr, per_sm);
   } else if (longer) {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, LongSteps2D<T, CV>::value>, a, num_sms, st,
-                             blocks, ExitRing<T, 2>::kBytes, &attr, per_sm);
+                             blocks, ExitRing<T, 2>::kBytes, spread, &attr, per_sm);
   } else {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, 2>, a, num_sms, st, blocks,
-                             ExitRing<T, 2>::kBytes, &attr, per_sm);
+                             ExitRing<T, 2>::kBytes, spread, &attr, per_sm);
   }
 }
 
@@ -1308,7 +1357,7 @@ static cudaError_t launch_coupled_one(const PathArgs& a, int num_sms, cudaStream
   static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
   static std::atomic<int> attr{0};
   return launch_persistent(paths_coupled<P, T, CV, D>, a, num_sms, st, blocks,
-                           PairRing<T>::kBytes, &attr, per_sm);
+                           PairRing<T>::kBytes, 0, &attr, per_sm);
 }
 
 template <class P, class T, int D>

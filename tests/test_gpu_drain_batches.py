@@ -2,10 +2,11 @@
 
 The drain takes a warp's last paths S steps at a time, S depending on how many
 paths the warp still holds, and finds the exits and the truncations afterwards.
-One warp is given every number of paths here, with caps on the steps that fall at the
+One warp is given every number of paths here (a claim of one path per lane
+keeps the launch from being spread), with caps on the steps that fall at the
 start, inside and at the end of a batch; the same paths of a launch of many
 are issued first and run in the ordinary iterations.  Everything is compared
-bit for bit.
+bit for bit, and spread launches with the unspread ones.
 """
 import numpy as np
 import pytest
@@ -55,3 +56,28 @@ def test_every_count_and_cap(env, kind, precision, y_exp, cv):
             ctx.set_claim(0)
         prob.close()
 
+
+@pytest.mark.parametrize("kind,precision", [("cfg0", 0), ("cfg0", 1), ("cube", 0)])
+def test_spread_launches(env, kind, precision):
+    """Around every line of the rule (paths per warp 1, 2 and 24, and none)."""
+    torch, pdd, ctx = env
+    k, grid = KINDS[kind]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    warps = 10 * sms if precision == 0 else 4 * sms
+    prob = pdd.Problem(ctx, k, precision=precision)
+    prob.set_control_grid(0, W.control_grid(k, grid, 1e-1))
+    nodes = np.full((1, 3 if kind == "cube" else 2), 0.5, np.float32)
+    for n in (1, 31, warps - 1, warps, warps + 1, 2 * warps, 2 * warps + 1, 24 * warps,
+              24 * warps + 1, 24 * 32 * sms, 24 * 32 * sms + 1):
+        a = prob.estimate(nodes, n, 1e-2, grid_id=0)
+        ctx.set_launch(0, 3)  # too few blocks for one claim per warp
+        c = prob.estimate(nodes, n, 1e-2, grid_id=0)
+        ctx.set_launch(0, 0)
+        ctx.set_claim(1)
+        b = prob.estimate(nodes, n, 1e-2, grid_id=0)
+        ctx.set_claim(0)
+        for f in pdd.STAT_FIELDS + pdd.COUNT_FIELDS:
+            assert torch.equal(a[f].nan_to_num(-1.0), b[f].nan_to_num(-1.0)), (n, f)
+            assert torch.equal(c[f].nan_to_num(-1.0), b[f].nan_to_num(-1.0)), (n, f)
+        assert int(a["n_paths"][0]) == n
+    prob.close()
