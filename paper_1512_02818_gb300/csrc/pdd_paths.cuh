@@ -659,11 +659,184 @@ __device__ __forceinline__ void put_vec(T* base, int step, int q, int A, T v0, T
   }
 }
 
+// Where a lane stands in a batch of A paths: it works for path q = lane mod A
+// as number m = lane / A of the lanes `mine`, and lanes below A own a path.
+struct BatchLane {
+  int lane, A, q, m;
+  unsigned mine;
+  __device__ __forceinline__ explicit BatchLane(int paths)
+      : lane((int)(threadIdx.x & 31u)), A(paths), q(lane % A), m(lane / A), mine(0u) {
+    for (int l = q; l < 32; l += A) mine |= 1u << l;
+  }
+};
+
+// Pass 1: Philox block blk of the lane's path into words 4m .. 4m + 3 of the
+// path's normals.
+template <class T, int D>
+__device__ __forceinline__ void batch_normals(const BatchLane& b, uint32_t blk, uint32_t path,
+                                              uint32_t node, uint32_t seed_hi, uint2 key, T sqh,
+                                              T* nrm) {
+  const uint4 w = philox4x32_10(make_uint4(blk, path, node, seed_hi), key);
+  T n[4];
+  box_muller(w.x, w.y, n[0], n[1], sqh);
+  box_muller(w.z, w.w, n[2], n[3], sqh);
+  if (D == 2) {
+    put_vec<T, D>(nrm, 2 * b.m, b.q, b.A, n[0], n[1], T(0));
+    put_vec<T, D>(nrm, 2 * b.m + 1, b.q, b.A, n[2], n[3], T(0));
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) nrm[(4 * b.m + c) * b.A + b.q] = n[c];
+  }
+}
+
+// Increment of step i; PAIR: the sum of those of steps 2i and 2i + 1.
+template <class T, int D, bool PAIR>
+__device__ __forceinline__ void batch_noise(const T* nrm, int i, const BatchLane& b, T* dW) {
+  get_vec<T, D>(nrm, PAIR ? 2 * i : i, b.q, b.A, dW);
+  if (PAIR) {
+    T e[3];
+    get_vec<T, D>(nrm, 2 * i + 1, b.q, b.A, e);
+#pragma unroll
+    for (int d = 0; d < D; ++d) dW[d] = dW[d] + e[d];
+  }
+}
+
+// Passes 2 to 4 over up to S steps of every path that is `on`; returns the
+// steps the lane's path takes and whether max_steps stopped it.  dots[(i A + q)
+// dot_stride] takes grad v . sigma dW in 2D (3D keeps it beside c and f).
+template <class P, class T, int D, int CV, bool PAIR>
+__device__ __forceinline__ int batch_steps(const PathArgs& a, const LaneSeg<T>& ls,
+                                           PathState<T>& s, const T* nrm, T* pos, T* dots,
+                                           int dot_stride, const BatchLane& b, int S, bool on,
+                                           bool use_cv, bool y_exp, bool& trunc) {
+  constexpr int kFold = 4;  // steps whose terms are read at once in pass 4
+  // (path, step) pairs per lane: a 2D block makes two steps, one of a pair's sums
+  constexpr int kItems = D == 2 && !PAIR ? 2 : 1;
+  // 2. positions; the normals are read U steps ahead (U divides S)
+  constexpr int U = PAIR ? 1 : 2;
+  const bool own = b.lane < b.A && on;
+  if (own) {
+    T dW[U][3], next[U][3];
+#pragma unroll
+    for (int j = 0; j < U; ++j) batch_noise<T, D, PAIR>(nrm, j, b, dW[j]);
+#pragma unroll 1
+    for (int i = 0; i < S; i += U) {
+      const int ahead = min(i + U, S - U);
+#pragma unroll
+      for (int j = 0; j < U; ++j) batch_noise<T, D, PAIR>(nrm, ahead + j, b, next[j]);
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        put_vec<T, D>(pos, i + j, b.q, b.A, s.x[0], s.x[1], s.x[2]);
+        Coef<T> o;
+        P::template eval<T, false>(s.x[0], s.x[1], s.x[2], o);
+        T sdW[3];
+        noise<P, T, D>(o, dW[j], sdW);
+        advance<P, T, D>(s.x, ls.h, o, sdW);
+#pragma unroll
+        for (int d = 0; d < D; ++d) dW[j][d] = next[j][d];
+      }
+    }
+  }
+  __syncwarp();
+  // 3. exit tests, then coefficients of the steps before the exit
+  unsigned f[kItems];
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const int i = kItems * b.m + j;
+    bool fin = false;
+    if (i < S && on) {
+      T x[3];
+      get_vec<T, D>(pos, i, b.q, b.A, x);
+      fin = outside<P, T, D>(x, ls.thr0);
+    }
+    f[j] = __ballot_sync(kFull, fin) & b.mine;
+  }
+  int n = on ? S : 0;
+  const unsigned any = f[0] | f[kItems - 1];
+  if (any != 0u) {
+    const int l = __ffs(any) - 1;
+    n = kItems * (l / b.A) + ((f[0] >> l) & 1u ? 0 : 1);
+  }
+  trunc = on && n >= ls.max_steps - s.k;
+  if (trunc) n = ls.max_steps - s.k;
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const int i = kItems * b.m + j;
+    if (i < n) {
+      T x[3];
+      get_vec<T, D>(pos, i, b.q, b.A, x);
+      T gv[3] = {T(0), T(0), T(0)}, dot = T(0);
+      if (CV == kCvGrid && use_cv) grid_gradient<T, D>(a, ls, x, gv);
+      Coef<T> o;
+      P::template eval<T, CV == kCvExact>(x[0], x[1], x[2], o);
+      if (use_cv) {
+        T dW[3], sdW[3];
+        batch_noise<T, D, PAIR>(nrm, i, b, dW);
+        noise<P, T, D>(o, dW, sdW);
+        if (CV == kCvExact) {
+          gv[0] = o.g0;
+          gv[1] = o.g1;
+          gv[2] = o.g2;
+        }
+        dot = cv_dot<T, D>(gv, sdW);
+      }
+      const T c = y_exp ? m_exp(mul_rn(-ls.h, o.c)) : o.c;
+      put_vec<T, D>(pos, i, b.q, b.A, c, o.f, dot);
+      if (D == 2 && use_cv) dots[(i * b.A + b.q) * dot_stride] = dot;
+    }
+  }
+  __syncwarp();
+  // 4. Y, Z and xi
+  if (own) {
+    auto fold = [&](const T* v) {
+      if (use_cv) kahan_add(s.XI, s.XIc, -s.Y, v[2]);
+      if (!P::kUnitY) {
+        const T hY = mul_rn(ls.h, s.Y);
+        kahan_add(s.Z, s.Zc, -hY, v[1]);
+        s.Y = y_exp ? mul_rn(s.Y, v[0]) : fma_rn(-hY, v[0], s.Y);
+      }
+    };
+    auto read = [&](int i, T* v) {
+      get_vec<T, D>(pos, i, b.q, b.A, v);
+      if (D == 2 && use_cv) v[2] = dots[(i * b.A + b.q) * dot_stride];
+    };
+    int i = 0;
+#pragma unroll 1
+    for (; i + kFold <= n; i += kFold) {
+      T v[kFold][3];
+#pragma unroll
+      for (int j = 0; j < kFold; ++j) read(i + j, v[j]);
+#pragma unroll
+      for (int j = 0; j < kFold; ++j) fold(v[j]);
+    }
+#pragma unroll 1
+    for (; i < n; ++i) {
+      T v[3];
+      read(i, v);
+      fold(v);
+    }
+    if (n < S) get_vec<T, D>(pos, n, b.q, b.A, s.x);  // X at the exit
+  }
+  s.k += n;
+  return n;
+}
+
+// The lane takes the path of lane `src` (position, sums and step).
+template <class T, int D>
+__device__ __forceinline__ void take_path(PathState<T>& s, int src) {
+#pragma unroll
+  for (int d = 0; d < D; ++d) s.x[d] = __shfl_sync(kFull, s.x[d], src);
+  s.Y = __shfl_sync(kFull, s.Y, src);
+  s.Z = __shfl_sync(kFull, s.Z, src);
+  s.Zc = __shfl_sync(kFull, s.Zc, src);
+  s.XI = __shfl_sync(kFull, s.XI, src);
+  s.XIc = __shfl_sync(kFull, s.XIc, src);
+  s.k = __shfl_sync(kFull, s.k, src);
+}
+
 template <class P, class T, int D, int CV, bool MULTI>
 __device__ __forceinline__ void drain(const PathArgs& a, const ExitRing<T, D> ring, RingCursor rc,
-                                   PathState<T> s, LaneSeg<T> ls, bool active) {
-  constexpr int kFold = 4;  // steps whose terms are read at once in pass 4
-  const int lane = (int)(threadIdx.x & 31u);
+                                      PathState<T> s, LaneSeg<T> ls, bool active) {
   // the ring's first half parks the exits from here on, its second is scratch
   if (rc.held > 0u) ring_drain<P, T, D, MULTI>(a, ring, rc.head - rc.held, rc.held);
   uint32_t held = 0;
@@ -671,17 +844,9 @@ __device__ __forceinline__ void drain(const PathArgs& a, const ExitRing<T, D> ri
   T* const pos = nrm + (D == 2 ? 4 * Drain<T, D>::kLanes : 96);  // X, then c, f (and the dot in 3D)
   unsigned runm = __ballot_sync(kFull, active);
   while (runm != 0u) {
-    // lane L takes path q = L mod A (its state in lanes L < A, its key and
-    // segment in every lane)
-    const int A = __popc(runm), q = lane % A, m = lane / A;
-    const int src = nth_set_bit(runm, q);
-    for (int d = 0; d < D; ++d) s.x[d] = __shfl_sync(kFull, s.x[d], src);
-    s.Y = __shfl_sync(kFull, s.Y, src);
-    s.Z = __shfl_sync(kFull, s.Z, src);
-    s.Zc = __shfl_sync(kFull, s.Zc, src);
-    s.XI = __shfl_sync(kFull, s.XI, src);
-    s.XIc = __shfl_sync(kFull, s.XIc, src);
-    s.k = __shfl_sync(kFull, s.k, src);
+    const BatchLane b(__popc(runm));
+    const int src = nth_set_bit(runm, b.q);
+    take_path<T, D>(s, src);
     s.node = __shfl_sync(kFull, s.node, src);
     s.path = __shfl_sync(kFull, s.path, src);
     if (MULTI) {
@@ -691,139 +856,22 @@ __device__ __forceinline__ void drain(const PathArgs& a, const ExitRing<T, D> ri
     const SegArgs& sg = a.seg[MULTI ? s.seg : 0];
     const uint32_t key0 = sg.key0, key1 = sg.key1, seed_hi = sg.seed_hi;
     const bool use_cv = CV != kCvNone && (CV != kCvGrid || !MULTI || ls.grad != nullptr);
-    const bool y_exp = MULTI && a.y_exp;
-    const int blocks = Drain<T, D>::blocks(A), S = Drain<T, D>::steps(A);
-    unsigned mine = 0u;  // the lanes of path q
-    for (int l = q; l < 32; l += A) mine |= 1u << l;
+    const int blocks = Drain<T, D>::blocks(b.A), S = Drain<T, D>::steps(b.A);
     unsigned endm = 0u;
     bool trunc = false;
     do {
-      // 1. random numbers
-      if (m < blocks) {
+      if (b.m < blocks) {
         const uint32_t blk0 = D == 2 ? (uint32_t)s.k >> 1 : 3u * ((uint32_t)s.k >> 2);
         // (the empty asm keeps the ten rounds' keys from living in registers
         // across the batches: 20 of them with per-lane keys)
         uint2 key = make_uint2(key0, key1);
         if (MULTI) asm volatile("" : "+r"(key.x), "+r"(key.y));
-        const uint4 w = philox4x32_10(make_uint4(blk0 + (uint32_t)m, s.path, s.node, seed_hi), key);
-        T n[4];
-        box_muller(w.x, w.y, n[0], n[1], ls.sqh);
-        box_muller(w.z, w.w, n[2], n[3], ls.sqh);
-        if (D == 2) {
-          put_vec<T, D>(nrm, 2 * m, q, A, n[0], n[1], T(0));
-          put_vec<T, D>(nrm, 2 * m + 1, q, A, n[2], n[3], T(0));
-        } else {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) nrm[(4 * m + c) * A + q] = n[c];
-        }
+        batch_normals<T, D>(b, blk0 + (uint32_t)b.m, s.path, s.node, seed_hi, key, ls.sqh, nrm);
       }
       __syncwarp();
-      // 2. positions (S is even; the normals are read two steps ahead)
-      if (lane < A) {
-        T dW[2][3], next[2][3];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) get_vec<T, D>(nrm, j, q, A, dW[j]);
-#pragma unroll 1
-        for (int i = 0; i < S; i += 2) {
-          const int ahead = min(i + 2, S - 2);
-#pragma unroll
-          for (int j = 0; j < 2; ++j) get_vec<T, D>(nrm, ahead + j, q, A, next[j]);
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            put_vec<T, D>(pos, i + j, q, A, s.x[0], s.x[1], s.x[2]);
-            Coef<T> o;
-            P::template eval<T, false>(s.x[0], s.x[1], s.x[2], o);
-            T sdW[3];
-            noise<P, T, D>(o, dW[j], sdW);
-            advance<P, T, D>(s.x, ls.h, o, sdW);
-#pragma unroll
-            for (int d = 0; d < D; ++d) dW[j][d] = next[j][d];
-          }
-        }
-      }
-      __syncwarp();
-      // 3. exit tests, then coefficients of the steps before the exit
-      constexpr int kItems = D == 2 ? 2 : 1;  // (path, step) pairs per lane
-      unsigned f[kItems];
-#pragma unroll
-      for (int j = 0; j < kItems; ++j) {
-        const int i = kItems * m + j;
-        bool fin = false;
-        if (i < S) {
-          T x[3];
-          get_vec<T, D>(pos, i, q, A, x);
-          fin = outside<P, T, D>(x, ls.thr0);
-        }
-        f[j] = __ballot_sync(kFull, fin) & mine;
-      }
-      int n = S;  // steps path q takes
-      const unsigned any = f[0] | f[kItems - 1];
-      if (any != 0u) {
-        const int l = __ffs(any) - 1;
-        n = kItems * (l / A) + ((f[0] >> l) & 1u ? 0 : 1);
-      }
-      trunc = n >= ls.max_steps - s.k;
-      if (trunc) n = ls.max_steps - s.k;
-#pragma unroll
-      for (int j = 0; j < kItems; ++j) {
-        const int i = kItems * m + j;
-        if (i < n) {
-          T x[3];
-          get_vec<T, D>(pos, i, q, A, x);
-          T gv[3] = {T(0), T(0), T(0)}, dot = T(0);
-          if (CV == kCvGrid && use_cv) grid_gradient<T, D>(a, ls, x, gv);
-          Coef<T> o;
-          P::template eval<T, CV == kCvExact>(x[0], x[1], x[2], o);
-          if (use_cv) {
-            T dW[3], sdW[3];
-            get_vec<T, D>(nrm, i, q, A, dW);
-            noise<P, T, D>(o, dW, sdW);
-            if (CV == kCvExact) {
-              gv[0] = o.g0;
-              gv[1] = o.g1;
-              gv[2] = o.g2;
-            }
-            dot = cv_dot<T, D>(gv, sdW);
-          }
-          const T c = y_exp ? m_exp(mul_rn(-ls.h, o.c)) : o.c;
-          put_vec<T, D>(pos, i, q, A, c, o.f, dot);
-          if (D == 2 && use_cv) nrm[2 * (i * A + q)] = dot;
-        }
-      }
-      __syncwarp();
-      // 4. Y, Z and xi
-      if (lane < A) {
-        auto fold = [&](const T* v, T dot) {
-          if (use_cv) kahan_add(s.XI, s.XIc, -s.Y, dot);
-          if (!P::kUnitY) {
-            const T hY = mul_rn(ls.h, s.Y);
-            kahan_add(s.Z, s.Zc, -hY, v[1]);
-            s.Y = y_exp ? mul_rn(s.Y, v[0]) : fma_rn(-hY, v[0], s.Y);
-          }
-        };
-        auto read = [&](int i, T* v) {
-          get_vec<T, D>(pos, i, q, A, v);
-          if (D == 2 && use_cv) v[2] = nrm[2 * (i * A + q)];
-        };
-        int i = 0;
-#pragma unroll 1
-        for (; i + kFold <= n; i += kFold) {
-          T v[kFold][3];
-#pragma unroll
-          for (int j = 0; j < kFold; ++j) read(i + j, v[j]);
-#pragma unroll
-          for (int j = 0; j < kFold; ++j) fold(v[j], v[j][2]);
-        }
-#pragma unroll 1
-        for (; i < n; ++i) {
-          T v[3];
-          read(i, v);
-          fold(v, v[2]);
-        }
-        if (n < S) get_vec<T, D>(pos, n, q, A, s.x);  // X at the exit
-      }
-      s.k += n;
-      endm = __ballot_sync(kFull, lane < A && (trunc || n < S));
+      const int n = batch_steps<P, T, D, CV, false>(a, ls, s, nrm, pos, nrm, 2, b, S, true, use_cv,
+                                                    MULTI && a.y_exp, trunc);
+      endm = __ballot_sync(kFull, b.lane < b.A && (trunc || n < S));
       __syncwarp();
     } while (endm == 0u);
     // park the exits
@@ -832,20 +880,24 @@ __device__ __forceinline__ void drain(const PathArgs& a, const ExitRing<T, D> ri
       ring_drain<P, T, D, MULTI>(a, ring, 0u, held);
       held = 0;
     }
-    if ((endm >> lane) & 1u)
-      ring_put<T, D>(ring, held + (uint32_t)__popc(endm & ((1u << lane) - 1u)), s, trunc);
+    if ((endm >> b.lane) & 1u)
+      ring_put<T, D>(ring, held + (uint32_t)__popc(endm & ((1u << b.lane) - 1u)), s, trunc);
     held += ended;
-    runm = ((1u << A) - 1u) & ~endm;
+    runm = ((1u << b.A) - 1u) & ~endm;
   }
   if (held > 0u) ring_drain<P, T, D, MULTI>(a, ring, 0u, held);
 }
 
-// The segment-table build keeps per-lane segment parameters in registers; at
-// 65 registers a 512-thread block rounds up to 72 per thread and only one
-// block fits an SM, so it is capped at 64 (two blocks), which measured faster
-// than the uncapped build.
+// The segment-table build keeps per-lane segment parameters in registers, 72
+// with the control variate (28 warps an SM).  A cap at 64 makes ptxas trade the
+// whole loop's schedule for registers: 2 x 256 nodes x 50,000 paths with the
+// control variate take 124 ms at 72 and 131 ms at 64.  Short paths want the
+// warps more (130 segments x 217 nodes x 4,942 paths of 10 to 100 steps:
+// 48.4 ms at 72, 47.3 ms at 64), so the short iteration is capped.
+template <class T, bool MULTI, int STEPS>
+constexpr int kMinBlocks2D = MULTI && sizeof(T) == 4 && STEPS == 2 ? 2 : PDD_MIN_BLOCKS_2D;
 template <class P, class T, int CV, bool MULTI, int STEPS>
-__global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_2D)
+__global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEPS>))
     paths_2d(const __grid_constant__ PathArgs a) {
   PathState<T> s;
   LaneSeg<T> ls;
@@ -983,24 +1035,46 @@ struct CoupledShape {
   static constexpr int kCoarse = kFine / 2;
 };
 
-// Per-warp ring of finished pairs (the coupled counterpart of ExitRing): the
-// two scores of each path, both exit indices, node, path and truncation
-// flags; drained 32 pairs at a time into the fine and difference records.
+// What a finished pair leaves: the two scores of each path, both exit indices.
+template <class T>
+struct PairEnd {
+  T phif, xif, phic, xic;
+  int kf, kc;
+  uint32_t node, path, trunc;  // truncated: bit 0 fine, bit 1 coarse
+};
+
+// Per-warp ring of finished pairs (the coupled counterpart of ExitRing),
+// drained 32 pairs at a time into the fine and difference records.
 template <class T>
 struct PairRing {
-  static constexpr size_t kBytes = kRing * (4 * sizeof(T) + 5 * sizeof(uint32_t));
-  T* f;         // 4 x kRing: phi_f, xi_f, phi_c, xi_c
-  uint32_t* u;  // 5 x kRing: k_f, k_c, node, path, truncated (bit 0 fine, bit 1 coarse)
+  static constexpr uint32_t kHalf = 32 * (4 * sizeof(T) + 5 * sizeof(uint32_t));
+  static constexpr size_t kBytes = 2 * kHalf;
+  char* base;
+  __device__ __forceinline__ T* f(uint32_t j) const {
+    return (T*)(base + (j >> 5) * kHalf) + (j & 31u);
+  }
+  __device__ __forceinline__ uint32_t* u(uint32_t j) const {
+    return (uint32_t*)(base + (j >> 5) * kHalf + 32 * 4 * sizeof(T)) + (j & 31u);
+  }
+  __device__ __forceinline__ void put(uint32_t j, const PairEnd<T>& e) const {
+    T* v = f(j);
+    uint32_t* w = u(j);
+    v[0] = e.phif;
+    v[32] = e.xif;
+    v[64] = e.phic;
+    v[96] = e.xic;
+    w[0] = (uint32_t)e.kf;
+    w[32] = (uint32_t)e.kc;
+    w[64] = e.node;
+    w[96] = e.path;
+    w[128] = e.trunc;
+  }
 };
 
 template <class T>
 __device__ __forceinline__ PairRing<T> pair_ring_of_warp(const PathArgs& a) {
-  char* base = (char*)s_cache + cache_bytes(a.cache_nodes) +
-               (size_t)(threadIdx.x >> 5) * PairRing<T>::kBytes;
-  PairRing<T> r;
-  r.f = (T*)base;
-  r.u = (uint32_t*)(base + kRing * 4 * sizeof(T));
-  return r;
+  return {(char*)s_cache + cache_bytes(a.cache_nodes) +
+          (size_t)(threadIdx.x >> 5) * PairRing<T>::kBytes};
 }
 
 template <class T>
@@ -1010,11 +1084,11 @@ __device__ __forceinline__ void pair_drain(const PathArgs& a, const PairRing<T>&
   const uint32_t lane = threadIdx.x & 31u;
   if (lane < count) {
     const uint32_t j = (first + lane) & (kRing - 1);
-    const T phif = r.f[j], xif = r.f[kRing + j], phic = r.f[2 * kRing + j],
-            xic = r.f[3 * kRing + j];
-    const int kf = (int)r.u[j], kc = (int)r.u[kRing + j];
-    const uint32_t node = r.u[2 * kRing + j], path = r.u[3 * kRing + j];
-    const uint32_t tr = r.u[4 * kRing + j];
+    const T* v = r.f(j);
+    const uint32_t* w = r.u(j);
+    const T phif = v[0], xif = v[32], phic = v[64], xic = v[96];
+    const int kf = (int)w[0], kc = (int)w[32];
+    const uint32_t node = w[64], path = w[96], tr = w[128];
     const SegArgs& s0 = a.seg[0];
     const SegArgs& s1 = a.seg[1];
     record_path(a, s0, node, phif, phif + xif, kf, (tr & 1u) != 0u);
@@ -1034,81 +1108,186 @@ __device__ __forceinline__ void pair_drain(const PathArgs& a, const PairRing<T>&
   __syncwarp();
 }
 
+// Per-lane state of a pair.
+template <class T>
+struct PairState {
+  PathState<T> f, c;  // fine and coarse path
+  bool af, ac;        // still running
+  bool tf, tc;        // truncated
+  T phif, xif, phic, xic;
+  uint32_t j;         // iterations of CoupledShape done
+  __device__ __forceinline__ PairEnd<T> end() const {
+    return {phif, xif, phic, xic, f.k, c.k, f.node, f.path, (tf ? 1u : 0u) | (tc ? 2u : 0u)};
+  }
+};
+
+// The drain of a warp's last pairs (see Drain): a batch draws the fine path's
+// normals once and takes S fine steps, then the S / 2 coarse ones that their
+// sums make.  A pair whose one path has ended goes on with the other.
+// 1,024 pairs at h = 1e-3 took 696 us plain and 935 us with the control variate
+// in ordinary iterations of one lane per pair, a step of which is as deep as
+// both paths' steps and the random numbers of a lane.
+template <class T, int D>
+struct PairDrain {
+  // 2D scratch: 4 normals, X or c and f of two steps and their dots per lane
+  static constexpr int kLanes = PairRing<T>::kHalf / (10 * sizeof(T)) < 32
+                                    ? PairRing<T>::kHalf / (10 * sizeof(T))
+                                    : 32;
+  static constexpr int kMaxRun = D == 2 ? 14 : 8;
+  __device__ static int blocks(int A) { return D == 2 ? kLanes / A : 3 * (8 / A); }
+  __device__ static int steps(int A) { return D == 2 ? 2 * (kLanes / A) : 4 * (8 / A); }
+};
+static_assert(32 * 6 * sizeof(float) <= PairRing<float>::kHalf, "3D pair drain scratch");
+
+template <class P, class T, int D, int CV>
+__device__ __forceinline__ void drain_pairs(const PathArgs& a, const PairRing<T> ring,
+                                            RingCursor rc, PairState<T> s, const LaneSeg<T>& lf,
+                                            const LaneSeg<T>& lc, bool active) {
+  using S4 = CoupledShape<D>;
+  using Shape = PairDrain<T, D>;
+  if (rc.held > 0u) pair_drain<T>(a, ring, rc.head - rc.held, rc.held);
+  uint32_t held = 0;
+  T* const nrm = (T*)(ring.base + PairRing<T>::kHalf);
+  T* const pos = nrm + (D == 2 ? 4 * Shape::kLanes : 96);
+  T* const dots = pos + 4 * Shape::kLanes;  // 2D
+  const SegArgs& sg = a.seg[0];
+  unsigned runm = __ballot_sync(kFull, active);
+  while (runm != 0u) {
+    const BatchLane b(__popc(runm));
+    const int src = nth_set_bit(runm, b.q);
+    take_path<T, D>(s.f, src);
+    take_path<T, D>(s.c, src);
+    s.f.node = __shfl_sync(kFull, s.f.node, src);
+    s.f.path = __shfl_sync(kFull, s.f.path, src);
+    s.j = __shfl_sync(kFull, s.j, src);
+    s.phif = __shfl_sync(kFull, s.phif, src);
+    s.xif = __shfl_sync(kFull, s.xif, src);
+    s.phic = __shfl_sync(kFull, s.phic, src);
+    s.xic = __shfl_sync(kFull, s.xic, src);
+    const unsigned flags = __shfl_sync(kFull, (s.af ? 1u : 0u) | (s.ac ? 2u : 0u) |
+                                                  (s.tf ? 4u : 0u) | (s.tc ? 8u : 0u), src);
+    s.af = (flags & 1u) != 0u;
+    s.ac = (flags & 2u) != 0u;
+    s.tf = (flags & 4u) != 0u;
+    s.tc = (flags & 8u) != 0u;
+    const int blocks = Shape::blocks(b.A), S = Shape::steps(b.A);
+    unsigned endm = 0u;
+    do {
+      if (b.m < blocks)
+        batch_normals<T, D>(b, S4::kBlocks * s.j + (uint32_t)b.m, s.f.path, s.f.node, sg.seed_hi,
+                            make_uint2(sg.key0, sg.key1), lf.sqh, nrm);
+      __syncwarp();
+      bool trunc = false;
+      int n = batch_steps<P, T, D, CV, false>(a, lf, s.f, nrm, pos, dots, 1, b, S, s.af,
+                                              CV != kCvNone, a.y_exp != 0, trunc);
+      if (s.af && (trunc || n < S)) {
+        s.af = false;
+        s.tf = trunc;
+        score_path<P, T, D>(s.f, s.phif, s.xif);
+      }
+      __syncwarp();
+      n = batch_steps<P, T, D, CV, true>(a, lc, s.c, nrm, pos, dots, 1, b, S / 2, s.ac,
+                                         CV != kCvNone, a.y_exp != 0, trunc);
+      if (s.ac && (trunc || n < S / 2)) {
+        s.ac = false;
+        s.tc = trunc;
+        score_path<P, T, D>(s.c, s.phic, s.xic);
+      }
+      s.j += (uint32_t)(S / S4::kFine);
+      endm = __ballot_sync(kFull, b.lane < b.A && !s.af && !s.ac);
+      __syncwarp();
+    } while (endm == 0u);
+    const uint32_t ended = (uint32_t)__popc(endm);
+    if (held + ended > 32u) {
+      pair_drain<T>(a, ring, 0u, held);
+      held = 0;
+    }
+    if ((endm >> b.lane) & 1u)
+      ring.put(held + (uint32_t)__popc(endm & ((1u << b.lane) - 1u)), s.end());
+    held += ended;
+    runm = ((1u << b.A) - 1u) & ~endm;
+  }
+  if (held > 0u) pair_drain<T>(a, ring, 0u, held);
+}
+
 template <class P, class T, int CV, int D>
 __global__ void __launch_bounds__(kMaxBlockThreads, 1) paths_coupled(
     const __grid_constant__ PathArgs a) {
   using S = CoupledShape<D>;
   const PairRing<T> ring = pair_ring_of_warp<T>(a);
   RingCursor rc;
-  PathState<T> f, c;
+  PairState<T> p;
+  PathState<T>& f = p.f;
+  PathState<T>& c = p.c;
   LaneSeg<T> lf, lc;
   init_lane<T, D>(a, f, lf);
   init_lane<T, D>(a, c, lc);
   load_seg<T, D>(a.seg[1], lc);
+  p.af = p.ac = p.tf = p.tc = false;
+  p.phif = p.xif = p.phic = p.xic = T(0);
+  p.j = 0;
   cache_init(a);
   bool active = false, exhausted = false;  // active: the pair still has work
-  bool af = false, ac = false;             // fine / coarse path running
-  bool tf = false, tc = false;             // truncated
-  T phif = T(0), xif = T(0), phic = T(0), xic = T(0);
-  uint32_t j = 0;
   unsigned long long bnext = 0, bend = 0;
+  spread_claim(a, bnext, bend);
   while (refill<T, D, false>(a, f, lf, active, bnext, bend, exhausted)) {
-    if (active && f.k == 0 && !af && !ac) {  // refill has just started a new pair in f
+    if (active && f.k == 0 && !p.af && !p.ac) {  // refill has just started a new pair in f
       c = f;
-      af = ac = true;
-      tf = tc = false;
-      j = 0;
+      p.af = p.ac = true;
+      p.tf = p.tc = false;
+      p.j = 0;
     }
+    if (exhausted && __popc(__ballot_sync(kFull, active)) <= PairDrain<T, D>::kMaxRun) break;
     if (active) {
       T n[S::kNormals];
 #pragma unroll
       for (int b = 0; b < S::kBlocks; ++b) {
-        const uint4 w = path_block<false>(a, 0, S::kBlocks * j + b, f.path, f.node);
+        const uint4 w = path_block<false>(a, 0, S::kBlocks * p.j + b, f.path, f.node);
         box_muller(w.x, w.y, n[4 * b], n[4 * b + 1], lf.sqh);
         box_muller(w.z, w.w, n[4 * b + 2], n[4 * b + 3], lf.sqh);
       }
-      if (af) {
+      if (p.af) {
 #pragma unroll
         for (int q = 0; q < S::kFine; ++q) {
-          if (af) {
+          if (p.af) {
             if (should_finish<P, T, D>(f, lf.thr0)) {
-              af = false;
+              p.af = false;
             } else {
               T d[3] = {n[D * q], n[D * q + 1], D == 3 ? n[D * q + 2] : T(0)};
               euler_step<P, T, D, CV, false, true>(a, f, lf, d);
               if (f.k >= lf.max_steps) {
-                af = false;
-                tf = true;
+                p.af = false;
+                p.tf = true;
               }
             }
           }
         }
-        if (!af) score_path<P, T, D>(f, phif, xif);
+        if (!p.af) score_path<P, T, D>(f, p.phif, p.xif);
       }
-      if (ac) {
+      if (p.ac) {
 #pragma unroll
         for (int q = 0; q < S::kCoarse; ++q) {
-          if (ac) {
+          if (p.ac) {
             if (should_finish<P, T, D>(c, lc.thr0)) {
-              ac = false;
+              p.ac = false;
             } else {
               const int o = 2 * D * q;  // fine steps 2q and 2q+1 of this iteration
               T d[3] = {n[o] + n[o + D], n[o + 1] + n[o + D + 1],
                         D == 3 ? n[o + 2] + n[o + D + 2] : T(0)};
               euler_step<P, T, D, CV, false, true>(a, c, lc, d);
               if (c.k >= lc.max_steps) {
-                ac = false;
-                tc = true;
+                p.ac = false;
+                p.tc = true;
               }
             }
           }
         }
-        if (!ac) score_path<P, T, D>(c, phic, xic);
+        if (!p.ac) score_path<P, T, D>(c, p.phic, p.xic);
       }
-      j += 1;
+      p.j += 1;
     }
     // park finished pairs; drain 32 at a time with the whole warp
-    const bool done = active && !af && !ac;
+    const bool done = active && !p.af && !p.ac;
     const unsigned m = __ballot_sync(kFull, done);
     // never more than kRing parked: fewer than 32 are held before this iteration
     // (bounds-checked build: an over-full ring drops the pairs, never stalls)
@@ -1117,16 +1296,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 1) paths_coupled(
     } else if (m != 0u) {
       if (done) {
         const unsigned lt = (1u << (threadIdx.x & 31u)) - 1u;
-        const uint32_t q = (rc.head + __popc(m & lt)) & (kRing - 1);
-        ring.f[q] = phif;
-        ring.f[kRing + q] = xif;
-        ring.f[2 * kRing + q] = phic;
-        ring.f[3 * kRing + q] = xic;
-        ring.u[q] = (uint32_t)f.k;
-        ring.u[kRing + q] = (uint32_t)c.k;
-        ring.u[2 * kRing + q] = f.node;
-        ring.u[3 * kRing + q] = f.path;
-        ring.u[4 * kRing + q] = (tf ? 1u : 0u) | (tc ? 2u : 0u);
+        ring.put((rc.head + __popc(m & lt)) & (kRing - 1), p.end());
         active = false;
       }
       rc.head += __popc(m);
@@ -1137,7 +1307,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 1) paths_coupled(
       }
     }
   }
-  if (rc.held > 0u) pair_drain<T>(a, ring, rc.head - rc.held, rc.held);
+  drain_pairs<P, T, D, CV>(a, ring, rc, p, lf, lc, active);
   cache_flush(a);
 }
 
@@ -1357,7 +1527,8 @@ static cudaError_t launch_coupled_one(const PathArgs& a, int num_sms, cudaStream
   static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
   static std::atomic<int> attr{0};
   return launch_persistent(paths_coupled<P, T, CV, D>, a, num_sms, st, blocks,
-                           PairRing<T>::kBytes, 0, &attr, per_sm);
+                           PairRing<T>::kBytes, spread_batch<T>(a, num_sms), &attr,
+                           per_sm);
 }
 
 template <class P, class T, int D>

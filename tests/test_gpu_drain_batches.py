@@ -81,3 +81,31 @@ def test_spread_launches(env, kind, precision):
             assert torch.equal(c[f].nan_to_num(-1.0), b[f].nan_to_num(-1.0)), (n, f)
         assert int(a["n_paths"][0]) == n
     prob.close()
+
+
+@pytest.mark.parametrize("kind,y_exp,cv", [("cfg0", 0, "grid"), ("cfg0", 1, "none"), ("aniso", 0, "grid"),
+                                           ("paper", 0, "exact"), ("cube", 0, "grid")])
+def test_pairs(env, kind, y_exp, cv):
+    """The coupled kernels: every number of pairs in a warp, caps that end one
+    path of a pair (the fine path has twice the steps) or both, and spread
+    launches; against the first pairs of a large launch."""
+    torch, pdd, ctx = env
+    k, grid = KINDS[kind]
+    node = np.full((1, 3 if kind == "cube" else 2), 0.5, np.float32)
+    for cap in (0, 37, 64):
+        prob = pdd.Problem(ctx, k, y_rule=y_exp, max_steps=cap)
+        gid = {"none": pdd.PDD_CV_NONE, "exact": pdd.PDD_CV_EXACT, "grid": 0}[cv]
+        if cv == "grid":
+            prob.set_control_grid(0, W.control_grid(k, grid, 1e-1))
+        big = prob.estimate_coupled(node, 130_000, 4e-3, grid_id=gid, emit_paths=True)
+        for claim, counts in ((1, (1, 2, 3, 5, 7, 8, 9, 11, 14, 15, 28, 32)), (0, (3, 1500, 9000))):
+            ctx.set_claim(claim)
+            try:
+                for n in counts:
+                    small = prob.estimate_coupled(node, n, 4e-3, grid_id=gid, emit_paths=True)
+                    for a, b in zip(small, big):
+                        for f in ("phi", "xi", "steps"):
+                            assert torch.equal(a[f], b[f][:, :n]), (cap, claim, n, f)
+            finally:
+                ctx.set_claim(0)
+        prob.close()
