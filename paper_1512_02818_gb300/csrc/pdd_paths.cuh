@@ -1314,22 +1314,46 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 1) paths_coupled(
 // ---------------------------------------------------------------------------
 // Launch dispatch.
 // ---------------------------------------------------------------------------
-// Shared-memory record slots of a launch (the segments' nodes in segment
-// order) when they fit kCacheMaxNodes; returns the dynamic shared memory the
-// cache needs (0: no cache).
-static size_t plan_cache(PathArgs& b) {
-  unsigned long long tot = 0;
-  for (int i = 0; i < b.n_segs; ++i) tot += b.seg[i].n_nodes;
-  b.cache_nodes = 0;
-  if (tot == 0 || tot > kCacheMaxNodes) return 0;
+// Whether a launch keeps its records in shared memory.  Finished paths cost
+// about 10 ns each per record line in L2 (13 atomics on one line), so the cache
+// pays when few records take many exits: 1.5e9 path-steps on 64 nodes take
+// 5.8 ms with it and 9.6 ms without at 100 steps a path, 5.5 and 5.5 ms at
+// 330; on 256 nodes 10 and 34 ms at 10 steps, 5.7 and 5.6 ms at 100.  But its
+// copies take shared memory from L1, and with less than about 40 KB of L1 left
+// the gathers of the control variate starve: 480 records in two blocks an SM
+// (204 KB) run 2e9 path-steps in 13.7 ms against 9.5 ms without the cache, 448
+// records (196 KB) 9.3 ms.  So:
+//  - a spread launch, in 128-thread blocks with a copy each, caches up to 64
+//    records (1 node x 18,000 10-step paths: 38 us with, 197 us without; 256
+//    nodes: no difference);
+//  - a kernel that lives by L1 (`l1`: a control grid, or the coupled kernels,
+//    which have room for one such block only: 21.3 against 19.2 ms) caches more
+//    than kCacheL1Bytes only when records x mean steps is under 2e4.
+// The mean number of steps is taken as 0.1 / h, that of the unit box.
+constexpr size_t kCacheL1Bytes = 97 * 1024;  // per block, rings included
+static bool use_cache(const PathArgs& a, unsigned long long records, bool spread, bool l1,
+                      size_t smem) {
+  if (records == 0 || records > kCacheMaxNodes) return false;
+  if (spread) return records <= 64;
+  if (!l1 || smem <= kCacheL1Bytes) return true;
+  double paths = 0.0, steps = 0.0;
+  for (int i = 0; i < a.n_segs; ++i) {
+    paths += (double)a.seg[i].total;
+    steps += (double)a.seg[i].total * 0.1 / a.seg[i].h;
+  }
+  return (double)records * steps < 2e4 * paths;
+}
+
+// Shared-memory record slots of a launch: the segments' nodes in segment order.
+static void place_records(PathArgs& b) {
   uint32_t base = 0;
   for (int i = 0; i < b.n_segs; ++i) {
     b.seg[i].cache_base = base;
     base += (uint32_t)b.seg[i].n_nodes;
   }
   b.cache_nodes = base;
-  return cache_bytes(base);
 }
+
 // Default block size of launches with the record cache: large, so that many
 // warps share one copy of the records, and two blocks to an SM where that
 // costs few warps (up to 64 registers a thread: 512 threads, 72: 448, which
@@ -1341,7 +1365,8 @@ static int cache_block_threads(int regs) { return regs > 64 && regs <= 72 ? 448 
 // SM count blocks (at most one warp per 32 paths), with the record cache
 // when the launch's nodes fit it and `ring_per_warp` bytes of exit ring per
 // warp.  `spread` > 0: that many paths per warp (see spread_batch), in blocks
-// of 128 threads so that the warps cover the SMs evenly.  `attr_set` /
+// of 128 threads so that the warps cover the SMs evenly.  `l1`: see use_cache.
+// `attr_set` /
 // `occ_cache` are the kernel's own (static) state: the
 // dynamic shared memory limit set so far and the occupancy per block size
 // without the cache.
@@ -1402,14 +1427,15 @@ static int spread_batch(const PathArgs& a, int num_sms) {
 
 template <class K>
 static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cudaStream_t st,
-                                     int* blocks, size_t ring_per_warp, int spread,
+                                     int* blocks, size_t ring_per_warp, int spread, bool l1,
                                      std::atomic<int>* attr_set, std::atomic<int>* occ_cache) {
   PathArgs b = a;
   b.warp_batch = spread > 0 ? (unsigned long long)spread
                             : kWarpBatch * (unsigned long long)resolve_claim(a, num_sms);
-  const size_t cache = plan_cache(b);
+  unsigned long long records = 0;
+  for (int i = 0; i < a.n_segs; ++i) records += a.seg[i].n_nodes;
   int threads = a.block_threads > 0 ? a.block_threads : kBlockThreads;
-  if (a.block_threads <= 0 && cache > 0 && spread == 0) {
+  if (a.block_threads <= 0 && spread == 0 && records <= kCacheMaxNodes) {
     // occ_cache[0] keeps the kernel's register count (block sizes start at 32)
     int regs = occ_cache[0].load(std::memory_order_relaxed);
     if (regs == 0) {
@@ -1426,6 +1452,15 @@ static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cud
     const unsigned long long full = (unsigned long long)threads / 32;
     if (per_sm <= full) threads = 32 * (int)per_sm;
     else if (per_sm <= 2 * full) threads = 32 * (int)((per_sm + 1) / 2);
+  }
+  size_t cache = 0;
+  b.cache_nodes = 0;
+  if (use_cache(a, records, spread > 0, l1,
+                cache_bytes((uint32_t)records) + (size_t)(threads / 32) * ring_per_warp)) {
+    cache = cache_bytes((uint32_t)records);
+    place_records(b);
+  } else if (a.block_threads <= 0) {
+    threads = kBlockThreads;
   }
   if (threads % 32 != 0 || threads > kMaxBlockThreads) return cudaErrorInvalidValue;
   const size_t smem = cache + (size_t)(threads / 32) * ring_per_warp;
@@ -1472,22 +1507,22 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, i
       static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
       static std::atomic<int> attr{0};
       return launch_persistent(paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>, a, num_sms,
-                               st, blocks, ExitRing<T, 3>::kBytes, spread, &attr, per_sm);
+                               st, blocks, ExitRing<T, 3>::kBytes, spread, CV == kCvGrid, &attr, per_sm);
     }
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_3d<P, T, CV, MULTI, 4>, a, num_sms, st, blocks,
-                             ExitRing<T, 3>::kBytes, spread, &attr, per_sm);
+                             ExitRing<T, 3>::kBytes, spread, CV == kCvGrid, &attr, per_sm);
   } else if (longer) {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, LongSteps2D<T, CV>::value>, a, num_sms, st,
-                             blocks, ExitRing<T, 2>::kBytes, spread, &attr, per_sm);
+                             blocks, ExitRing<T, 2>::kBytes, spread, CV == kCvGrid, &attr, per_sm);
   } else {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, 2>, a, num_sms, st, blocks,
-                             ExitRing<T, 2>::kBytes, spread, &attr, per_sm);
+                             ExitRing<T, 2>::kBytes, spread, CV == kCvGrid, &attr, per_sm);
   }
 }
 
@@ -1527,8 +1562,8 @@ static cudaError_t launch_coupled_one(const PathArgs& a, int num_sms, cudaStream
   static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
   static std::atomic<int> attr{0};
   return launch_persistent(paths_coupled<P, T, CV, D>, a, num_sms, st, blocks,
-                           PairRing<T>::kBytes, spread_batch<T>(a, num_sms), &attr,
-                           per_sm);
+                           PairRing<T>::kBytes, spread_batch<T>(a, num_sms), true,
+                           &attr, per_sm);
 }
 
 template <class P, class T, int D>
