@@ -190,7 +190,9 @@ template <bool MULTI>
 __device__ __forceinline__ uint4 path_block(const PathArgs& a, uint32_t seg, uint32_t blk,
                                             uint32_t path, uint32_t node) {
   const SegArgs& sg = a.seg[MULTI ? seg : 0];
-  return philox4x32_10(make_uint4(blk, path, node, sg.seed_hi), make_uint2(sg.key0, sg.key1));
+  uint2 key = make_uint2(sg.key0, sg.key1);
+  if (MULTI) asm volatile("" : "+r"(key.x), "+r"(key.y));  // see drain()
+  return philox4x32_10(make_uint4(blk, path, node, sg.seed_hi), key);
 }
 
 // Gradient of the control grid at x.
@@ -912,25 +914,38 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEP
     // warp-uniform: few paths left, on to the drain
     if (exhausted && __popc(__ballot_sync(kFull, active)) <= Drain<T, 2>::kMaxRun) break;
     bool fin = false, trunc = false;
-#pragma unroll
-    for (int half = 0; half < STEPS / 2; ++half) {
-      uint4 w = make_uint4(0, 0, 0, 0);
-      if (active && !fin) fin = should_finish<P, T, 2>(s, ls.thr0);
-      if (active && !fin) {
-        w = path_block<MULTI>(a, s.seg, (uint32_t)(s.k >> 1), s.path, s.node);
+    // A path that ends leaves the iteration: one divergent region per iteration
+    // with one branch per test.  As a chain of steps that each ask whether the
+    // path still runs (a region, its join and a flag per step and half-step) the
+    // plain 256 x 20,000 launch took 16.9 ms, now 15.3; with the control variate
+    // 256 x 100,000 107.7 and 102.  Unrolled, the segment-table build takes 94
+    // registers instead of 72 (fixed-error run 3.24 and 3.00 ms).
+    if (active) {
+#pragma unroll (MULTI ? 1 : STEPS / 2)
+      for (int half = 0; half < STEPS / 2; ++half) {
         T n[3];
+        n[2] = T(0);
+        if (should_finish<P, T, 2>(s, ls.thr0)) {
+          fin = true;
+          break;
+        }
+        const uint4 w = path_block<MULTI>(a, s.seg, (uint32_t)(s.k >> 1), s.path, s.node);
         box_muller(w.x, w.y, n[0], n[1], ls.sqh);
-        n[2] = T(0);
         euler_step<P, T, 2, CV, MULTI>(a, s, ls, n);
-        if (s.k >= ls.max_steps) fin = trunc = true;
-      }
-      if (active && !fin) fin = should_finish<P, T, 2>(s, ls.thr0);
-      if (active && !fin) {
-        T n[3];
+        if (s.k >= ls.max_steps) {
+          fin = trunc = true;
+          break;
+        }
+        if (should_finish<P, T, 2>(s, ls.thr0)) {
+          fin = true;
+          break;
+        }
         box_muller(w.z, w.w, n[0], n[1], ls.sqh);
-        n[2] = T(0);
         euler_step<P, T, 2, CV, MULTI>(a, s, ls, n);
-        if (s.k >= ls.max_steps) fin = trunc = true;
+        if (s.k >= ls.max_steps) {
+          fin = trunc = true;
+          break;
+        }
       }
     }
     ring_exit<P, T, 2, MULTI>(a, ring, rc, s, active && fin, trunc);
@@ -960,50 +975,66 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
   while (refill<T, 3, MULTI>(a, s, ls, active, bnext, bend, exhausted)) {
     if (exhausted && __popc(__ballot_sync(kFull, active)) <= Drain<T, 3>::kMaxRun) break;
     bool fin = false, trunc = false;
-#pragma unroll
-    for (int quad = 0; quad < STEPS / 4; ++quad) {
-      T carry0 = T(0), carry1 = T(0);  // normals left over from the previous block
-      uint4 w = make_uint4(0, 0, 0, 0);
-      const uint32_t blk0 = 3u * ((uint32_t)s.k >> 2);
-      // step 0
-      if (active && !fin) fin = should_finish<P, T, 3>(s, ls.thr0);
-      if (active && !fin) {
-        w = path_block<MULTI>(a, s.seg, blk0, s.path, s.node);
-        T n[3], n3;
+    // as in paths_2d; 9,216 nodes x 2,000 paths at h = 1e-3: 4.99 -> 4.50 ms
+    // plain (4.67 unrolled), 8.89 -> 8.56 ms with the control variate (8.70
+    // not unrolled), whose bound is L1: two record loads of 32 distinct lines
+    // each are 64 wavefronts of its data pipe a warp step, 80 % of the cycles
+    if (active) {
+#pragma unroll (CV == kCvNone ? 1 : STEPS / 4)
+      for (int quad = 0; quad < STEPS / 4; ++quad) {
+        T n[3], carry0, carry1;  // carry: normals left over from the previous block
+        const uint32_t blk0 = 3u * ((uint32_t)s.k >> 2);
+        // step 0
+        if (should_finish<P, T, 3>(s, ls.thr0)) {
+          fin = true;
+          break;
+        }
+        uint4 w = path_block<MULTI>(a, s.seg, blk0, s.path, s.node);
         box_muller(w.x, w.y, n[0], n[1], ls.sqh);
-        box_muller(w.z, w.w, n[2], n3, ls.sqh);
-        carry0 = n3;
+        box_muller(w.z, w.w, n[2], carry0, ls.sqh);
         euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-        if (s.k >= ls.max_steps) fin = trunc = true;
-      }
-      // step 1
-      if (active && !fin) fin = should_finish<P, T, 3>(s, ls.thr0);
-      if (active && !fin) {
+        if (s.k >= ls.max_steps) {
+          fin = trunc = true;
+          break;
+        }
+        // step 1
+        if (should_finish<P, T, 3>(s, ls.thr0)) {
+          fin = true;
+          break;
+        }
         w = path_block<MULTI>(a, s.seg, blk0 + 1u, s.path, s.node);
-        T n[3];
         n[0] = carry0;
         box_muller(w.x, w.y, n[1], n[2], ls.sqh);
         euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-        if (s.k >= ls.max_steps) fin = trunc = true;
-      }
-      // step 2
-      if (active && !fin) fin = should_finish<P, T, 3>(s, ls.thr0);
-      if (active && !fin) {
-        T n[3];
+        if (s.k >= ls.max_steps) {
+          fin = trunc = true;
+          break;
+        }
+        // step 2
+        if (should_finish<P, T, 3>(s, ls.thr0)) {
+          fin = true;
+          break;
+        }
         box_muller(w.z, w.w, n[0], n[1], ls.sqh);
         w = path_block<MULTI>(a, s.seg, blk0 + 2u, s.path, s.node);
         box_muller(w.x, w.y, n[2], carry1, ls.sqh);
         euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-        if (s.k >= ls.max_steps) fin = trunc = true;
-      }
-      // step 3
-      if (active && !fin) fin = should_finish<P, T, 3>(s, ls.thr0);
-      if (active && !fin) {
-        T n[3];
+        if (s.k >= ls.max_steps) {
+          fin = trunc = true;
+          break;
+        }
+        // step 3
+        if (should_finish<P, T, 3>(s, ls.thr0)) {
+          fin = true;
+          break;
+        }
         n[0] = carry1;
         box_muller(w.z, w.w, n[1], n[2], ls.sqh);
         euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
-        if (s.k >= ls.max_steps) fin = trunc = true;
+        if (s.k >= ls.max_steps) {
+          fin = trunc = true;
+          break;
+        }
       }
     }
     ring_exit<P, T, 3, MULTI>(a, ring, rc, s, active && fin, trunc);
