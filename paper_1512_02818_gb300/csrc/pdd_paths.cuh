@@ -539,6 +539,30 @@ struct RingCursor {
   uint32_t head = 0, held = 0;
 };
 
+// Moves the parked exits (fewer than 32, anywhere in the ring) to the first
+// entries: NF words of type T and NU of 32 bits each.
+template <int NF, int NU = 4, class Ring>
+__device__ __forceinline__ void ring_move(const Ring& r, const RingCursor& c) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t from = (c.head - c.held + lane) & (kRing - 1);
+  if (((c.head - c.held) & (kRing - 1)) == 0u) return;
+  typename std::remove_pointer<decltype(r.f(0u))>::type f[NF];
+  uint32_t u[NU];
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < NF; ++i) f[i] = r.f(from)[32 * i];
+#pragma unroll
+  for (int i = 0; i < NU; ++i) u[i] = r.u(from)[32 * i];
+  __syncwarp();
+  if (lane < c.held) {
+#pragma unroll
+    for (int i = 0; i < NF; ++i) r.f(lane)[32 * i] = f[i];
+#pragma unroll
+    for (int i = 0; i < NU; ++i) r.u(lane)[32 * i] = u[i];
+  }
+  __syncwarp();
+}
+
 // Park the exits of this iteration (`done` lanes) and drain a full batch.
 template <class P, class T, int D, bool MULTI>
 __device__ __forceinline__ void ring_exit(const PathArgs& a, const ExitRing<T, D>& r,
@@ -840,8 +864,8 @@ template <class P, class T, int D, int CV, bool MULTI>
 __device__ __forceinline__ void drain(const PathArgs& a, const ExitRing<T, D> ring, RingCursor rc,
                                       PathState<T> s, LaneSeg<T> ls, bool active) {
   // the ring's first half parks the exits from here on, its second is scratch
-  if (rc.held > 0u) ring_drain<P, T, D, MULTI>(a, ring, rc.head - rc.held, rc.held);
-  uint32_t held = 0;
+  uint32_t held = rc.held;
+  ring_move<D + 3>(ring, rc);
   T* const nrm = (T*)(ring.base + ExitRing<T, D>::kHalf);  // scaled normals, then grad v . sigma dW
   T* const pos = nrm + (D == 2 ? 4 * Drain<T, D>::kLanes : 96);  // X, then c, f (and the dot in 3D)
   unsigned runm = __ballot_sync(kFull, active);
@@ -1176,8 +1200,8 @@ __device__ __forceinline__ void drain_pairs(const PathArgs& a, const PairRing<T>
                                             const LaneSeg<T>& lc, bool active) {
   using S4 = CoupledShape<D>;
   using Shape = PairDrain<T, D>;
-  if (rc.held > 0u) pair_drain<T>(a, ring, rc.head - rc.held, rc.held);
-  uint32_t held = 0;
+  uint32_t held = rc.held;
+  ring_move<4, 5>(ring, rc);
   T* const nrm = (T*)(ring.base + PairRing<T>::kHalf);
   T* const pos = nrm + (D == 2 ? 4 * Shape::kLanes : 96);
   T* const dots = pos + 4 * Shape::kLanes;  // 2D
