@@ -1420,8 +1420,8 @@ static int cache_block_threads(int regs) { return regs > 64 && regs <= 72 ? 448 
 // SM count blocks (at most one warp per 32 paths), with the record cache
 // when the launch's nodes fit it and `ring_per_warp` bytes of exit ring per
 // warp.  `spread` > 0: that many paths per warp (see spread_batch), in blocks
-// of 128 threads so that the warps cover the SMs evenly.  `l1`: see use_cache.
-// `attr_set` /
+// of 128 threads so that the warps cover the SMs evenly.  `warps`: see
+// target_warps; `l1`: see use_cache.  `attr_set` /
 // `occ_cache` are the kernel's own (static) state: the
 // dynamic shared memory limit set so far and the occupancy per block size
 // without the cache.
@@ -1467,6 +1467,8 @@ static int resolve_claim(const PathArgs& a, int num_sms) {
 // per warp, 450 with 4, 532 with 8; 20,480 paths: 685 us with 8, 621 with 12,
 // 703 with 16), and from 24 paths per warp on a full chip in ordinary
 // iterations is as fast (102,400 paths: 1,376 us with 24, 1,485 with 32).
+// Short paths end before the sharing pays: 100,000 of 10 steps take 37 us in
+// full warps and 43 with 24 paths per warp (20,480: 31 us and 27 with 12).
 // FP64 paths are bound by the SM's one FP64 pipe, which a warp's instruction
 // holds as long for one lane as for 32: they get one warp per scheduler.
 constexpr int kSpreadMax = 24;
@@ -1476,13 +1478,33 @@ static int spread_batch(const PathArgs& a, int num_sms) {
   const unsigned long long want = sizeof(T) == 4 ? 10 * sms : 4 * sms;  // warps
   const unsigned long long each = (a.total + want - 1) / want;
   if (a.claim > 0) return 0;  // the caller chose the claim
-  if (each <= (unsigned long long)kSpreadMax) return (int)each;
-  return sizeof(T) == 4 && a.total <= kSpreadMax * 32ull * sms ? kSpreadMax : 0;
+  const bool longer = long_iterations(a);
+  if (each <= (unsigned long long)(longer ? kSpreadMax : kSpreadMax / 2)) return (int)each;
+  return sizeof(T) == 4 && longer && a.total <= kSpreadMax * 32ull * sms ? kSpreadMax : 0;
+}
+
+// Warps per SM a launch asks for, 0 for all that fit.  With few paths per lane a
+// launch's end weighs as much as its bulk, and the fewer warps share an SM's
+// issue slots then the faster the longest paths go, while 24 (16 for the plain
+// 2D step, which waits for no load) fill them as well as 28 or 32: 256 nodes x
+// 1,000 paths at h = 1e-4 take 2.36 ms with 28 warps and 2.17 with 24 with the
+// control variate, 1.70 with 28 and 1.46 with 16 plain; x 8,000 paths 9.50 and
+// 9.67, 6.68 and 6.77.  Short paths finish so often that the plain step too
+// wants 24 (x 2,000 paths at h = 1e-2: 70 us with 28, 72 with 24, 78 with 16).
+// FP64 paths wait for the SM's one FP64 pipe, which four warps keep busy: 64
+// nodes x 1,000 paths at h = 1e-3 7.7 ms with 12 warps, 6.3 with 8, 5.2 with 4.
+template <class T, int D, int CV>
+static int target_warps(const PathArgs& a, int num_sms) {
+  if (a.block_threads > 0 || a.max_blocks > 0) return 0;  // the caller chose the shape
+  if (sizeof(T) == 8) return 4;
+  const auto few = [&](int warps) { return a.total <= 8ull * 32ull * warps * num_sms; };
+  if (D == 2 && CV == kCvNone && long_iterations(a) && few(16)) return 16;
+  return few(24) ? 24 : 0;
 }
 
 template <class K>
 static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cudaStream_t st,
-                                     int* blocks, size_t ring_per_warp, int spread, bool l1,
+                                     int* blocks, size_t ring_per_warp, int spread, int warps, bool l1,
                                      std::atomic<int>* attr_set, std::atomic<int>* occ_cache) {
   PathArgs b = a;
   b.warp_batch = spread > 0 ? (unsigned long long)spread
@@ -1502,8 +1524,9 @@ static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cud
     }
     threads = cache_block_threads(regs);
     // a launch that does not fill the chip: as many warps on every SM
-    const unsigned long long per_sm =
+    unsigned long long per_sm =
         ((a.total + b.warp_batch - 1ull) / b.warp_batch + num_sms - 1) / num_sms;
+    if (warps > 0 && per_sm > (unsigned long long)warps) per_sm = warps;
     const unsigned long long full = (unsigned long long)threads / 32;
     if (per_sm <= full) threads = 32 * (int)per_sm;
     else if (per_sm <= 2 * full) threads = 32 * (int)((per_sm + 1) / 2);
@@ -1541,6 +1564,11 @@ static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cud
       (warps_needed + (threads / 32) - 1) / (threads / 32);
   unsigned long long nb = (unsigned long long)occ * (unsigned long long)num_sms;
   if (spread > 0 && nb < blocks_needed) nb = blocks_needed;
+  if (spread == 0 && warps > 0) {
+    const unsigned long long most =
+        (unsigned long long)num_sms * ((32 * warps + threads - 1) / threads);
+    if (nb > most) nb = most;
+  }
   if (a.max_blocks > 0 && nb > (unsigned long long)a.max_blocks) nb = a.max_blocks;
   if (nb > blocks_needed) nb = blocks_needed;
   if (nb < 1) nb = 1;
@@ -1557,27 +1585,28 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, i
   const bool longer = sizeof(T) == 4 && (a.iter_mode == PDD_ITER_LONG ||
                                          (a.iter_mode == PDD_ITER_AUTO && long_iterations(a)));
   const int spread = spread_batch<T>(a, num_sms);
+  const int warps = target_warps<T, P::kDim, CV>(a, num_sms);
   if constexpr (P::kDim == 3) {
     if (longer) {
       static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
       static std::atomic<int> attr{0};
       return launch_persistent(paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>, a, num_sms,
-                               st, blocks, ExitRing<T, 3>::kBytes, spread, CV == kCvGrid, &attr, per_sm);
+                               st, blocks, ExitRing<T, 3>::kBytes, spread, warps, CV == kCvGrid, &attr, per_sm);
     }
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_3d<P, T, CV, MULTI, 4>, a, num_sms, st, blocks,
-                             ExitRing<T, 3>::kBytes, spread, CV == kCvGrid, &attr, per_sm);
+                             ExitRing<T, 3>::kBytes, spread, warps, CV == kCvGrid, &attr, per_sm);
   } else if (longer) {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, LongSteps2D<T, CV>::value>, a, num_sms, st,
-                             blocks, ExitRing<T, 2>::kBytes, spread, CV == kCvGrid, &attr, per_sm);
+                             blocks, ExitRing<T, 2>::kBytes, spread, warps, CV == kCvGrid, &attr, per_sm);
   } else {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, 2>, a, num_sms, st, blocks,
-                             ExitRing<T, 2>::kBytes, spread, CV == kCvGrid, &attr, per_sm);
+                             ExitRing<T, 2>::kBytes, spread, warps, CV == kCvGrid, &attr, per_sm);
   }
 }
 
@@ -1617,7 +1646,7 @@ static cudaError_t launch_coupled_one(const PathArgs& a, int num_sms, cudaStream
   static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
   static std::atomic<int> attr{0};
   return launch_persistent(paths_coupled<P, T, CV, D>, a, num_sms, st, blocks,
-                           PairRing<T>::kBytes, spread_batch<T>(a, num_sms), true,
+                           PairRing<T>::kBytes, spread_batch<T>(a, num_sms), 0, true,
                            &attr, per_sm);
 }
 
