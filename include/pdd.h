@@ -253,7 +253,8 @@ int pdd_ctx_get_claim(pdd_ctx* ctx, int* paths_per_lane);
    path run.  Applies to pdd_estimate_nodes / _levels, pdd_accumulate, the
    coupled calls and what runs on them (fit, MLMC); not to the
    allocation-free call or to servers (use pdd_cancel).  It allocates
-   nothing: the context made its stream, event and 16 page-locked bytes.    */
+   nothing: the context made its stream, event and 16 page-locked bytes
+   (of the 320 KB that stage the arrays of calls with host arrays).         */
 int pdd_ctx_abort(pdd_ctx* ctx);
 
 int pdd_create_problem(pdd_ctx* ctx, const pdd_problem_desc* desc, pdd_problem** out);

@@ -98,7 +98,19 @@ struct pdd_ctx {
   cudaEvent_t abort_ev = nullptr;
   unsigned long long* abort_src = nullptr;  // page-locked: {cursor past any launch, flag}
   std::atomic<bool> abort_pending{false};
+  // page-locked staging of host coordinates and results, after abort_src in its
+  // allocation; used by one call at a time (mu), which waits for its copies
+  char* pinned = nullptr;
 };
+
+// A copy to or from pageable memory costs about 8 us of the caller's time, and a
+// call with host arrays makes up to 17: 164 us for one node against 44 us with
+// device arrays.  Coordinates and results that fit go through page-locked memory
+// in one copy each way instead (45 us); beyond that the copies' own time is the
+// larger part (2,000 nodes: 224 KB).
+constexpr size_t kPinnedIn = 64 * 1024;
+constexpr size_t kPinnedOut = 256 * 1024;
+constexpr size_t kPinnedHeader = 256;
 
 struct GridSlot {
   int n = 0;
@@ -328,14 +340,22 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   const size_t off_acc = 256;
   size_t off = align_up(off_acc + total_nodes * kAccWords * 8, 256);
   size_t coord_off[PDD_MAX_LEVELS], out_off[PDD_MAX_LEVELS];
+  const size_t coords_at = off;
   for (int l = 0; l < n_levels; ++l) {
     coord_off[l] = off;
     if (!levels[l].coords_on_device) off += align_up((size_t)levels[l].n_nodes * 4, 256) * dim;
   }
+  const size_t outs_at = off;
   for (int l = 0; l < n_levels; ++l) {
     out_off[l] = off;
     if (!outs[l].on_device) off += 14 * align_up((size_t)levels[l].n_nodes * 8, 256);
   }
+  // through page-locked memory where they fit (see kPinnedIn)
+  const bool pin_in = outs_at - coords_at <= kPinnedIn;
+  const bool pin_out = off - outs_at <= kPinnedOut;
+  char* const host_hdr = c->pinned;
+  char* const host_in = c->pinned + kPinnedHeader;
+  char* const host_out = host_in + kPinnedIn;
   int rc = ensure_workspace(c, off);
   if (rc != PDD_OK) return rc;
   char* ws = (char*)c->ws;
@@ -451,12 +471,21 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
     const pdd_estimate_args& a = levels[l];
     if (a.coords_on_device || a.n_nodes == 0) continue;
     for (int j = 0; j < dim; ++j) {
-      float* dst = (float*)(ws + coord_off[l] + j * align_up((size_t)a.n_nodes * 4, 256));
+      const size_t at = coord_off[l] + j * align_up((size_t)a.n_nodes * 4, 256);
+      if (pin_in) {
+        memcpy(host_in + (at - coords_at), a.coords[j], (size_t)a.n_nodes * 4);
+        continue;
+      }
+      float* dst = (float*)(ws + at);
       PDD_CUDA(cudaMemcpyAsync(dst, a.coords[j], (size_t)a.n_nodes * 4, cudaMemcpyHostToDevice,
                                c->stream),
                "cudaMemcpyAsync(coords)");
     }
   }
+  if (pin_in && outs_at > coords_at)
+    PDD_CUDA(cudaMemcpyAsync(ws + coords_at, host_in, outs_at - coords_at, cudaMemcpyHostToDevice,
+                             c->stream),
+             "cudaMemcpyAsync(coords)");
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   if (c->timing) {
     PDD_CUDA(cudaEventCreate(&ev0), "cudaEventCreate");
@@ -512,33 +541,41 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   }
   if (c->timing) c->events.emplace_back(ev0, ev1);
   c->launches += n_launch;
-  // host outputs
-  for (int l = 0; l < n_levels; ++l) {
-    const pdd_node_stats& o = outs[l];
-    if (o.on_device || levels[l].n_nodes == 0) continue;
-    const size_t nb = (size_t)levels[l].n_nodes * 8;
-    double* const user_d[12] = {o.mean_phi, o.var_phi, o.mean_cv, o.var_cv, o.cov_phi_xi,
-                                o.var_xi, o.rho, o.se_phi, o.se_cv, o.vr, o.pred_speedup,
-                                o.mean_steps};
-    uint64_t* const user_u[2] = {o.n_paths, o.n_truncated};
-    double* const dd[12] = {sp[l].mean_phi, sp[l].var_phi, sp[l].mean_cv, sp[l].var_cv,
-                            sp[l].cov_phi_xi, sp[l].var_xi, sp[l].rho, sp[l].se_phi,
-                            sp[l].se_cv, sp[l].vr, sp[l].pred_speedup, sp[l].mean_steps};
-    unsigned long long* const du[2] = {sp[l].n_paths, sp[l].n_truncated};
-    for (int i = 0; i < 12; ++i)
-      if (user_d[i])
-        PDD_CUDA(cudaMemcpyAsync(user_d[i], dd[i], nb, cudaMemcpyDeviceToHost, c->stream),
-                 "cudaMemcpyAsync(outputs)");
-    for (int i = 0; i < 2; ++i)
-      if (user_u[i])
-        PDD_CUDA(cudaMemcpyAsync(user_u[i], du[i], nb, cudaMemcpyDeviceToHost, c->stream),
-                 "cudaMemcpyAsync(outputs)");
+  // host outputs: the results land in host_out and are copied to the caller's
+  // arrays after the wait, or each array is copied by itself
+  auto each_host_output = [&](auto&& f) {
+    for (int l = 0; l < n_levels; ++l) {
+      const pdd_node_stats& o = outs[l];
+      if (o.on_device || levels[l].n_nodes == 0) continue;
+      void* const user[14] = {o.mean_phi,  o.var_phi, o.mean_cv, o.var_cv, o.cov_phi_xi,
+                              o.var_xi,    o.rho,     o.se_phi,  o.se_cv,  o.vr,
+                              o.pred_speedup, o.mean_steps, o.n_paths, o.n_truncated};
+      const size_t nb = (size_t)levels[l].n_nodes * 8;
+      for (int i = 0; i < 14; ++i)
+        if (user[i]) f(user[i], out_off[l] + i * align_up(nb, 256), nb);
+    }
+  };
+  cudaError_t ce = cudaSuccess;
+  if (pin_out) {
+    if (off > outs_at)
+      ce = cudaMemcpyAsync(host_out, ws + outs_at, off - outs_at, cudaMemcpyDeviceToHost, c->stream);
+  } else {
+    each_host_output([&](void* user, size_t at, size_t nb) {
+      if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(user, ws + at, nb, cudaMemcpyDeviceToHost, c->stream);
+    });
   }
+  PDD_CUDA(ce, "cudaMemcpyAsync(outputs)");
   if (async) return PDD_OK;
-  WsHeader h{};
-  PDD_CUDA(cudaMemcpyAsync(&h, hdr, sizeof(h), cudaMemcpyDeviceToHost, c->stream),
+  PDD_CUDA(cudaMemcpyAsync(host_hdr, hdr, sizeof(WsHeader), cudaMemcpyDeviceToHost, c->stream),
            "cudaMemcpyAsync(header)");
   PDD_CUDA(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+  if (pin_out)
+    each_host_output([&](void* user, size_t at, size_t nb) {
+      memcpy(user, host_out + (at - outs_at), nb);
+    });
+  WsHeader h;
+  memcpy(&h, host_hdr, sizeof(h));
   if (h.aborted) return aborted_status(who);
   if (h.err != 0u) return error_word_status(h.err, who);
   if (h.cursor < pa.total) {
@@ -588,13 +625,14 @@ int pdd_ctx_create(int device, void* cuda_stream, size_t mem_budget, pdd_ctx** o
   cudaError_t ea = cudaStreamCreateWithFlags(&c->abort_stream, cudaStreamNonBlocking);
   if (ea == cudaSuccess) ea = cudaEventCreateWithFlags(&c->abort_ev, cudaEventDisableTiming);
   if (ea == cudaSuccess)
-    ea = cudaMallocHost((void**)&c->abort_src, 2 * sizeof(unsigned long long));
+    ea = cudaMallocHost((void**)&c->abort_src, 256 + kPinnedHeader + kPinnedIn + kPinnedOut);
   if (ea != cudaSuccess) {
     if (c->abort_ev) cudaEventDestroy(c->abort_ev);
     if (c->abort_stream) cudaStreamDestroy(c->abort_stream);
     delete c;
     return cuda_fail(ea, "pdd_ctx_create: abort resources");
   }
+  c->pinned = (char*)c->abort_src + 256;
   c->abort_src[0] = 1ull << 62;  // past the index space of any launch (< 2^62 paths)
   c->abort_src[1] = 1ull;        // low word: the header's `aborted`
   if (cuda_stream) {
