@@ -293,6 +293,31 @@ static int query_occupancy(pdd_problem* p, int grid_id, int threads, int* occ) {
   return PDD_OK;
 }
 
+// Copies of the node records for a launch of several levels.  The levels' paths
+// run one level after the other, so at any time only one level's records take
+// exits, about 10 ns each per record line: where a level's nodes x mean steps
+// (0.1 / dt, that of the unit box) is under about 2,000 that is as long as the
+// steps themselves.  With copies, blocks of different residues add into
+// different lines (a launch of up to kCacheMaxNodes records adds in shared
+// memory anyway).  100 levels of 6 nodes at dt = 3e-3, 4e7 paths, take 26 ms
+// instead of 225; 71 of 64 nodes, 1.2e8 paths of 10 to 100 steps, 32 instead of
+// 70; 100 of 24 nodes x 1,000 paths 0.70 instead of 0.72.
+static unsigned record_copies(int n_levels, const pdd_estimate_args* levels, size_t total_nodes) {
+  constexpr size_t kMostBytes = 16u << 20;
+  if (n_levels < 2 || total_nodes <= kCacheMaxNodes) return 1;
+  double paths = 0.0, need = 0.0;
+  for (int l = 0; l < n_levels; ++l) {
+    const double n = (double)levels[l].n_nodes * (double)levels[l].n_paths;
+    paths += n;
+    if (n > 0.0) need += n * 6000.0 * levels[l].dt / (0.1 * (double)levels[l].n_nodes);
+  }
+  unsigned copies = 1;
+  while (copies < 16 && copies * paths < need &&
+         2 * copies * total_nodes * kAccWords * 8 <= kMostBytes)
+    copies *= 2;
+  return copies;
+}
+
 static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* levels,
                          pdd_node_stats* outs, uint32_t call_flags, const char* who) {
   const int dim = p->dim;
@@ -338,7 +363,16 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   }
   // workspace: header | records | staged coordinates | staged outputs
   const size_t off_acc = 256;
-  size_t off = align_up(off_acc + total_nodes * kAccWords * 8, 256);
+  const size_t rec_bytes = total_nodes * kAccWords * 8;
+  unsigned copies = record_copies(n_levels, levels, total_nodes);
+  if (c->budget != 0) {  // copies only where the rest leaves room for them
+    size_t rest = off_acc + 256;
+    for (int l = 0; l < n_levels; ++l)
+      rest += (levels[l].coords_on_device ? 0 : dim * align_up((size_t)levels[l].n_nodes * 4, 256)) +
+              (outs[l].on_device ? 0 : 14 * align_up((size_t)levels[l].n_nodes * 8, 256));
+    while (copies > 1 && rest + copies * rec_bytes > c->budget) copies /= 2;
+  }
+  size_t off = align_up(off_acc + copies * rec_bytes, 256);
   size_t coord_off[PDD_MAX_LEVELS], out_off[PDD_MAX_LEVELS];
   const size_t coords_at = off;
   for (int l = 0; l < n_levels; ++l) {
@@ -376,6 +410,8 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   pa.block_threads = c->block_threads;
   pa.iter_mode = c->iter_mode;
   pa.claim = c->claim;
+  pa.copy_mask = copies - 1;
+  pa.copy_words = rec_bytes / 8;
   const double c0 = p->desc.exit_rule == PDD_EXIT_GOBET_MENOZZI ? 0.5826 : 0.0;
   uint32_t rec_base[PDD_MAX_LEVELS];
   {
@@ -457,14 +493,17 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   // every level.  With PDD_FLAG_GRAPH it is captured once into a CUDA graph and
   // replayed while the arguments stay the same.
   auto enqueue = [&](cudaStream_t st) -> cudaError_t {
-    cudaError_t e = cudaMemsetAsync(ws, 0, off_acc + total_nodes * kAccWords * 8, st);
+    cudaError_t e = cudaMemsetAsync(ws, 0, off_acc + copies * rec_bytes, st);
     if (e != cudaSuccess) return e;
     int blocks = 0;
     e = launch_paths(p->desc.kind, p->desc.precision, cv, pa, c->num_sms, st, &blocks);
+    if (e == cudaSuccess && copies > 1)
+      e = launch_merge_records(acc, (unsigned)total_nodes, copies, pa.copy_words, st);
     if (e != cudaSuccess) return e;
     return launch_finalize_levels(acc, n_levels, rec_base, lvl_nodes, lvl_kappa, sp, st);
   };
-  const int n_launch = 2;  // the path kernel and one finalisation for every level
+  // the path kernel, the records' copies, and one finalisation for every level
+  const int n_launch = copies > 1 ? 3 : 2;
 
   // host inputs
   for (int l = 0; l < n_levels; ++l) {
@@ -529,13 +568,15 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
     if (c->timing) PDD_CUDA(cudaEventRecord(ev1, c->stream), "cudaEventRecord");
   } else {
     wait_abort(c);
-    PDD_CUDA(cudaMemsetAsync(ws, 0, off_acc + total_nodes * kAccWords * 8, c->stream),
-             "cudaMemsetAsync");
+    PDD_CUDA(cudaMemsetAsync(ws, 0, off_acc + copies * rec_bytes, c->stream), "cudaMemsetAsync");
     if (c->timing) PDD_CUDA(cudaEventRecord(ev0, c->stream), "cudaEventRecord");
     int blocks = 0;
     PDD_CUDA(launch_paths(p->desc.kind, p->desc.precision, cv, pa, c->num_sms, c->stream, &blocks),
              "path kernel launch");
     if (c->timing) PDD_CUDA(cudaEventRecord(ev1, c->stream), "cudaEventRecord");
+    if (copies > 1)
+      PDD_CUDA(launch_merge_records(acc, (unsigned)total_nodes, copies, pa.copy_words, c->stream),
+               "merge launch");
     PDD_CUDA(launch_finalize_levels(acc, n_levels, rec_base, lvl_nodes, lvl_kappa, sp, c->stream),
              "finalize launch");
   }

@@ -79,6 +79,10 @@ struct PathArgs {
   int n_segs;                  // 1 .. kMaxSegments; segments in increasing `begin`
   uint32_t cache_nodes;        // record slots cached in shared memory per block (0: none);
                                // set by the launchers
+  // Copies of the segments' records, one per residue of the block index
+  // (copy_mask = copies - 1), copy_words words apart; 0: the records themselves.
+  unsigned copy_mask;
+  unsigned long long copy_words;
   SegArgs seg[kMaxSegments];
 };
 
@@ -166,6 +170,10 @@ cudaError_t launch_grid_pack(const double* g, int n, int dim, void* table, cudaS
 // one leaves the binary16 range).
 cudaError_t launch_grid_cells(const void* nodal, int n, int dim, void* cells, unsigned* overflow,
                               cudaStream_t st);
+// Adds the copies 1 .. copies - 1 of n_records records, `stride` words apart,
+// into the first.
+cudaError_t launch_merge_records(unsigned long long* acc, unsigned n_records, unsigned copies,
+                                 unsigned long long stride, cudaStream_t st);
 // FP32 -> FP64 copy on the device.
 cudaError_t launch_f32_to_f64(const float* src, double* dst, size_t count, cudaStream_t st);
 

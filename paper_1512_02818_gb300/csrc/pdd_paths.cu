@@ -56,6 +56,23 @@ __global__ void finalize_nodes(const unsigned long long* __restrict__ acc, uint3
   finalize_one(acc + (size_t)i * kAccWords, i, kappa, out);
 }
 
+// One thread per pair of words of a record: seven 128-bit sums, and the two
+// counts of the last pair.  Memory bound: copies x 128 B per record.
+__global__ void merge_records(unsigned long long* __restrict__ acc, unsigned pairs, unsigned copies,
+                              unsigned long long stride) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= pairs) return;
+  ulonglong2* const p = (ulonglong2*)acc + t;
+  ulonglong2 s = *p;
+  const bool counts = t % (kAccWords / 2) == kAccWords / 2 - 1;
+  for (unsigned c = 1; c < copies; ++c) {
+    const ulonglong2 v = *(const ulonglong2*)((const unsigned long long*)p + c * stride);
+    s.x += v.x;
+    s.y += v.y + (!counts && s.x < v.x ? 1ull : 0ull);
+  }
+  *p = s;
+}
+
 // All levels of a launch in one kernel: thread t finalises record t of the
 // contiguous record array, whose level is the last one with base <= t.
 struct FinalizeLevels {
@@ -141,6 +158,13 @@ cudaError_t launch_finalize_levels(const unsigned long long* acc, int n_levels,
   f.total = total;
   const unsigned threads = 128;
   finalize_levels<<<(total + threads - 1) / threads, threads, 0, st>>>(acc, f);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_merge_records(unsigned long long* acc, unsigned n_records, unsigned copies,
+                                 unsigned long long stride, cudaStream_t st) {
+  const unsigned pairs = n_records * (kAccWords / 2), threads = 256;
+  merge_records<<<(pairs + threads - 1) / threads, threads, 0, st>>>(acc, pairs, copies, stride);
   return cudaGetLastError();
 }
 

@@ -376,7 +376,9 @@ __device__ __forceinline__ void record_path(const PathArgs& a, const SegArgs& sg
                a.steps_total != nullptr ? s_cache + (size_t)a.cache_nodes * kCacheStride : nullptr,
                phi, psi, k_steps, trunc);
   } else {
-    accumulate(a, sg.acc + (size_t)node * kAccWords, a.steps_total, phi, psi, k_steps, trunc);
+    accumulate(a,
+               sg.acc + (size_t)(blockIdx.x & a.copy_mask) * a.copy_words + (size_t)node * kAccWords,
+               a.steps_total, phi, psi, k_steps, trunc);
   }
 }
 
