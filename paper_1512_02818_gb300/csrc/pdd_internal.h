@@ -76,6 +76,7 @@ struct PathArgs {
   unsigned long long warp_batch;  // path indices a warp claims at once; set by the launcher
   int one_claim;               // every warp starts one batch of its own (spread launches); set by
                                // the launcher
+  int refill_min;              // idle lanes at which a warp starts new paths; set by the launcher
   int n_segs;                  // 1 .. kMaxSegments; segments in increasing `begin`
   uint32_t cache_nodes;        // record slots cached in shared memory per block (0: none);
                                // set by the launchers

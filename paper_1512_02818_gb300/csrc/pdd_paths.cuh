@@ -113,18 +113,24 @@ __device__ __forceinline__ void load_seg(const SegArgs& sg, LaneSeg<T>& ls) {
 }
 
 // Start path g of the launch's flat index space.
+// Segment of path index g: the last one whose begin <= g.
+__device__ __forceinline__ uint32_t segment_of(const PathArgs& a, unsigned long long g) {
+  int lo = 0, hi = a.n_segs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.seg[mid].begin <= g) lo = mid;
+    else hi = mid - 1;
+  }
+  return (uint32_t)lo;
+}
+
 template <class T, int D, bool MULTI>
-__device__ __forceinline__ void start_path(const PathArgs& a, unsigned long long g,
+__device__ __forceinline__ void start_path(const PathArgs& a, unsigned long long g, uint32_t from,
                                            PathState<T>& s, LaneSeg<T>& ls) {
   uint32_t si = 0;
-  if (MULTI) {  // last segment whose begin <= g (segments in increasing begin)
-    int lo = 0, hi = a.n_segs - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.seg[mid].begin <= g) lo = mid;
-      else hi = mid - 1;
-    }
-    si = (uint32_t)lo;
+  if (MULTI) {
+    si = from;
+    while ((int)si + 1 < a.n_segs && a.seg[si + 1].begin <= g) ++si;
   }
   const SegArgs& sg = a.seg[si];
   const unsigned long long li = g - sg.begin;
@@ -408,16 +414,19 @@ __device__ __forceinline__ void finish_path(const PathArgs& a, const PathState<T
   }
 }
 
-// Refill idle lanes from the warp's batch; returns false when no lane of the
-// warp has a path left to run.  All arguments except the lane state are
-// warp-uniform.
+// Refill idle lanes from the warp's batch once a.refill_min of them are idle;
+// returns false when no lane of the warp has a path left to run.  All arguments
+// except the lane state are warp-uniform; bseg is the segment of the batch's
+// first path.
 template <class T, int D, bool MULTI>
 __device__ __forceinline__ bool refill(const PathArgs& a, PathState<T>& s, LaneSeg<T>& ls,
                                        bool& active, unsigned long long& bnext,
-                                       unsigned long long& bend, bool& exhausted) {
+                                       unsigned long long& bend, uint32_t& bseg,
+                                       bool& exhausted) {
   const unsigned lane = threadIdx.x & 31u;
   const unsigned lt = (1u << lane) - 1u;
   unsigned idle = __ballot_sync(kFull, !active);
+  if (__popc(idle) < a.refill_min) return true;
   while (idle != 0u && !exhausted) {
     if (bnext >= bend) {
       unsigned long long base = 0;
@@ -429,11 +438,12 @@ __device__ __forceinline__ bool refill(const PathArgs& a, PathState<T>& s, LaneS
       }
       bnext = base;
       bend = min(base + a.warp_batch, a.total);
+      if (MULTI) bseg = segment_of(a, base);
     }
     const unsigned avail = (unsigned)min(bend - bnext, 32ull);
     const unsigned rank = __popc(idle & lt);
     if (!active && rank < avail) {
-      start_path<T, D, MULTI>(a, bnext + rank, s, ls);
+      start_path<T, D, MULTI>(a, bnext + rank, bseg, s, ls);
       active = true;
     }
     bnext += min((unsigned)__popc(idle), avail);
@@ -444,14 +454,16 @@ __device__ __forceinline__ bool refill(const PathArgs& a, PathState<T>& s, LaneS
 
 // Spread launches (see spread_batch): every warp has a batch of its own, and
 // the cursor is past the last path when the warp asks it for more.
+template <bool MULTI>
 __device__ __forceinline__ void spread_claim(const PathArgs& a, unsigned long long& bnext,
-                                             unsigned long long& bend) {
+                                             unsigned long long& bend, uint32_t& bseg) {
   if (a.one_claim == 0) return;
   // (the shuffle tells the compiler that the batch is the warp's: without it
   // the kernels take 20 registers more)
   const unsigned warp = __shfl_sync(kFull, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, 0);
   bnext = min(warp * a.warp_batch, a.total);
   bend = min(bnext + a.warp_batch, a.total);
+  if (MULTI) bseg = segment_of(a, bnext);
   if ((threadIdx.x & 31u) == 0u) atomicAdd(a.cursor, a.total);
 }
 
@@ -935,8 +947,9 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEP
   RingCursor rc;
   bool active = false, exhausted = false;
   unsigned long long bnext = 0, bend = 0;
-  spread_claim(a, bnext, bend);
-  while (refill<T, 2, MULTI>(a, s, ls, active, bnext, bend, exhausted)) {
+  uint32_t bseg = 0;
+  spread_claim<MULTI>(a, bnext, bend, bseg);
+  while (refill<T, 2, MULTI>(a, s, ls, active, bnext, bend, bseg, exhausted)) {
     // warp-uniform: few paths left, on to the drain
     if (exhausted && __popc(__ballot_sync(kFull, active)) <= Drain<T, 2>::kMaxRun) break;
     bool fin = false, trunc = false;
@@ -997,8 +1010,9 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
   RingCursor rc;
   bool active = false, exhausted = false;
   unsigned long long bnext = 0, bend = 0;
-  spread_claim(a, bnext, bend);
-  while (refill<T, 3, MULTI>(a, s, ls, active, bnext, bend, exhausted)) {
+  uint32_t bseg = 0;
+  spread_claim<MULTI>(a, bnext, bend, bseg);
+  while (refill<T, 3, MULTI>(a, s, ls, active, bnext, bend, bseg, exhausted)) {
     if (exhausted && __popc(__ballot_sync(kFull, active)) <= Drain<T, 3>::kMaxRun) break;
     bool fin = false, trunc = false;
     // as in paths_2d; 9,216 nodes x 2,000 paths at h = 1e-3: 4.99 -> 4.50 ms
@@ -1286,8 +1300,9 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 1) paths_coupled(
   cache_init(a);
   bool active = false, exhausted = false;  // active: the pair still has work
   unsigned long long bnext = 0, bend = 0;
-  spread_claim(a, bnext, bend);
-  while (refill<T, D, false>(a, f, lf, active, bnext, bend, exhausted)) {
+  uint32_t bseg = 0;
+  spread_claim<false>(a, bnext, bend, bseg);
+  while (refill<T, D, false>(a, f, lf, active, bnext, bend, bseg, exhausted)) {
     if (active && f.k == 0 && !p.af && !p.ac) {  // refill has just started a new pair in f
       c = f;
       p.af = p.ac = true;
@@ -1423,7 +1438,7 @@ static int cache_block_threads(int regs) { return regs > 64 && regs <= 72 ? 448 
 // when the launch's nodes fit it and `ring_per_warp` bytes of exit ring per
 // warp.  `spread` > 0: that many paths per warp (see spread_batch), in blocks
 // of 128 threads so that the warps cover the SMs evenly.  `warps`: see
-// target_warps; `l1`: see use_cache.  `attr_set` /
+// target_warps; `refill`: see refill_min; `l1`: see use_cache.  `attr_set` /
 // `occ_cache` are the kernel's own (static) state: the
 // dynamic shared memory limit set so far and the occupancy per block size
 // without the cache.
@@ -1485,6 +1500,25 @@ static int spread_batch(const PathArgs& a, int num_sms) {
   return sizeof(T) == 4 && longer && a.total <= kSpreadMax * 32ull * sms ? kSpreadMax : 0;
 }
 
+// Idle lanes at which a warp starts new paths.  Starting one costs the whole
+// warp a path's set-up, so short paths, of which some lane ends at almost every
+// iteration, are started a few at a time; a lane that waits loses steps, so
+// long ones are not.  1.5e9 path-steps of the plain 2D problem with 1, 2, 3, 6
+// and 8 lanes: 9.44, 9.38, 9.26, 8.98, 8.96 ms at 10 steps a path; 7.61, 7.31,
+// 7.12, 6.99, 7.05 at 25; 5.11, 5.05, 5.05, 5.17, 5.30 at 100; 4.84, 4.79, 4.82,
+// 4.99, 5.13 at 250; 5.22, 5.25, 5.29, 5.42, 5.62 at 1,000.  The lines are the
+// same with the control variate and on the other problems.  FP64 paths: 1.
+template <class T>
+static int refill_min(const PathArgs& a) {
+  double paths = 0.0, steps = 0.0;  // 0.1 / h steps a path, that of the unit box
+  for (int i = 0; i < a.n_segs; ++i) {
+    paths += (double)a.seg[i].total;
+    steps += (double)a.seg[i].total * 0.1 / a.seg[i].h;
+  }
+  if (sizeof(T) == 8 || steps > 500.0 * paths) return 1;
+  return steps > 150.0 * paths ? 2 : steps > 30.0 * paths ? 3 : 6;
+}
+
 // Warps per SM a launch asks for, 0 for all that fit.  With few paths per lane a
 // launch's end weighs as much as its bulk, and the fewer warps share an SM's
 // issue slots then the faster the longest paths go, while 24 (16 for the plain
@@ -1506,9 +1540,10 @@ static int target_warps(const PathArgs& a, int num_sms) {
 
 template <class K>
 static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cudaStream_t st,
-                                     int* blocks, size_t ring_per_warp, int spread, int warps, bool l1,
+                                     int* blocks, size_t ring_per_warp, int spread, int warps, int refill, bool l1,
                                      std::atomic<int>* attr_set, std::atomic<int>* occ_cache) {
   PathArgs b = a;
+  b.refill_min = refill;
   b.warp_batch = spread > 0 ? (unsigned long long)spread
                             : kWarpBatch * (unsigned long long)resolve_claim(a, num_sms);
   unsigned long long records = 0;
@@ -1588,27 +1623,28 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, i
                                          (a.iter_mode == PDD_ITER_AUTO && long_iterations(a)));
   const int spread = spread_batch<T>(a, num_sms);
   const int warps = target_warps<T, P::kDim, CV>(a, num_sms);
+  const int refill = refill_min<T>(a);
   if constexpr (P::kDim == 3) {
     if (longer) {
       static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
       static std::atomic<int> attr{0};
       return launch_persistent(paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>, a, num_sms,
-                               st, blocks, ExitRing<T, 3>::kBytes, spread, warps, CV == kCvGrid, &attr, per_sm);
+                               st, blocks, ExitRing<T, 3>::kBytes, spread, warps, refill, CV == kCvGrid, &attr, per_sm);
     }
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_3d<P, T, CV, MULTI, 4>, a, num_sms, st, blocks,
-                             ExitRing<T, 3>::kBytes, spread, warps, CV == kCvGrid, &attr, per_sm);
+                             ExitRing<T, 3>::kBytes, spread, warps, refill, CV == kCvGrid, &attr, per_sm);
   } else if (longer) {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, LongSteps2D<T, CV>::value>, a, num_sms, st,
-                             blocks, ExitRing<T, 2>::kBytes, spread, warps, CV == kCvGrid, &attr, per_sm);
+                             blocks, ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid, &attr, per_sm);
   } else {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, 2>, a, num_sms, st, blocks,
-                             ExitRing<T, 2>::kBytes, spread, warps, CV == kCvGrid, &attr, per_sm);
+                             ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid, &attr, per_sm);
   }
 }
 
@@ -1648,7 +1684,7 @@ static cudaError_t launch_coupled_one(const PathArgs& a, int num_sms, cudaStream
   static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
   static std::atomic<int> attr{0};
   return launch_persistent(paths_coupled<P, T, CV, D>, a, num_sms, st, blocks,
-                           PairRing<T>::kBytes, spread_batch<T>(a, num_sms), 0, true,
+                           PairRing<T>::kBytes, spread_batch<T>(a, num_sms), 0, 1, true,
                            &attr, per_sm);
 }
 
