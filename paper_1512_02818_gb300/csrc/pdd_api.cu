@@ -829,6 +829,15 @@ int pdd_create_problem(pdd_ctx* c, const pdd_problem_desc* d, pdd_problem** out)
     set_error("pdd_create_problem: unknown precision %d", d->precision);
     return PDD_ERR_INVALID;
   }
+  if (d->precision == PDD_PATH_FP64) {
+    DeviceGuard g(c->device);
+    const F64Tables* tables = nullptr;
+    if (!g.ok) {
+      set_error("pdd_create_problem: cannot select device %d", c->device);
+      return PDD_ERR_CUDA;
+    }
+    PDD_CUDA(f64_tables(&tables), "pdd_create_problem: FP64 tables");
+  }
   pdd_problem* p = new pdd_problem();
   p->ctx = c;
   p->desc = *d;

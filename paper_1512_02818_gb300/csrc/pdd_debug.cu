@@ -46,7 +46,7 @@ __global__ void curand_philox_kernel(const uint32_t* ctr, const uint32_t* key, u
 
 template <class T>
 __global__ void normals_kernel(uint64_t seed, uint32_t tag, uint32_t node, uint32_t path,
-                               uint64_t first, int64_t count, T* out) {
+                               uint64_t first, int64_t count, T* out, const pdd::F64Tables* tb) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= count) return;
   const uint64_t i = first + (uint64_t)j;
@@ -55,9 +55,9 @@ __global__ void normals_kernel(uint64_t seed, uint32_t tag, uint32_t node, uint3
       make_uint2((uint32_t)seed, tag));
   T a, b;
   if ((i % 4) < 2)
-    pdd::box_muller(w.x, w.y, a, b);
+    pdd::box_muller(w.x, w.y, a, b, T(1), tb);
   else
-    pdd::box_muller(w.z, w.w, a, b);
+    pdd::box_muller(w.z, w.w, a, b, T(1), tb);
   out[j] = (i % 2 == 0) ? a : b;
 }
 
@@ -105,9 +105,13 @@ extern "C" int pdd_debug_normals(uint64_t seed, uint32_t tag, uint32_t node, uin
   if (count == 0) return PDD_OK;
   const unsigned blocks = (unsigned)((count + 255) / 256);
   if (precision == 0)
-    normals_kernel<float><<<blocks, 256>>>(seed, tag, node, path, first, count, out_f32);
-  else
-    normals_kernel<double><<<blocks, 256>>>(seed, tag, node, path, first, count, out_f64);
+    normals_kernel<float><<<blocks, 256>>>(seed, tag, node, path, first, count, out_f32, nullptr);
+  else {
+    const pdd::F64Tables* tb = nullptr;
+    cudaError_t e = pdd::f64_tables(&tb);
+    if (e != cudaSuccess) return finish(e);
+    normals_kernel<double><<<blocks, 256>>>(seed, tag, node, path, first, count, out_f64, tb);
+  }
   return finish(cudaGetLastError());
 }
 

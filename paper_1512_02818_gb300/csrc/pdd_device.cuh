@@ -77,8 +77,9 @@ __device__ __forceinline__ float unit_f(uint32_t w) {
 // fast sine/cosine are accurate) and the signs flipped back:
 // cos(2 pi u) = -cos(theta), sin(2 pi u) = -sin(theta).
 // `scale` multiplies both outputs (the kernels pass sqrt(h) to get dW directly).
+struct F64Tables;
 __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, float& n0, float& n1,
-                                           float scale = 1.0f) {
+                                           float scale, const F64Tables*) {
   const float ua = unit_f(wa), ub = unit_f(wb);
   const float t = -2.0f * __logf(ua);  // > 0 since ua < 1
   const float r = (scale * t) * rsqrtf(t);
@@ -88,17 +89,96 @@ __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, float& n0, 
   n0 = -r * c;
   n1 = -r * s;
 }
-__device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, double& n0, double& n1,
-                                           double scale = 1.0) {
-  const double ua = ((double)(wa >> 9) + 0.5) * 0x1p-23;
-  const double ub = ((double)(wb >> 9) + 0.5) * 0x1p-23;
-  const double r = scale * sqrt(-2.0 * log(ua));
-  const double th = (ub - 0.5) * 6.283185307179586476925286766559;
-  double s, c;
-  sincos(th, &s, &c);
-  n0 = -r * c;
-  n1 = -r * s;
+
+// ---------------------------------------------------------------------------
+// FP64 elementary functions by table.  GB300's SM has an FP64 pipe 1/64 as wide
+// as its FP32 one (16 cycles a warp instruction), and with the library's
+// functions a 2D step took about 375 FP64 instructions.  The arguments here are
+// special: 23-bit uniforms, and coordinates in [0,1].  Splitting an argument
+// into a table point and a remainder leaves a few multiply-adds, with errors of
+// about one unit in the last place (the tables are rounded from extended
+// precision): 64 nodes x 1,000 paths at h = 1e-3 with a control grid 5.2 -> 3.3
+// ms, 16,000 paths 4.0e9 path-steps/s, which is about 157 FP64 instructions a
+// step.  Errors against 113 bits over [0,1]^2, root mean square, the library's
+// and these: the normals 1.4e-16 and 1.1e-16, sin y 2.9e-17 and 2.4e-17, f
+// 7.1e-16 and 7.0e-16, grad u 3.7e-16 and 3.7e-16.
+// ---------------------------------------------------------------------------
+struct F64Tables {
+  double2 turn[4096];  // (cos, sin) of 2 pi i / 4096
+  double2 fine[2048];  // (cos - 1, sin) of 2 pi (i + 1/2) 2^-23
+  double2 ln[1024];    // (r, 2 ln r), r the FP32 reciprocal of the middle of cell i: [1 + i/1024,
+                       // 1 + (i+1)/1024), halved from 3/2 on; r = 1 in the first and last cell
+  double ln2[32];      // 2 i ln 2
+  double unit[513][6];  // sin, cos, exp of i / 256, and what rounding took from each
+};
+
+// -2 ln u of u = (2 (w >> 9) + 1) 2^-24: u = x 2^-k with x in [3/4, 3/2),
+// x = (1 + d) / r, and a polynomial in d, |d| < 2^-10 (|d| < 2^-11 and relative
+// accuracy where u is near 1).
+__device__ __forceinline__ double minus_2_ln(uint32_t w, const F64Tables* __restrict__ tb) {
+  const uint32_t m = (w >> 9) * 2u + 1u;
+  const int lz = __clz((int)m);
+  const uint32_t f = (m << lz) << 1;  // the bits below the leading one
+  const uint32_t up = f >> 31;        // x >= 3/2: halved
+  const double x = __hiloint2double((int)((0x3FF00000u - (up << 20)) | (f >> 12)), (int)(f << 20));
+  const double2 t = __ldg(&tb->ln[f >> 22]);
+  const double base = add_rn(__ldg(&tb->ln2[lz - 7 - (int)up]), t.y);
+  const double e = fma_rn(x, t.x, -1.0);
+  double p = fma_rn(e, -0.4, 0.5);
+  p = fma_rn(e, p, -2.0 / 3.0);
+  p = fma_rn(e, p, 1.0);
+  p = fma_rn(e, p, -2.0);
+  return fma_rn(e, p, base);
 }
+
+__device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, double& n0, double& n1,
+                                           double scale, const F64Tables* __restrict__ tb) {
+  const double t = minus_2_ln(wa, tb);
+  const double r = mul_rn(mul_rn(scale, t), rsqrt(t));
+  // the angle 2 pi u_b from its upper 12 bits and the rest
+  const uint32_t m = wb >> 9;
+  const double2 a = __ldg(&tb->turn[m >> 11]), b = __ldg(&tb->fine[m & 2047u]);
+  n0 = mul_rn(r, add_rn(a.x, fma_rn(a.x, b.x, -mul_rn(a.y, b.y))));
+  n1 = mul_rn(r, add_rn(a.y, fma_rn(a.y, b.x, mul_rn(a.x, b.y))));
+}
+
+// sin, cos and exp of x in [0,2]: table point i / 256 and |d| <= 1/512.  The
+// table holds its values in two parts, so the result is rounded about once.
+// (Outside, where only the drain's positions past an exit get, the point is
+// clamped and the values are not used.)
+struct UnitPoint {
+  const double* e;
+  double d, d2;
+  __device__ __forceinline__ UnitPoint(double x, const F64Tables* __restrict__ tb) {
+    const double z = add_rn(x, 0x1.8p44);  // rounds to a multiple of 1/256
+    const int i = min(max(__double2loint(z), 0), 512);
+    e = tb->unit[i];
+    d = sub_rn(x, sub_rn(z, 0x1.8p44));
+    d2 = mul_rn(d, d);
+  }
+  __device__ __forceinline__ double sin_d() const {
+    return fma_rn(d, mul_rn(d2, fma_rn(d2, 1.0 / 120.0, -1.0 / 6.0)), d);
+  }
+  __device__ __forceinline__ double cos_d_minus_1() const {
+    return mul_rn(d2, fma_rn(d2, 1.0 / 24.0, -0.5));
+  }
+  __device__ __forceinline__ double sin() const {
+    const double s = __ldg(e), c = __ldg(e + 1);
+    return add_rn(s, fma_rn(c, sin_d(), fma_rn(s, cos_d_minus_1(), __ldg(e + 3))));
+  }
+  __device__ __forceinline__ double cos() const {
+    const double s = __ldg(e), c = __ldg(e + 1);
+    return add_rn(c, fma_rn(-s, sin_d(), fma_rn(c, cos_d_minus_1(), __ldg(e + 4))));
+  }
+  __device__ __forceinline__ double exp() const {
+    const double x = __ldg(e + 2);
+    double p = fma_rn(d, 1.0 / 120.0, 1.0 / 24.0);
+    p = fma_rn(d, p, 1.0 / 6.0);
+    p = fma_rn(d, p, 0.5);
+    p = fma_rn(d2, p, d);
+    return add_rn(x, fma_rn(x, p, __ldg(e + 5)));
+  }
+};
 
 // ---------------------------------------------------------------------------
 // Built-in problems (1/2 sum a_ij d_ij u + b.grad u - c u = f on [0,1]^D,
@@ -116,11 +196,22 @@ struct Coef {
 // control variate) f is formed with the common factor e^{x+y} taken out, two
 // multiplies fewer per step (C1 plain pass +2 %, control variate +0.7 %).
 template <class T, bool GRAD>
-__device__ __forceinline__ void exp_cos_2d(T x, T y, Coef<T>& o, T& u) {
-  const T sy = m_sin(y), cx = m_cos(x);
-  const T E = m_exp(add_rn(x, y));
-  T sn, cs;
-  m_sincos(sub_rn(x, y), &sn, &cs);
+__device__ __forceinline__ void exp_cos_2d(T x, T y, Coef<T>& o, T& u, const F64Tables* tb) {
+  T sy, cx, E, sn, cs;
+  if constexpr (sizeof(T) == 8) {
+    const T w = sub_rn(x, y);
+    const UnitPoint pw(fabs(w), tb);
+    sy = UnitPoint(y, tb).sin();
+    cx = UnitPoint(x, tb).cos();
+    E = UnitPoint(add_rn(x, y), tb).exp();
+    sn = copysign(pw.sin(), w);
+    cs = pw.cos();
+  } else {
+    sy = m_sin(y);
+    cx = m_cos(x);
+    E = m_exp(add_rn(x, y));
+    m_sincos(sub_rn(x, y), &sn, &cs);
+  }
   u = mul_rn(E, cs);
   // b = (sin y, cos x) / 2 is returned without the 1/2 (kDriftHalf: the
   // Euler step multiplies it by h/2, which is exact, so X is unchanged)
@@ -150,9 +241,9 @@ struct Cfg0 {
   static constexpr bool kAniso = false;
   static constexpr bool kUnitY = false;
   template <class T, bool GRAD>
-  __device__ __forceinline__ static void eval(T x, T y, T, Coef<T>& o) {
+  __device__ __forceinline__ static void eval(T x, T y, T, Coef<T>& o, const F64Tables* tb) {
     T u;
-    exp_cos_2d<T, GRAD>(x, y, o, u);
+    exp_cos_2d<T, GRAD>(x, y, o, u, tb);
     o.sa = T(1);
   }
   template <class T>
@@ -172,13 +263,14 @@ struct Aniso {
   // a(x) = 1 + sin(2 pi x)/2, with sin(2 pi x) = -sin(2 pi (x - 1/2)).
   template <class T>
   __device__ __forceinline__ static T a_of(T x) {
+    if constexpr (sizeof(T) == 8) return fma_rn(T(-0.5), sinpi(mul_rn(T(2), sub_rn(x, T(0.5)))), T(1));
     return fma_rn(T(-0.5), m_sin(mul_rn(T(6.283185307179586476925286766559), sub_rn(x, T(0.5)))),
                   T(1));
   }
   template <class T, bool GRAD>
-  __device__ __forceinline__ static void eval(T x, T y, T, Coef<T>& o) {
+  __device__ __forceinline__ static void eval(T x, T y, T, Coef<T>& o, const F64Tables* tb) {
     T u;
-    exp_cos_2d<T, GRAD>(x, y, o, u);
+    exp_cos_2d<T, GRAD>(x, y, o, u, tb);
     const T a = a_of(x);
     // 1/2 sum a_ij u_ij = 1/2 * 2 * (a/2) * u_xy with u_xy = 2u
     o.f = fma_rn(a, u, o.f);
@@ -199,13 +291,21 @@ struct Cube3 {
   static constexpr bool kAniso = false;
   static constexpr bool kUnitY = false;
   template <class T, bool GRAD>
-  __device__ __forceinline__ static void eval(T x, T y, T z, Coef<T>& o) {
-    const T ex = m_exp(x);
-    T sy, cy, sz, cz;
-    if (GRAD) {
+  __device__ __forceinline__ static void eval(T x, T y, T z, Coef<T>& o, const F64Tables* tb) {
+    T ex, sy, cy, sz, cz;
+    if constexpr (sizeof(T) == 8) {
+      const UnitPoint py(y, tb), pz(z, tb);
+      ex = UnitPoint(x, tb).exp();
+      sy = py.sin();
+      cz = pz.cos();
+      cy = GRAD ? py.cos() : T(0);
+      sz = GRAD ? pz.sin() : T(0);
+    } else if (GRAD) {
+      ex = m_exp(x);
       m_sincos(y, &sy, &cy);
       m_sincos(z, &sz, &cz);
     } else {
+      ex = m_exp(x);
       sy = m_sin(y);
       cz = m_cos(z);
       cy = sz = T(0);
@@ -237,7 +337,7 @@ struct PaperEx {
   static constexpr bool kIsoScaled = true;  // sigma = sa * I with sa = sqrt(2)
   static constexpr bool kUnitY = false;
   template <class T, bool GRAD>
-  __device__ __forceinline__ static void eval(T x, T y, T, Coef<T>& o) {
+  __device__ __forceinline__ static void eval(T x, T y, T, Coef<T>& o, const F64Tables* tb) {
     T sp, cp, sq, cq, ss, cs;
     const T ym2 = sub_rn(y, T(2)), xm2 = sub_rn(x, T(2));
     const T p = mul_rn(mul_rn(T(2), x), ym2), q = mul_rn(mul_rn(T(3), y), xm2);
@@ -276,7 +376,7 @@ struct Harmonic {
   static constexpr bool kAniso = false;
   static constexpr bool kUnitY = true;  // c = f = 0: Y = 1, Z = 0 on every path
   template <class T, bool GRAD>
-  __device__ __forceinline__ static void eval(T x, T y, T, Coef<T>& o) {
+  __device__ __forceinline__ static void eval(T x, T y, T, Coef<T>& o, const F64Tables* tb) {
     o.b0 = o.b1 = o.b2 = T(0);
     o.c = T(0);
     o.f = T(0);
@@ -357,6 +457,18 @@ __device__ __forceinline__ bool cell_in_table(unsigned* err, int ix, int iy, int
 #endif
 }
 
+// An FP32 value of the nodal table as FP64, by its bits: conversions run on the
+// FP64 pipe.  Denormals give zero; infinities and NaN large finite values, which
+// leave the scores' fixed-point range as they do.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v);
+  const uint32_t hi = ((b >> 3) & 0x0FFFFFFFu) + 0x38000000u;
+  return __hiloint2double((int)((b & 0x7F800000u) != 0u ? hi | (b & 0x80000000u) : b & 0x80000000u),
+                          (int)((b & 0x7F800000u) != 0u ? b << 29 : 0u));
+}
+__device__ __forceinline__ float widen_to(float v, float) { return v; }
+__device__ __forceinline__ double widen_to(float v, double) { return widen(v); }
+
 // Cell index min(max(floor(x s), 0), n - 2) and the offset of x s in it,
 // frac = x s - i with one rounding.  For x s >= 0 truncation is the floor,
 // and for x s < 0 both give an index that the clamp takes to 0, so the
@@ -366,6 +478,16 @@ __device__ __forceinline__ int cell_of(T x, T s, int n, T& frac) {
   int i = (int)mul_rn(x, s);
   i = min(max(i, 0), n - 2);
   frac = fma_rn(x, s, -(T)i);
+  return i;
+}
+
+// The same in FP64 without conversions: adding 3 x 2^51 with rounding down
+// leaves floor(x s) in the low bits.
+__device__ __forceinline__ int cell_of(double x, double s, int n, double& frac) {
+  const double t = mul_rn(x, s);
+  int i = __double2loint(__dadd_rd(t, 0x1.8p52));
+  i = min(max(i, 0), n - 2);
+  frac = fma_rn(x, s, -sub_rn(__hiloint2double(0x43380000, i), 0x1.8p52));
   return i;
 }
 
@@ -381,10 +503,10 @@ __device__ __forceinline__ void grid_grad_2d(const float2* __restrict__ G, int n
   }
   const float2* p = G + (size_t)iy * n + ix;
   const float2 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + n), d = __ldg(p + n + 1);
-  const T lx0 = fma_rn(fx, sub_rn((T)b.x, (T)a.x), (T)a.x);
-  const T lx1 = fma_rn(fx, sub_rn((T)d.x, (T)c.x), (T)c.x);
-  const T ly0 = fma_rn(fx, sub_rn((T)b.y, (T)a.y), (T)a.y);
-  const T ly1 = fma_rn(fx, sub_rn((T)d.y, (T)c.y), (T)c.y);
+  const T lx0 = fma_rn(fx, sub_rn(widen_to(b.x, T(0)), widen_to(a.x, T(0))), widen_to(a.x, T(0)));
+  const T lx1 = fma_rn(fx, sub_rn(widen_to(d.x, T(0)), widen_to(c.x, T(0))), widen_to(c.x, T(0)));
+  const T ly0 = fma_rn(fx, sub_rn(widen_to(b.y, T(0)), widen_to(a.y, T(0))), widen_to(a.y, T(0)));
+  const T ly1 = fma_rn(fx, sub_rn(widen_to(d.y, T(0)), widen_to(c.y, T(0))), widen_to(c.y, T(0)));
   gx = fma_rn(fy, sub_rn(lx1, lx0), lx0);
   gy = fma_rn(fy, sub_rn(ly1, ly0), ly0);
 }
@@ -409,9 +531,9 @@ __device__ __forceinline__ void grid_grad_3d(const float4* __restrict__ G, int n
     for (int cy = 0; cy < 2; ++cy) {
       const float4* q = p + cz * nn + cy * n;
       const float4 a = __ldg(q), b = __ldg(q + 1);
-      acc[0][cy][cz] = fma_rn(fx, sub_rn((T)b.x, (T)a.x), (T)a.x);
-      acc[1][cy][cz] = fma_rn(fx, sub_rn((T)b.y, (T)a.y), (T)a.y);
-      acc[2][cy][cz] = fma_rn(fx, sub_rn((T)b.z, (T)a.z), (T)a.z);
+      acc[0][cy][cz] = fma_rn(fx, sub_rn(widen_to(b.x, T(0)), widen_to(a.x, T(0))), widen_to(a.x, T(0)));
+      acc[1][cy][cz] = fma_rn(fx, sub_rn(widen_to(b.y, T(0)), widen_to(a.y, T(0))), widen_to(a.y, T(0)));
+      acc[2][cy][cz] = fma_rn(fx, sub_rn(widen_to(b.z, T(0)), widen_to(a.z, T(0))), widen_to(a.z, T(0)));
     }
   }
   T out[3];

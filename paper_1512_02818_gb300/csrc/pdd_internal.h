@@ -61,6 +61,11 @@ struct SegArgs {
   int max_steps;
 };
 
+struct F64Tables;
+// The current device's tables of the FP64 paths (pdd_device.cuh), filled by the
+// first call for the device (made when an FP64 problem is created).
+cudaError_t f64_tables(const F64Tables** tables);
+
 // Arguments of one path-kernel launch (passed by value as a grid constant).
 struct PathArgs {
   unsigned long long total;    // sum of the segments' totals
@@ -68,6 +73,7 @@ struct PathArgs {
   unsigned* err;               // error bits (kErr*)
   unsigned long long* trunc_total;
   unsigned long long* steps_total;  // optional: sum of the exit indices of all paths run
+  const F64Tables* f64;        // FP64 paths: set by launch_paths
   int y_exp;
   int max_blocks;              // 0 = occupancy x SM count
   int block_threads;           // 0 = default (256)

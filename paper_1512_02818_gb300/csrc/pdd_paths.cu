@@ -100,8 +100,13 @@ __global__ void finalize_levels(const unsigned long long* __restrict__ acc,
 // ---------------------------------------------------------------------------
 // Dispatch by problem.
 // ---------------------------------------------------------------------------
-cudaError_t launch_paths(int kind, int precision, int cv, const PathArgs& a, int num_sms,
+cudaError_t launch_paths(int kind, int precision, int cv, const PathArgs& args, int num_sms,
                          cudaStream_t st, int* blocks) {
+  PathArgs a = args;
+  if (precision == 1) {
+    cudaError_t e = f64_tables(&a.f64);
+    if (e != cudaSuccess) return e;
+  }
   if (a.n_segs < 1 || a.n_segs > kMaxSegments) return cudaErrorInvalidValue;
   // the single-segment build follows the Euler Y rule only (see euler_step)
   const bool multi = a.n_segs > 1 || a.y_exp != 0;

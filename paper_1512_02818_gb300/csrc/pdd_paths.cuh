@@ -273,7 +273,7 @@ __device__ __forceinline__ void euler_step(const PathArgs& a, PathState<T>& s,
   T gv[3] = {T(0), T(0), T(0)};
   if (CV == kCvGrid && use_cv) grid_gradient<T, D>(a, ls, s.x, gv);
   Coef<T> o;
-  P::template eval<T, CV == kCvExact>(s.x[0], s.x[1], s.x[2], o);
+  P::template eval<T, CV == kCvExact>(s.x[0], s.x[1], s.x[2], o, a.f64);
   T sdW[3];
   noise<P, T, D>(o, dW, sdW);
   if (use_cv) {
@@ -715,11 +715,11 @@ struct BatchLane {
 template <class T, int D>
 __device__ __forceinline__ void batch_normals(const BatchLane& b, uint32_t blk, uint32_t path,
                                               uint32_t node, uint32_t seed_hi, uint2 key, T sqh,
-                                              T* nrm) {
+                                              T* nrm, const F64Tables* tb) {
   const uint4 w = philox4x32_10(make_uint4(blk, path, node, seed_hi), key);
   T n[4];
-  box_muller(w.x, w.y, n[0], n[1], sqh);
-  box_muller(w.z, w.w, n[2], n[3], sqh);
+  box_muller(w.x, w.y, n[0], n[1], sqh, tb);
+  box_muller(w.z, w.w, n[2], n[3], sqh, tb);
   if (D == 2) {
     put_vec<T, D>(nrm, 2 * b.m, b.q, b.A, n[0], n[1], T(0));
     put_vec<T, D>(nrm, 2 * b.m + 1, b.q, b.A, n[2], n[3], T(0));
@@ -768,7 +768,7 @@ __device__ __forceinline__ int batch_steps(const PathArgs& a, const LaneSeg<T>& 
       for (int j = 0; j < U; ++j) {
         put_vec<T, D>(pos, i + j, b.q, b.A, s.x[0], s.x[1], s.x[2]);
         Coef<T> o;
-        P::template eval<T, false>(s.x[0], s.x[1], s.x[2], o);
+        P::template eval<T, false>(s.x[0], s.x[1], s.x[2], o, a.f64);
         T sdW[3];
         noise<P, T, D>(o, dW[j], sdW);
         advance<P, T, D>(s.x, ls.h, o, sdW);
@@ -808,7 +808,7 @@ __device__ __forceinline__ int batch_steps(const PathArgs& a, const LaneSeg<T>& 
       T gv[3] = {T(0), T(0), T(0)}, dot = T(0);
       if (CV == kCvGrid && use_cv) grid_gradient<T, D>(a, ls, x, gv);
       Coef<T> o;
-      P::template eval<T, CV == kCvExact>(x[0], x[1], x[2], o);
+      P::template eval<T, CV == kCvExact>(x[0], x[1], x[2], o, a.f64);
       if (use_cv) {
         T dW[3], sdW[3];
         batch_noise<T, D, PAIR>(nrm, i, b, dW);
@@ -906,7 +906,8 @@ __device__ __forceinline__ void drain(const PathArgs& a, const ExitRing<T, D> ri
         // across the batches: 20 of them with per-lane keys)
         uint2 key = make_uint2(key0, key1);
         if (MULTI) asm volatile("" : "+r"(key.x), "+r"(key.y));
-        batch_normals<T, D>(b, blk0 + (uint32_t)b.m, s.path, s.node, seed_hi, key, ls.sqh, nrm);
+        batch_normals<T, D>(b, blk0 + (uint32_t)b.m, s.path, s.node, seed_hi, key, ls.sqh, nrm,
+                            a.f64);
       }
       __syncwarp();
       const int n = batch_steps<P, T, D, CV, false>(a, ls, s, nrm, pos, nrm, 2, b, S, true, use_cv,
@@ -969,7 +970,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEP
           break;
         }
         const uint4 w = path_block<MULTI>(a, s.seg, (uint32_t)(s.k >> 1), s.path, s.node);
-        box_muller(w.x, w.y, n[0], n[1], ls.sqh);
+        box_muller(w.x, w.y, n[0], n[1], ls.sqh, a.f64);
         euler_step<P, T, 2, CV, MULTI>(a, s, ls, n);
         if (s.k >= ls.max_steps) {
           fin = trunc = true;
@@ -979,7 +980,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEP
           fin = true;
           break;
         }
-        box_muller(w.z, w.w, n[0], n[1], ls.sqh);
+        box_muller(w.z, w.w, n[0], n[1], ls.sqh, a.f64);
         euler_step<P, T, 2, CV, MULTI>(a, s, ls, n);
         if (s.k >= ls.max_steps) {
           fin = trunc = true;
@@ -1030,8 +1031,8 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
           break;
         }
         uint4 w = path_block<MULTI>(a, s.seg, blk0, s.path, s.node);
-        box_muller(w.x, w.y, n[0], n[1], ls.sqh);
-        box_muller(w.z, w.w, n[2], carry0, ls.sqh);
+        box_muller(w.x, w.y, n[0], n[1], ls.sqh, a.f64);
+        box_muller(w.z, w.w, n[2], carry0, ls.sqh, a.f64);
         euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
         if (s.k >= ls.max_steps) {
           fin = trunc = true;
@@ -1044,7 +1045,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
         }
         w = path_block<MULTI>(a, s.seg, blk0 + 1u, s.path, s.node);
         n[0] = carry0;
-        box_muller(w.x, w.y, n[1], n[2], ls.sqh);
+        box_muller(w.x, w.y, n[1], n[2], ls.sqh, a.f64);
         euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
         if (s.k >= ls.max_steps) {
           fin = trunc = true;
@@ -1055,9 +1056,9 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
           fin = true;
           break;
         }
-        box_muller(w.z, w.w, n[0], n[1], ls.sqh);
+        box_muller(w.z, w.w, n[0], n[1], ls.sqh, a.f64);
         w = path_block<MULTI>(a, s.seg, blk0 + 2u, s.path, s.node);
-        box_muller(w.x, w.y, n[2], carry1, ls.sqh);
+        box_muller(w.x, w.y, n[2], carry1, ls.sqh, a.f64);
         euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
         if (s.k >= ls.max_steps) {
           fin = trunc = true;
@@ -1069,7 +1070,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
           break;
         }
         n[0] = carry1;
-        box_muller(w.z, w.w, n[1], n[2], ls.sqh);
+        box_muller(w.z, w.w, n[1], n[2], ls.sqh, a.f64);
         euler_step<P, T, 3, CV, MULTI>(a, s, ls, n);
         if (s.k >= ls.max_steps) {
           fin = trunc = true;
@@ -1246,7 +1247,7 @@ __device__ __forceinline__ void drain_pairs(const PathArgs& a, const PairRing<T>
     do {
       if (b.m < blocks)
         batch_normals<T, D>(b, S4::kBlocks * s.j + (uint32_t)b.m, s.f.path, s.f.node, sg.seed_hi,
-                            make_uint2(sg.key0, sg.key1), lf.sqh, nrm);
+                            make_uint2(sg.key0, sg.key1), lf.sqh, nrm, a.f64);
       __syncwarp();
       bool trunc = false;
       int n = batch_steps<P, T, D, CV, false>(a, lf, s.f, nrm, pos, dots, 1, b, S, s.af,
@@ -1315,8 +1316,8 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 1) paths_coupled(
 #pragma unroll
       for (int b = 0; b < S::kBlocks; ++b) {
         const uint4 w = path_block<false>(a, 0, S::kBlocks * p.j + b, f.path, f.node);
-        box_muller(w.x, w.y, n[4 * b], n[4 * b + 1], lf.sqh);
-        box_muller(w.z, w.w, n[4 * b + 2], n[4 * b + 3], lf.sqh);
+        box_muller(w.x, w.y, n[4 * b], n[4 * b + 1], lf.sqh, a.f64);
+        box_muller(w.z, w.w, n[4 * b + 2], n[4 * b + 3], lf.sqh, a.f64);
       }
       if (p.af) {
 #pragma unroll
@@ -1527,13 +1528,14 @@ static int refill_min(const PathArgs& a) {
 // control variate, 1.70 with 28 and 1.46 with 16 plain; x 8,000 paths 9.50 and
 // 9.67, 6.68 and 6.77.  Short paths finish so often that the plain step too
 // wants 24 (x 2,000 paths at h = 1e-2: 70 us with 28, 72 with 24, 78 with 16).
-// FP64 paths wait for the SM's one FP64 pipe, which four warps keep busy: 64
-// nodes x 1,000 paths at h = 1e-3 7.7 ms with 12 warps, 6.3 with 8, 5.2 with 4.
+// FP64 paths wait for the SM's one FP64 pipe, which six warps keep busy, four
+// almost: 64 nodes x 1,000 paths at h = 1e-3 take 4.5 ms with 12 warps, 3.3 with
+// 6 and with 4, x 16,000 paths 27.0, 26.2 and 28.1.
 template <class T, int D, int CV>
 static int target_warps(const PathArgs& a, int num_sms) {
   if (a.block_threads > 0 || a.max_blocks > 0) return 0;  // the caller chose the shape
-  if (sizeof(T) == 8) return 4;
   const auto few = [&](int warps) { return a.total <= 8ull * 32ull * warps * num_sms; };
+  if (sizeof(T) == 8) return few(4) ? 4 : 6;
   if (D == 2 && CV == kCvNone && long_iterations(a) && few(16)) return 16;
   return few(24) ? 24 : 0;
 }
