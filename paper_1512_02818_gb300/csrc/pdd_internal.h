@@ -37,28 +37,36 @@ constexpr uint32_t kCacheMaxNodes = 512;
 // time step, control grid, random-stream key and output records.
 // The segment covers paths path_off .. path_off + n_paths - 1 of each of its
 // n_nodes nodes (a slice of a request when a request is spread over launches).
-struct SegArgs {
+// The fields stand by use, each group within one 64-byte line of the constant
+// bank: lanes of a warp may read different segments, a line at a time, and a
+// group across two lines costs twice (the Philox words alone, read at every
+// block: 100 levels of short paths 591 us, 703 us across a line).
+struct alignas(64) SegArgs {
+  // read at every Philox block
+  uint32_t key0, key1, seed_hi;
+  uint32_t path_off;           // first path index of the segment
+  // read when a path starts
+  unsigned long long begin;    // first index of the segment in the launch's flat path space
+  unsigned long long total;    // n_nodes * n_paths
+  unsigned long long n_nodes;  // nodes of this segment
   const float* cx;
   const float* cy;
   const float* cz;
-  unsigned long long begin;    // first index of the segment in the launch's flat path space
-  unsigned long long total;    // n_nodes * n_paths
-  unsigned long long n_paths;  // paths per node in this segment
-  unsigned long long n_nodes;  // nodes of this segment
-  unsigned long long* acc;     // node records of the segment's nodes (16 words each)
   const void* grad;            // float2 (2D) / float4 (3D) gradient table; null: no grid
+  int grid_n;
+  int max_steps;
+  float h32, sqrt_h32, thr32;  // h, sqrt_h, thr0 rounded; set by the launchers
+  // read when a path ends
+  uint32_t cache_base;         // first shared-memory record slot of the segment's nodes
+  unsigned long long* acc;     // node records of the segment's nodes (16 words each)
   float* emit_phi;             // optional per-path outputs: [node * emit_stride + path]
+  unsigned long long n_paths;  // paths per node in this segment
   float* emit_xi;
   int* emit_steps;
   unsigned long long emit_stride;
   double h;
   double sqrt_h;
   double thr0;                 // c0 sqrt(h)
-  uint32_t path_off;           // first path index of the segment
-  uint32_t cache_base;         // first shared-memory record slot of the segment's nodes
-  uint32_t key0, key1, seed_hi;
-  int grid_n;
-  int max_steps;
 };
 
 struct F64Tables;

@@ -102,9 +102,15 @@ struct LaneSeg {
 
 template <class T, int D>
 __device__ __forceinline__ void load_seg(const SegArgs& sg, LaneSeg<T>& ls) {
-  ls.h = (T)sg.h;
-  ls.sqh = (T)sg.sqrt_h;
-  ls.thr0 = (T)sg.thr0;
+  if constexpr (sizeof(T) == 4) {
+    ls.h = sg.h32;
+    ls.sqh = sg.sqrt_h32;
+    ls.thr0 = sg.thr32;
+  } else {
+    ls.h = sg.h;
+    ls.sqh = sg.sqrt_h;
+    ls.thr0 = sg.thr0;
+  }
   ls.grad = sg.grad;
   if (UseCells<T, D>::value && sg.grad != nullptr)
     ls.grad = (const char*)sg.grad + cell_table_offset(sg.grid_n, D);
@@ -1546,6 +1552,11 @@ static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cud
                                      std::atomic<int>* attr_set, std::atomic<int>* occ_cache) {
   PathArgs b = a;
   b.refill_min = refill;
+  for (int i = 0; i < a.n_segs; ++i) {
+    b.seg[i].h32 = (float)a.seg[i].h;
+    b.seg[i].sqrt_h32 = (float)a.seg[i].sqrt_h;
+    b.seg[i].thr32 = (float)a.seg[i].thr0;
+  }
   b.warp_batch = spread > 0 ? (unsigned long long)spread
                             : kWarpBatch * (unsigned long long)resolve_claim(a, num_sms);
   unsigned long long records = 0;
