@@ -133,6 +133,7 @@ struct WsHeader {
   unsigned long long trunc_total;
 };
 static_assert(offsetof(WsHeader, aborted) == 12, "abort flag offset");
+static_assert(sizeof(WsHeader) == 8 * kHeaderWords, "header copied by the finalisation");
 
 // Orders the context stream after an abort enqueued since its last call, so
 // that the abort's copies land before this call resets the header.
@@ -465,12 +466,19 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   pa.total = begin;
 
   StatPtrs sp[PDD_MAX_LEVELS];
+  const unsigned long long* lvl_acc[PDD_MAX_LEVELS];
   uint32_t lvl_nodes[PDD_MAX_LEVELS];
   double lvl_kappa[PDD_MAX_LEVELS];
   for (int l = 0; l < n_levels; ++l) {
+    lvl_acc[l] = acc + (size_t)rec_base[l] * kAccWords;
     lvl_nodes[l] = (uint32_t)levels[l].n_nodes;
     lvl_kappa[l] = levels[l].kappa > 0.0 ? levels[l].kappa : 1.0;
   }
+  // host results that fit are finalised straight into page-locked memory, where
+  // outs_at of the workspace would be host_out; the header of a call that waits
+  // goes with them (a captured launch serves calls of both kinds: copied there)
+  char* const outs_mem = pin_out ? host_out - outs_at : ws;
+  char* const fin_hdr = async || graph ? nullptr : host_hdr;
   for (int l = 0; l < n_levels; ++l) {
     const pdd_node_stats& o = outs[l];
     double* const user_d[12] = {o.mean_phi, o.var_phi, o.mean_cv, o.var_cv, o.cov_phi_xi,
@@ -481,10 +489,11 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
     unsigned long long* u[2];
     const size_t n8 = align_up((size_t)levels[l].n_nodes * 8, 256);
     for (int i = 0; i < 12; ++i)
-      d[i] = (!o.on_device && user_d[i]) ? (double*)(ws + out_off[l] + i * n8) : user_d[i];
+      d[i] = (!o.on_device && user_d[i]) ? (double*)(outs_mem + out_off[l] + i * n8) : user_d[i];
     for (int i = 0; i < 2; ++i)
-      u[i] = (!o.on_device && user_u[i]) ? (unsigned long long*)(ws + out_off[l] + (12 + i) * n8)
-                                         : (unsigned long long*)user_u[i];
+      u[i] = (!o.on_device && user_u[i])
+                 ? (unsigned long long*)(outs_mem + out_off[l] + (12 + i) * n8)
+                 : (unsigned long long*)user_u[i];
     sp[l] = StatPtrs{d[0], d[1], d[2], d[3], d[4], d[5], d[6], d[7], d[8], d[9], d[10], d[11],
                      u[0], u[1]};
   }
@@ -500,7 +509,7 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
     if (e == cudaSuccess && copies > 1)
       e = launch_merge_records(acc, (unsigned)total_nodes, copies, pa.copy_words, st);
     if (e != cudaSuccess) return e;
-    return launch_finalize_levels(acc, n_levels, rec_base, lvl_nodes, lvl_kappa, sp, st);
+    return launch_finalize_levels(n_levels, lvl_acc, lvl_nodes, lvl_kappa, sp, hdr, fin_hdr, st);
   };
   // the path kernel, the records' copies, and one finalisation for every level
   const int n_launch = copies > 1 ? 3 : 2;
@@ -577,12 +586,13 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
     if (copies > 1)
       PDD_CUDA(launch_merge_records(acc, (unsigned)total_nodes, copies, pa.copy_words, c->stream),
                "merge launch");
-    PDD_CUDA(launch_finalize_levels(acc, n_levels, rec_base, lvl_nodes, lvl_kappa, sp, c->stream),
+    PDD_CUDA(launch_finalize_levels(n_levels, lvl_acc, lvl_nodes, lvl_kappa, sp, hdr, fin_hdr,
+                                    c->stream),
              "finalize launch");
   }
   if (c->timing) c->events.emplace_back(ev0, ev1);
   c->launches += n_launch;
-  // host outputs: the results land in host_out and are copied to the caller's
+  // host outputs: the results lie in host_out and are copied to the caller's
   // arrays after the wait, or each array is copied by itself
   auto each_host_output = [&](auto&& f) {
     for (int l = 0; l < n_levels; ++l) {
@@ -597,10 +607,7 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
     }
   };
   cudaError_t ce = cudaSuccess;
-  if (pin_out) {
-    if (off > outs_at)
-      ce = cudaMemcpyAsync(host_out, ws + outs_at, off - outs_at, cudaMemcpyDeviceToHost, c->stream);
-  } else {
+  if (!pin_out) {
     each_host_output([&](void* user, size_t at, size_t nb) {
       if (ce == cudaSuccess)
         ce = cudaMemcpyAsync(user, ws + at, nb, cudaMemcpyDeviceToHost, c->stream);
@@ -608,8 +615,9 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   }
   PDD_CUDA(ce, "cudaMemcpyAsync(outputs)");
   if (async) return PDD_OK;
-  PDD_CUDA(cudaMemcpyAsync(host_hdr, hdr, sizeof(WsHeader), cudaMemcpyDeviceToHost, c->stream),
-           "cudaMemcpyAsync(header)");
+  if (!fin_hdr)
+    PDD_CUDA(cudaMemcpyAsync(host_hdr, hdr, sizeof(WsHeader), cudaMemcpyDeviceToHost, c->stream),
+             "cudaMemcpyAsync(header)");
   PDD_CUDA(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
   if (pin_out)
     each_host_output([&](void* user, size_t at, size_t nb) {

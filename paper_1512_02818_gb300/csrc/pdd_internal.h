@@ -101,7 +101,7 @@ struct PathArgs {
   SegArgs seg[kMaxSegments];
 };
 
-// Per-node output pointers (device; any may be null).
+// Per-node output pointers (device or page-locked host memory; any may be null).
 struct StatPtrs {
   double* mean_phi;
   double* var_phi;
@@ -171,11 +171,26 @@ cudaError_t launch_coupled(int kind, int cv, const PathArgs& a, int num_sms, cud
                            int* blocks);
 cudaError_t launch_finalize(const unsigned long long* acc, uint32_t n_nodes, double kappa,
                             const StatPtrs& out, cudaStream_t st);
-// One launch for the records of up to kMaxSegments levels stored back to
-// back from `acc` (level l at record node_base[l]; empty levels skipped).
-cudaError_t launch_finalize_levels(const unsigned long long* acc, int n_levels,
-                                   const uint32_t* node_base, const uint32_t* n_nodes,
-                                   const double* kappa, const StatPtrs* out, cudaStream_t st);
+// One launch for the records of up to kMaxSegments levels (empty ones skipped;
+// one at least has a node).  It also copies a launch's header, kHeaderWords
+// words, to header_out (page-locked host memory) unless that is null.
+constexpr int kHeaderWords = 3;
+cudaError_t launch_finalize_levels(int n_levels, const unsigned long long* const* acc,
+                                   const uint32_t* n_nodes, const double* kappa,
+                                   const StatPtrs* out, const void* header, void* header_out,
+                                   cudaStream_t st);
+// A request entering the server's batch, in 16-byte words: records to clear,
+// and coordinates to copy from page-locked host memory.
+struct StageRequest {
+  uint4* records;
+  uint4* coords;
+  const uint4* host_coords;
+  size_t n_records, n_coords;
+};
+struct StageTable {
+  StageRequest req[kMaxSegments];
+};
+cudaError_t launch_stage_requests(const StageTable& t, int n, cudaStream_t st);
 // Gradient table of grid values v (FP64, n^D, x fastest) into float2/float4.
 cudaError_t launch_grid_gradient(const double* v, int n, int dim, void* table, cudaStream_t st);
 // Pack D interleaved gradient components (FP64) into float2/float4.

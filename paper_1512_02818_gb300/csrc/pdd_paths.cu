@@ -73,20 +73,30 @@ __global__ void merge_records(unsigned long long* __restrict__ acc, unsigned pai
   *p = s;
 }
 
-// All levels of a launch in one kernel: thread t finalises record t of the
-// contiguous record array, whose level is the last one with base <= t.
+// All levels of a launch (or all requests that end with it) in one kernel:
+// thread t finalises a record of the last level with base <= t.  Small levels
+// are bound by the launch alone, whose cost grows with its parameters (an empty
+// kernel and its wait, GB300: 8.6 us with 256 B, 10.4 with 16 KB), so the table
+// has the least of three lengths that holds the levels.  The results may lie in
+// page-locked host memory, which the threads then write themselves, with the
+// launch's header: two copies less behind a call (4.2 us of 13.3).
+template <int N>
 struct FinalizeLevels {
   uint32_t n_levels;
   uint32_t total;
-  uint32_t base[kMaxSegments + 1];  // first record of each level; base[n_levels] = total
-  double kappa[kMaxSegments];
-  StatPtrs out[kMaxSegments];
+  const unsigned long long* header;  // kHeaderWords words copied to header_out
+  unsigned long long* header_out;    // null: none
+  uint32_t base[N + 1];              // first thread of each level; base[n_levels] = total
+  double kappa[N];
+  const unsigned long long* acc[N];
+  StatPtrs out[N];
 };
-static_assert(sizeof(FinalizeLevels) < 32000, "kernel parameter size");
+static_assert(sizeof(FinalizeLevels<kMaxSegments>) < 32000, "kernel parameter size");
 
-__global__ void finalize_levels(const unsigned long long* __restrict__ acc,
-                                const __grid_constant__ FinalizeLevels f) {
+template <int N>
+__global__ void finalize_levels(const __grid_constant__ FinalizeLevels<N> f) {
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < (uint32_t)kHeaderWords && f.header_out) f.header_out[t] = f.header[t];
   if (t >= f.total) return;
   int lo = 0, hi = (int)f.n_levels - 1;
   while (lo < hi) {
@@ -94,7 +104,58 @@ __global__ void finalize_levels(const unsigned long long* __restrict__ acc,
     if (f.base[mid] <= t) lo = mid;
     else hi = mid - 1;
   }
-  finalize_one(acc + (size_t)t * kAccWords, t - f.base[lo], f.kappa[lo], f.out[lo]);
+  const uint32_t i = t - f.base[lo];
+  finalize_one(f.acc[lo] + (size_t)i * kAccWords, i, f.kappa[lo], f.out[lo]);
+}
+
+template <int N>
+static cudaError_t launch_finalize_table(int n_levels, const unsigned long long* const* acc,
+                                         const uint32_t* n_nodes, const double* kappa,
+                                         const StatPtrs* out, const void* header, void* header_out,
+                                         cudaStream_t st) {
+  FinalizeLevels<N> f{};
+  uint32_t total = 0;
+  int k = 0;
+  for (int l = 0; l < n_levels; ++l) {
+    if (n_nodes[l] == 0) continue;
+    f.base[k] = total;
+    f.kappa[k] = kappa[l];
+    f.acc[k] = acc[l];
+    f.out[k] = out[l];
+    total += n_nodes[l];
+    ++k;
+  }
+  if (k == 0) return cudaErrorInvalidValue;  // the caller has a node to finalise
+  f.n_levels = (uint32_t)k;
+  f.base[k] = total;
+  f.total = total;
+  f.header = (const unsigned long long*)header;
+  f.header_out = (unsigned long long*)header_out;
+  const unsigned threads = 128;
+  finalize_levels<N><<<(total + threads - 1) / threads, threads, 0, st>>>(f);
+  return cudaGetLastError();
+}
+
+// Requests entering the server's batch: their records cleared and their
+// coordinates fetched from page-locked host memory, blockIdx.y = the request.
+__global__ void stage_requests(const __grid_constant__ StageTable t) {
+  const StageRequest r = t.req[blockIdx.y];
+  const uint32_t step = gridDim.x * blockDim.x;
+  for (size_t i = blockIdx.x * blockDim.x + threadIdx.x; i < r.n_records; i += step)
+    r.records[i] = make_uint4(0, 0, 0, 0);
+  for (size_t i = blockIdx.x * blockDim.x + threadIdx.x; i < r.n_coords; i += step)
+    r.coords[i] = r.host_coords[i];
+}
+
+cudaError_t launch_stage_requests(const StageTable& t, int n, cudaStream_t st) {
+  if (n < 1 || n > kMaxSegments) return cudaErrorInvalidValue;
+  size_t most = 0;
+  for (int i = 0; i < n; ++i)
+    most = most > t.req[i].n_records ? most : t.req[i].n_records;
+  const size_t threads = 256, blocks = (most + threads - 1) / threads;
+  stage_requests<<<dim3((unsigned)(blocks < 304 ? blocks : 304), (unsigned)n), (unsigned)threads, 0,
+                   st>>>(t);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -141,29 +202,15 @@ cudaError_t launch_coupled(int kind, int cv, const PathArgs& a, int num_sms, cud
   }
 }
 
-cudaError_t launch_finalize_levels(const unsigned long long* acc, int n_levels,
-                                   const uint32_t* node_base, const uint32_t* n_nodes,
-                                   const double* kappa, const StatPtrs* out, cudaStream_t st) {
+cudaError_t launch_finalize_levels(int n_levels, const unsigned long long* const* acc,
+                                   const uint32_t* n_nodes, const double* kappa,
+                                   const StatPtrs* out, const void* header, void* header_out,
+                                   cudaStream_t st) {
   if (n_levels < 1 || n_levels > kMaxSegments) return cudaErrorInvalidValue;
-  FinalizeLevels f{};
-  uint32_t total = 0;
-  int k = 0;
-  for (int l = 0; l < n_levels; ++l) {
-    if (n_nodes[l] == 0) continue;
-    if (node_base[l] != total) return cudaErrorInvalidValue;  // records must be contiguous
-    f.base[k] = total;
-    f.kappa[k] = kappa[l];
-    f.out[k] = out[l];
-    total += n_nodes[l];
-    ++k;
-  }
-  if (k == 0) return cudaSuccess;
-  f.n_levels = (uint32_t)k;
-  f.base[k] = total;
-  f.total = total;
-  const unsigned threads = 128;
-  finalize_levels<<<(total + threads - 1) / threads, threads, 0, st>>>(acc, f);
-  return cudaGetLastError();
+  auto* const launch = n_levels == 1    ? launch_finalize_table<1>
+                       : n_levels <= 16 ? launch_finalize_table<16>
+                                        : launch_finalize_table<kMaxSegments>;
+  return launch(n_levels, acc, n_nodes, kappa, out, header, header_out, st);
 }
 
 cudaError_t launch_merge_records(unsigned long long* acc, unsigned n_records, unsigned copies,

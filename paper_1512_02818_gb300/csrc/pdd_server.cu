@@ -12,8 +12,8 @@
 // the previous launch drains.  A request's node records accumulate exact
 // integer sums across its slices, so its result is bit-identical to running
 // it alone (pdd_estimate_nodes).  When its last slice has been issued, its
-// finalisation and the copy of its results to page-locked host memory follow
-// on the same stream; the scheduler polls CUDA events (host side) and
+// finalisation into page-locked host memory follows on the same stream, in one
+// launch for all requests that end there; the scheduler polls CUDA events (host side) and
 // pdd_poll hands the results over.  No device code waits on anything.
 //
 // Admission by predicted work: a request's work is predicted as n_nodes x
@@ -126,8 +126,7 @@ struct Request {
   bool has_mem = false;
   int inflight = 0;  // in-flight launches that reference this request
   bool in_active = false;  // in the running batch (until the scheduler drops it)
-  cudaEvent_t ready = nullptr;  // inputs copied and records cleared
-  cudaEvent_t done = nullptr;   // results in host memory
+  cudaEvent_t done = nullptr;  // results in host memory
   Clock::time_point t_submit, t_done;
   double est_steps = 0;  // expected steps per path (for slicing)
   int group = 0;         // requests that can share a launch (problem, CV class)
@@ -160,9 +159,10 @@ struct pdd_server {
   pdd_server_desc desc{};
   cudaStream_t stream[2] = {nullptr, nullptr};
   cudaStream_t copy_stream = nullptr;
+  cudaEvent_t staged = nullptr;  // inputs of every request admitted so far
   int next_stream = 0;
   char* dev_arena = nullptr;
-  char* host_arena = nullptr;  // page-locked results
+  char* host_arena = nullptr;  // page-locked: a request's coordinates, later its results
   char* hdr = nullptr;         // per-launch header slots (cursor, err, trunc, steps): 2 x 256 B
   unsigned long long* hdr_host = nullptr;  // page-locked copies of the 2 headers (4 words each)
   cudaStream_t pilot_stream = nullptr;
@@ -193,7 +193,7 @@ namespace {
 
 int request_cv_class(const Request& r) { return r.cv == 2 ? 2 : 0; }
 
-// Bytes of device arena a request needs: records, coordinates, outputs.
+// Bytes of device arena a request takes: records, coordinates, outputs.
 size_t dev_need(int64_t n, int dim) {
   return align256((size_t)n * kAccWords * 8) + dim * align256((size_t)n * 4) +
          14 * align256((size_t)n * 8);
@@ -211,6 +211,12 @@ char* req_out_dev(pdd_server* s, const Request& r) {
   return s->dev_arena + r.dev_off + align256((size_t)r.n_nodes * kAccWords * 8) +
          r.pv.dim * align256((size_t)r.n_nodes * 4);
 }
+// Requests of at most this many nodes exchange inputs and results with host
+// memory in kernels, larger ones by copies (GB300, medians, kernels / copies: 12
+// requests of 1,000 nodes 0.75 / 0.89 ms, 12 of 20,000 3.94 / 4.10, 4 of 200,000
+// 8.8 / 9.0, 2 of 1,000,000 31.8 / 28.5: their inputs pass through the scheduler
+// thread's cache on the way to page-locked memory).
+constexpr int64_t kDirectNodes = (int64_t)1 << 18;
 
 void release_mem(pdd_server* s, Request& r) {
   if (!r.has_mem) return;
@@ -337,6 +343,9 @@ int run_pilot(pdd_server* s, const Request& r, double* steps) {
 
 // Admit pending requests while slots and arena room allow (FIFO, no overtaking).
 void admit(pdd_server* s) {
+  StageTable stage;
+  int n_stage = 0;
+  std::vector<Request*> entered;
   while (!s->pending.empty() && (int)s->active.size() < s->desc.max_active) {
     const uint64_t t = s->pending.front();
     auto it = s->reqs.find(t);
@@ -364,23 +373,46 @@ void admit(pdd_server* s) {
     r.host_bytes = hneed;
     r.has_mem = true;
     s->pending.pop_front();
-    // inputs and cleared records, ordered before every launch by `ready`
-    cudaError_t e = cudaMemsetAsync(req_acc(s, r), 0, (size_t)r.n_nodes * kAccWords * 8,
-                                    s->copy_stream);
-    for (int j = 0; j < r.pv.dim && e == cudaSuccess; ++j)
-      e = cudaMemcpyAsync(req_coord(s, r, j), r.coords[j].data(), (size_t)r.n_nodes * 4,
-                          cudaMemcpyHostToDevice, s->copy_stream);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r.ready, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventRecord(r.ready, s->copy_stream);
+    cudaError_t e = cudaSuccess;
+    if (r.n_nodes <= kDirectNodes) {
+      // the coordinates wait in the request's host memory, which its results
+      // need only once every launch of the request has run
+      const size_t n4 = align256((size_t)r.n_nodes * 4);
+      char* const host = s->host_arena + r.host_off;
+      for (int j = 0; j < r.pv.dim; ++j)
+        std::memcpy(host + j * n4, r.coords[j].data(), (size_t)r.n_nodes * 4);
+      stage.req[n_stage++] =
+          StageRequest{(uint4*)req_acc(s, r), (uint4*)req_coord(s, r, 0), (const uint4*)host,
+                       (size_t)r.n_nodes * kAccWords / 2, r.pv.dim * n4 / 16};
+    } else {
+      e = cudaMemsetAsync(req_acc(s, r), 0, (size_t)r.n_nodes * kAccWords * 8, s->copy_stream);
+      for (int j = 0; j < r.pv.dim && e == cudaSuccess; ++j)
+        e = cudaMemcpyAsync(req_coord(s, r, j), r.coords[j].data(), (size_t)r.n_nodes * 4,
+                            cudaMemcpyHostToDevice, s->copy_stream);
+    }
     if (e != cudaSuccess) {
       release_mem(s, r);
       finish_request(s, r, RState::kFailed, PDD_ERR_CUDA);
       continue;
     }
+    entered.push_back(&r);
     r.state = RState::kActive;
     r.in_active = true;
     s->active.push_back(t);
     s->st.admitted++;
+  }
+  if (entered.empty()) return;
+  // cleared records and inputs of the small ones in one launch, before every path
+  // launch by `staged` (memset, copies and event of eleven small requests held
+  // their launch up by 54 us)
+  cudaError_t e = cudaSuccess;
+  if (n_stage > 0) e = launch_stage_requests(stage, n_stage, s->copy_stream);
+  if (e == cudaSuccess) e = cudaEventRecord(s->staged, s->copy_stream);
+  if (e == cudaSuccess) return;
+  for (Request* r : entered) {
+    r->next_path = r->n_paths;  // dropped from the batch by the next retirement
+    s->st.admitted--;
+    finish_request(s, *r, RState::kFailed, PDD_ERR_CUDA);
   }
 }
 
@@ -466,9 +498,9 @@ bool issue_launch(pdd_server* s) {
   unsigned long long begin = 0;
   int ns = 0;
   Launch L;
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->staged, 0);
   for (size_t bi = 0; bi < batch.size(); ++bi) {
     Request* r = batch[bi];
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, r->ready, 0);
     const uint64_t m = take[bi];
     SegArgs& sg = pa.seg[ns++];
     sg.cx = req_coord(s, *r, 0);
@@ -512,23 +544,37 @@ bool issue_launch(pdd_server* s) {
   L.stream = sidx;
   L.t_issue = Clock::now();
   s->st.launches++;
-  // requests whose last slice is in this launch: finalise and copy out
+  // requests whose last slice is in this launch: finalised in one launch
+  // (eleven launches, copies and their gaps: 90 us behind a path launch)
   const cudaEvent_t prev = s->inflight.empty() ? nullptr : s->inflight.back().ev;
+  const unsigned long long* acc[kMaxSegments];
+  uint32_t nodes[kMaxSegments];
+  double kappa[kMaxSegments];
+  StatPtrs sp[kMaxSegments];
+  int n_last = 0;
   for (Request* r : batch) {
-    if (r->next_path < r->n_paths || e != cudaSuccess) continue;
-    // earlier slices may be in the launch on the other stream
-    if (prev) e = cudaStreamWaitEvent(st, prev, 0);
-    StatPtrs sp{};
-    char* o = req_out_dev(s, *r);
+    if (r->next_path < r->n_paths) continue;
+    acc[n_last] = req_acc(s, *r);
+    nodes[n_last] = (uint32_t)r->n_nodes;
+    kappa[n_last] = r->kappa;
+    char* o = r->n_nodes <= kDirectNodes ? s->host_arena + r->host_off : req_out_dev(s, *r);
     const size_t n8 = align256((size_t)r->n_nodes * 8);
     double* d[12];
     for (int i = 0; i < 12; ++i) d[i] = (double*)(o + i * n8);
-    sp = StatPtrs{d[0], d[1], d[2], d[3], d[4], d[5], d[6], d[7], d[8], d[9], d[10], d[11],
-                  (unsigned long long*)(o + 12 * n8), (unsigned long long*)(o + 13 * n8)};
+    sp[n_last++] = StatPtrs{d[0], d[1], d[2], d[3], d[4], d[5], d[6], d[7], d[8], d[9], d[10], d[11],
+                            (unsigned long long*)(o + 12 * n8), (unsigned long long*)(o + 13 * n8)};
+  }
+  if (n_last > 0) {
+    // earlier slices may be in the launch on the other stream
+    if (e == cudaSuccess && prev) e = cudaStreamWaitEvent(st, prev, 0);
     if (e == cudaSuccess)
-      e = launch_finalize(req_acc(s, *r), (uint32_t)r->n_nodes, r->kappa, sp, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(s->host_arena + r->host_off, o, 14 * n8, cudaMemcpyDeviceToHost, st);
+      e = launch_finalize_levels(n_last, acc, nodes, kappa, sp, nullptr, nullptr, st);
+  }
+  for (Request* r : batch) {
+    if (r->next_path < r->n_paths || e != cudaSuccess) continue;
+    if (r->n_nodes > kDirectNodes)
+      e = cudaMemcpyAsync(s->host_arena + r->host_off, req_out_dev(s, *r), host_need(r->n_nodes),
+                          cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r->done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(r->done, st);
     r->state = RState::kFinishing;
@@ -697,6 +743,7 @@ int pdd_server_create(pdd_ctx* ctx, const pdd_server_desc* desc, pdd_server** ou
   for (int i = 0; i < 2 && e == cudaSuccess; ++i)
     e = cudaStreamCreateWithFlags(&s->stream[i], cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->staged, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->pilot_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     set_error("pdd_server_create: %s", cudaGetErrorString(e));
@@ -709,6 +756,7 @@ int pdd_server_create(pdd_ctx* ctx, const pdd_server_desc* desc, pdd_server** ou
     for (auto& x : s->stream)
       if (x) cudaStreamDestroy(x);
     if (s->copy_stream) cudaStreamDestroy(s->copy_stream);
+    if (s->staged) cudaEventDestroy(s->staged);
     if (s->pilot_stream) cudaStreamDestroy(s->pilot_stream);
     return e == cudaErrorMemoryAllocation ? PDD_ERR_NOMEM : PDD_ERR_CUDA;
   }
@@ -899,7 +947,6 @@ int pdd_poll(pdd_server* s, uint64_t ticket, pdd_node_stats* out, int timeout_us
     }
     release_mem(s, r);
   }
-  if (r.ready) cudaEventDestroy(r.ready);
   if (r.done) cudaEventDestroy(r.done);
   s->reqs.erase(it);
   if (status < 0 && status != PDD_ERR_CANCELLED) set_error("pdd_poll: request failed (%d)", status);
@@ -971,7 +1018,6 @@ void pdd_server_destroy(pdd_server* s) {
   cudaStreamSynchronize(s->copy_stream);
   cudaStreamSynchronize(s->pilot_stream);
   for (auto& kv : s->reqs) {
-    if (kv.second->ready) cudaEventDestroy(kv.second->ready);
     if (kv.second->done) cudaEventDestroy(kv.second->done);
   }
   for (auto& L : s->inflight)
@@ -984,6 +1030,7 @@ void pdd_server_destroy(pdd_server* s) {
   cudaFreeHost(s->pilot_host);
   for (auto& x : s->stream) cudaStreamDestroy(x);
   cudaStreamDestroy(s->copy_stream);
+  cudaEventDestroy(s->staged);
   cudaStreamDestroy(s->pilot_stream);
   delete s;
 }
