@@ -530,10 +530,6 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
                "cudaMemcpyAsync(coords)");
     }
   }
-  if (pin_in && outs_at > coords_at)
-    PDD_CUDA(cudaMemcpyAsync(ws + coords_at, host_in, outs_at - coords_at, cudaMemcpyHostToDevice,
-                             c->stream),
-             "cudaMemcpyAsync(coords)");
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   if (c->timing) {
     PDD_CUDA(cudaEventCreate(&ev0), "cudaEventCreate");
@@ -577,7 +573,14 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
     if (c->timing) PDD_CUDA(cudaEventRecord(ev1, c->stream), "cudaEventRecord");
   } else {
     wait_abort(c);
-    PDD_CUDA(cudaMemsetAsync(ws, 0, off_acc + copies * rec_bytes, c->stream), "cudaMemsetAsync");
+    const size_t clear = off_acc + copies * rec_bytes;
+    if (pin_in && outs_at > coords_at) {  // header, records and coordinates in one launch
+      const StageRequest sr{(uint4*)ws, (uint4*)(ws + coords_at), (const uint4*)host_in, clear / 16,
+                            (outs_at - coords_at) / 16};
+      PDD_CUDA(launch_stage_requests(&sr, 1, c->stream), "staging launch");
+    } else {
+      PDD_CUDA(cudaMemsetAsync(ws, 0, clear, c->stream), "cudaMemsetAsync");
+    }
     if (c->timing) PDD_CUDA(cudaEventRecord(ev0, c->stream), "cudaEventRecord");
     int blocks = 0;
     PDD_CUDA(launch_paths(p->desc.kind, p->desc.precision, cv, pa, c->num_sms, c->stream, &blocks),

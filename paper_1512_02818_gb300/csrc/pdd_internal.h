@@ -179,18 +179,15 @@ cudaError_t launch_finalize_levels(int n_levels, const unsigned long long* const
                                    const uint32_t* n_nodes, const double* kappa,
                                    const StatPtrs* out, const void* header, void* header_out,
                                    cudaStream_t st);
-// A request entering the server's batch, in 16-byte words: records to clear,
-// and coordinates to copy from page-locked host memory.
+// A call about to run, in 16-byte words: records to clear, and coordinates to
+// copy from page-locked host memory.
 struct StageRequest {
   uint4* records;
   uint4* coords;
   const uint4* host_coords;
   size_t n_records, n_coords;
 };
-struct StageTable {
-  StageRequest req[kMaxSegments];
-};
-cudaError_t launch_stage_requests(const StageTable& t, int n, cudaStream_t st);
+cudaError_t launch_stage_requests(const StageRequest* req, int n, cudaStream_t st);
 // Gradient table of grid values v (FP64, n^D, x fastest) into float2/float4.
 cudaError_t launch_grid_gradient(const double* v, int n, int dim, void* table, cudaStream_t st);
 // Pack D interleaved gradient components (FP64) into float2/float4.

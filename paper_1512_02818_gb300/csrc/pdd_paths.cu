@@ -136,9 +136,18 @@ static cudaError_t launch_finalize_table(int n_levels, const unsigned long long*
   return cudaGetLastError();
 }
 
-// Requests entering the server's batch: their records cleared and their
-// coordinates fetched from page-locked host memory, blockIdx.y = the request.
-__global__ void stage_requests(const __grid_constant__ StageTable t) {
+// Calls about to run (one, or the requests entering the server's batch): their
+// records cleared and their coordinates fetched from page-locked host memory,
+// blockIdx.y = the call.  In place of a memset and a copy in front of a path
+// launch (GB300, whole calls on host arrays: 2,000 nodes x 20 paths 62.3 -> 59.6
+// us, 256 x 100 52.9 -> 51.4, one node the same).
+template <int N>
+struct StageTable {
+  StageRequest req[N];
+};
+
+template <int N>
+__global__ void stage_requests(const __grid_constant__ StageTable<N> t) {
   const StageRequest r = t.req[blockIdx.y];
   const uint32_t step = gridDim.x * blockDim.x;
   for (size_t i = blockIdx.x * blockDim.x + threadIdx.x; i < r.n_records; i += step)
@@ -147,15 +156,23 @@ __global__ void stage_requests(const __grid_constant__ StageTable t) {
     r.coords[i] = r.host_coords[i];
 }
 
-cudaError_t launch_stage_requests(const StageTable& t, int n, cudaStream_t st) {
-  if (n < 1 || n > kMaxSegments) return cudaErrorInvalidValue;
-  size_t most = 0;
-  for (int i = 0; i < n; ++i)
-    most = most > t.req[i].n_records ? most : t.req[i].n_records;
+template <int N>
+static cudaError_t launch_stage_table(const StageRequest* req, int n, cudaStream_t st) {
+  StageTable<N> t;
+  size_t most = 1;
+  for (int i = 0; i < n; ++i) {
+    t.req[i] = req[i];
+    most = most > req[i].n_records ? most : req[i].n_records;
+  }
   const size_t threads = 256, blocks = (most + threads - 1) / threads;
-  stage_requests<<<dim3((unsigned)(blocks < 304 ? blocks : 304), (unsigned)n), (unsigned)threads, 0,
-                   st>>>(t);
+  stage_requests<N><<<dim3((unsigned)(blocks < 304 ? blocks : 304), (unsigned)n),
+                      (unsigned)threads, 0, st>>>(t);
   return cudaGetLastError();
+}
+
+cudaError_t launch_stage_requests(const StageRequest* req, int n, cudaStream_t st) {
+  if (n < 1 || n > kMaxSegments) return cudaErrorInvalidValue;
+  return n == 1 ? launch_stage_table<1>(req, n, st) : launch_stage_table<kMaxSegments>(req, n, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -343,7 +343,7 @@ int run_pilot(pdd_server* s, const Request& r, double* steps) {
 
 // Admit pending requests while slots and arena room allow (FIFO, no overtaking).
 void admit(pdd_server* s) {
-  StageTable stage;
+  StageRequest stage[kMaxSegments];
   int n_stage = 0;
   std::vector<Request*> entered;
   while (!s->pending.empty() && (int)s->active.size() < s->desc.max_active) {
@@ -381,7 +381,7 @@ void admit(pdd_server* s) {
       char* const host = s->host_arena + r.host_off;
       for (int j = 0; j < r.pv.dim; ++j)
         std::memcpy(host + j * n4, r.coords[j].data(), (size_t)r.n_nodes * 4);
-      stage.req[n_stage++] =
+      stage[n_stage++] =
           StageRequest{(uint4*)req_acc(s, r), (uint4*)req_coord(s, r, 0), (const uint4*)host,
                        (size_t)r.n_nodes * kAccWords / 2, r.pv.dim * n4 / 16};
     } else {
