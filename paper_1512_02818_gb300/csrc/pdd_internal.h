@@ -75,7 +75,11 @@ struct F64Tables;
 cudaError_t f64_tables(const F64Tables** tables);
 
 // Arguments of one path-kernel launch (passed by value as a grid constant).
-struct PathArgs {
+// The kernels of one segment and of coupled pairs take a table of that length:
+// a launch's cost grows with its parameters (an empty kernel and its wait on
+// GB300: 11.1 us with 24 KB, 8.6 us with 256 B; a whole call of one node x 1,000
+// paths: 66 -> 61 us).
+struct PathHead {
   unsigned long long total;    // sum of the segments' totals
   unsigned long long* cursor;  // flat path cursor, zeroed before the launch
   unsigned* err;               // error bits (kErr*)
@@ -84,7 +88,7 @@ struct PathArgs {
   const F64Tables* f64;        // FP64 paths: set by launch_paths
   int y_exp;
   int max_blocks;              // 0 = occupancy x SM count
-  int block_threads;           // 0 = default (256)
+  int block_threads;           // 0 = by the launch's size
   int iter_mode;               // Euler steps per iteration: PDD_ITER_AUTO / _SHORT / _LONG
   int claim;                   // paths per lane a warp claims from the cursor at once (0: auto)
   unsigned long long warp_batch;  // path indices a warp claims at once; set by the launcher
@@ -98,8 +102,12 @@ struct PathArgs {
   // (copy_mask = copies - 1), copy_words words apart; 0: the records themselves.
   unsigned copy_mask;
   unsigned long long copy_words;
-  SegArgs seg[kMaxSegments];
 };
+template <int N>
+struct PathArgsN : PathHead {
+  SegArgs seg[N];
+};
+using PathArgs = PathArgsN<kMaxSegments>;
 
 // Per-node output pointers (device or page-locked host memory; any may be null).
 struct StatPtrs {

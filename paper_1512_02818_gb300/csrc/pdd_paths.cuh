@@ -118,9 +118,12 @@ __device__ __forceinline__ void load_seg(const SegArgs& sg, LaneSeg<T>& ls) {
   ls.max_steps = sg.max_steps;
 }
 
-// Start path g of the launch's flat index space.
+template <bool MULTI>
+constexpr int kSegs = MULTI ? kMaxSegments : 1;  // length of a kernel's segment table
+
 // Segment of path index g: the last one whose begin <= g.
-__device__ __forceinline__ uint32_t segment_of(const PathArgs& a, unsigned long long g) {
+template <class A>
+__device__ __forceinline__ uint32_t segment_of(const A& a, unsigned long long g) {
   int lo = 0, hi = a.n_segs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -130,8 +133,9 @@ __device__ __forceinline__ uint32_t segment_of(const PathArgs& a, unsigned long 
   return (uint32_t)lo;
 }
 
-template <class T, int D, bool MULTI>
-__device__ __forceinline__ void start_path(const PathArgs& a, unsigned long long g, uint32_t from,
+// Start path g of the launch's flat index space.
+template <class T, int D, bool MULTI, class A>
+__device__ __forceinline__ void start_path(const A& a, unsigned long long g, uint32_t from,
                                            PathState<T>& s, LaneSeg<T>& ls) {
   uint32_t si = 0;
   if (MULTI) {
@@ -198,8 +202,8 @@ __device__ __forceinline__ bool should_finish(const PathState<T>& s, T thr0) {
 }
 
 // Philox block `blk` of the lane's path.
-template <bool MULTI>
-__device__ __forceinline__ uint4 path_block(const PathArgs& a, uint32_t seg, uint32_t blk,
+template <bool MULTI, class A>
+__device__ __forceinline__ uint4 path_block(const A& a, uint32_t seg, uint32_t blk,
                                             uint32_t path, uint32_t node) {
   const SegArgs& sg = a.seg[MULTI ? seg : 0];
   uint2 key = make_uint2(sg.key0, sg.key1);
@@ -208,8 +212,8 @@ __device__ __forceinline__ uint4 path_block(const PathArgs& a, uint32_t seg, uin
 }
 
 // Gradient of the control grid at x.
-template <class T, int D>
-__device__ __forceinline__ void grid_gradient(const PathArgs& a, const LaneSeg<T>& ls,
+template <class T, int D, class A>
+__device__ __forceinline__ void grid_gradient(const A& a, const LaneSeg<T>& ls,
                                               const T* x, T* gv) {
   unsigned* err = PDD_DEBUG_BOUNDS ? a.err : nullptr;
   if (D == 2) {
@@ -267,8 +271,8 @@ __device__ __forceinline__ void advance(T* x, T h, const Coef<T>& o, const T* sd
 // path kernels has YRULE = false and launches with the exponential rule go to
 // the segment-table build: dropping the per-step choice made the
 // single-segment build 2.4 % faster with the control variate, 5 % without.
-template <class P, class T, int D, int CV, bool MULTI, bool YRULE = MULTI>
-__device__ __forceinline__ void euler_step(const PathArgs& a, PathState<T>& s,
+template <class P, class T, int D, int CV, bool MULTI, bool YRULE = MULTI, class A>
+__device__ __forceinline__ void euler_step(const A& a, PathState<T>& s,
                                            const LaneSeg<T>& ls, const T* dW) {
   const T h = ls.h;
   // with several segments a segment without a grid runs the plain estimator
@@ -302,8 +306,8 @@ __device__ __forceinline__ void euler_step(const PathArgs& a, PathState<T>& s,
 // Exact fixed-point accumulation of one path's (phi, psi = phi + xi, k) into a
 // node record (global, or the block's shared-memory copy), and of k into the
 // launch's step counter `steps` when there is one.
-template <class T>
-__device__ __forceinline__ void accumulate(const PathArgs& a, unsigned long long* w,
+template <class T, class A>
+__device__ __forceinline__ void accumulate(const A& a, unsigned long long* w,
                                            unsigned long long* steps, T phi, T psi, int k_steps,
                                            bool trunc) {
   long long qa, qb;
@@ -338,14 +342,16 @@ extern __shared__ unsigned long long s_cache[];
 // word of consecutive slots falls in different shared-memory banks.
 constexpr uint32_t kCacheStride = kAccWords + 1;
 
-__device__ __forceinline__ void cache_init(const PathArgs& a) {
+template <class A>
+__device__ __forceinline__ void cache_init(const A& a) {
   if (a.cache_nodes == 0) return;
   const uint32_t words = a.cache_nodes * kCacheStride + 1;
   for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) s_cache[i] = 0ull;
   __syncthreads();
 }
 
-__device__ __forceinline__ void cache_flush(const PathArgs& a) {
+template <class A>
+__device__ __forceinline__ void cache_flush(const A& a) {
   if (a.cache_nodes == 0) return;
   __syncthreads();
   const uint32_t pairs = a.cache_nodes * (kAccWords / 2);
@@ -378,8 +384,8 @@ __device__ __forceinline__ void cache_flush(const PathArgs& a) {
 }
 
 // Add one path into the record of `node` of segment `sg` (cached or global).
-template <class T>
-__device__ __forceinline__ void record_path(const PathArgs& a, const SegArgs& sg, uint32_t node,
+template <class T, class A>
+__device__ __forceinline__ void record_path(const A& a, const SegArgs& sg, uint32_t node,
                                             T phi, T psi, int k_steps, bool trunc) {
   if (!PDD_IN_BOUNDS(a, node < sg.n_nodes, kErrBoundsRecord)) return;
   if (a.cache_nodes != 0) {
@@ -405,8 +411,8 @@ __device__ __forceinline__ void score_path(const PathState<T>& s, T& phi, T& xi)
 }
 
 // Exit scoring and the exact fixed-point accumulation into the node record.
-template <class P, class T, int D, bool MULTI>
-__device__ __forceinline__ void finish_path(const PathArgs& a, const PathState<T>& s, bool trunc) {
+template <class P, class T, int D, bool MULTI, class A>
+__device__ __forceinline__ void finish_path(const A& a, const PathState<T>& s, bool trunc) {
   T phi, xi;
   score_path<P, T, D>(s, phi, xi);
   const SegArgs& sg = a.seg[MULTI ? s.seg : 0];
@@ -424,8 +430,8 @@ __device__ __forceinline__ void finish_path(const PathArgs& a, const PathState<T
 // returns false when no lane of the warp has a path left to run.  All arguments
 // except the lane state are warp-uniform; bseg is the segment of the batch's
 // first path.
-template <class T, int D, bool MULTI>
-__device__ __forceinline__ bool refill(const PathArgs& a, PathState<T>& s, LaneSeg<T>& ls,
+template <class T, int D, bool MULTI, class A>
+__device__ __forceinline__ bool refill(const A& a, PathState<T>& s, LaneSeg<T>& ls,
                                        bool& active, unsigned long long& bnext,
                                        unsigned long long& bend, uint32_t& bseg,
                                        bool& exhausted) {
@@ -460,8 +466,8 @@ __device__ __forceinline__ bool refill(const PathArgs& a, PathState<T>& s, LaneS
 
 // Spread launches (see spread_batch): every warp has a batch of its own, and
 // the cursor is past the last path when the warp asks it for more.
-template <bool MULTI>
-__device__ __forceinline__ void spread_claim(const PathArgs& a, unsigned long long& bnext,
+template <bool MULTI, class A>
+__device__ __forceinline__ void spread_claim(const A& a, unsigned long long& bnext,
                                              unsigned long long& bend, uint32_t& bseg) {
   if (a.one_claim == 0) return;
   // (the shuffle tells the compiler that the batch is the warp's: without it
@@ -503,8 +509,8 @@ __host__ __device__ __forceinline__ size_t cache_bytes(uint32_t cache_nodes) {
   return (((size_t)cache_nodes * (kAccWords + 1) + 1) * 8 + 15) / 16 * 16;
 }
 
-template <class T, int D>
-__device__ __forceinline__ ExitRing<T, D> ring_of_warp(const PathArgs& a) {
+template <class T, int D, class A>
+__device__ __forceinline__ ExitRing<T, D> ring_of_warp(const A& a) {
   return {(char*)s_cache + cache_bytes(a.cache_nodes) +
           (size_t)(threadIdx.x >> 5) * ExitRing<T, D>::kBytes};
 }
@@ -526,8 +532,8 @@ __device__ __forceinline__ void ring_put(const ExitRing<T, D>& r, uint32_t j,
 }
 
 // Score and record `count` (<= 32) parked exits starting at ring slot `first`.
-template <class P, class T, int D, bool MULTI>
-__device__ __forceinline__ void ring_drain(const PathArgs& a, const ExitRing<T, D>& r,
+template <class P, class T, int D, bool MULTI, class A>
+__device__ __forceinline__ void ring_drain(const A& a, const ExitRing<T, D>& r,
                                            uint32_t first, uint32_t count) {
   __syncwarp();
   const uint32_t lane = threadIdx.x & 31u;
@@ -584,8 +590,8 @@ __device__ __forceinline__ void ring_move(const Ring& r, const RingCursor& c) {
 }
 
 // Park the exits of this iteration (`done` lanes) and drain a full batch.
-template <class P, class T, int D, bool MULTI>
-__device__ __forceinline__ void ring_exit(const PathArgs& a, const ExitRing<T, D>& r,
+template <class P, class T, int D, bool MULTI, class A>
+__device__ __forceinline__ void ring_exit(const A& a, const ExitRing<T, D>& r,
                                           RingCursor& c, const PathState<T>& s, bool done,
                                           bool trunc) {
   const unsigned m = __ballot_sync(kFull, done);
@@ -604,8 +610,8 @@ __device__ __forceinline__ void ring_exit(const PathArgs& a, const ExitRing<T, D
   }
 }
 
-template <class T, int D>
-__device__ __forceinline__ void init_lane(const PathArgs& a, PathState<T>& s, LaneSeg<T>& ls) {
+template <class T, int D, class A>
+__device__ __forceinline__ void init_lane(const A& a, PathState<T>& s, LaneSeg<T>& ls) {
   s.x[0] = s.x[1] = s.x[2] = T(0);
   s.Y = s.Z = s.Zc = s.XI = s.XIc = T(0);
   s.k = 0;
@@ -750,8 +756,8 @@ __device__ __forceinline__ void batch_noise(const T* nrm, int i, const BatchLane
 // Passes 2 to 4 over up to S steps of every path that is `on`; returns the
 // steps the lane's path takes and whether max_steps stopped it.  dots[(i A + q)
 // dot_stride] takes grad v . sigma dW in 2D (3D keeps it beside c and f).
-template <class P, class T, int D, int CV, bool PAIR>
-__device__ __forceinline__ int batch_steps(const PathArgs& a, const LaneSeg<T>& ls,
+template <class P, class T, int D, int CV, bool PAIR, class A>
+__device__ __forceinline__ int batch_steps(const A& a, const LaneSeg<T>& ls,
                                            PathState<T>& s, const T* nrm, T* pos, T* dots,
                                            int dot_stride, const BatchLane& b, int S, bool on,
                                            bool use_cv, bool y_exp, bool& trunc) {
@@ -880,8 +886,8 @@ __device__ __forceinline__ void take_path(PathState<T>& s, int src) {
   s.k = __shfl_sync(kFull, s.k, src);
 }
 
-template <class P, class T, int D, int CV, bool MULTI>
-__device__ __forceinline__ void drain(const PathArgs& a, const ExitRing<T, D> ring, RingCursor rc,
+template <class P, class T, int D, int CV, bool MULTI, class A>
+__device__ __forceinline__ void drain(const A& a, const ExitRing<T, D> ring, RingCursor rc,
                                       PathState<T> s, LaneSeg<T> ls, bool active) {
   // the ring's first half parks the exits from here on, its second is scratch
   uint32_t held = rc.held;
@@ -945,7 +951,7 @@ template <class T, bool MULTI, int STEPS>
 constexpr int kMinBlocks2D = MULTI && sizeof(T) == 4 && STEPS == 2 ? 2 : PDD_MIN_BLOCKS_2D;
 template <class P, class T, int CV, bool MULTI, int STEPS>
 __global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEPS>))
-    paths_2d(const __grid_constant__ PathArgs a) {
+    paths_2d(const __grid_constant__ PathArgsN<kSegs<MULTI>> a) {
   PathState<T> s;
   LaneSeg<T> ls;
   init_lane<T, 2>(a, s, ls);
@@ -1008,7 +1014,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEP
 // groups of four steps run per iteration (between lane refills).
 template <class P, class T, int CV, bool MULTI, int STEPS>
 __global__ void __launch_bounds__(kMaxBlockThreads, PDD_MIN_BLOCKS_3D)
-    paths_3d(const __grid_constant__ PathArgs a) {
+    paths_3d(const __grid_constant__ PathArgsN<kSegs<MULTI>> a) {
   PathState<T> s;
   LaneSeg<T> ls;
   init_lane<T, 3>(a, s, ls);
@@ -1149,14 +1155,14 @@ struct PairRing {
   }
 };
 
-template <class T>
-__device__ __forceinline__ PairRing<T> pair_ring_of_warp(const PathArgs& a) {
+template <class T, class A>
+__device__ __forceinline__ PairRing<T> pair_ring_of_warp(const A& a) {
   return {(char*)s_cache + cache_bytes(a.cache_nodes) +
           (size_t)(threadIdx.x >> 5) * PairRing<T>::kBytes};
 }
 
-template <class T>
-__device__ __forceinline__ void pair_drain(const PathArgs& a, const PairRing<T>& r,
+template <class T, class A>
+__device__ __forceinline__ void pair_drain(const A& a, const PairRing<T>& r,
                                            uint32_t first, uint32_t count) {
   __syncwarp();
   const uint32_t lane = threadIdx.x & 31u;
@@ -1217,8 +1223,8 @@ struct PairDrain {
 };
 static_assert(32 * 6 * sizeof(float) <= PairRing<float>::kHalf, "3D pair drain scratch");
 
-template <class P, class T, int D, int CV>
-__device__ __forceinline__ void drain_pairs(const PathArgs& a, const PairRing<T> ring,
+template <class P, class T, int D, int CV, class A>
+__device__ __forceinline__ void drain_pairs(const A& a, const PairRing<T> ring,
                                             RingCursor rc, PairState<T> s, const LaneSeg<T>& lf,
                                             const LaneSeg<T>& lc, bool active) {
   using S4 = CoupledShape<D>;
@@ -1290,7 +1296,7 @@ __device__ __forceinline__ void drain_pairs(const PathArgs& a, const PairRing<T>
 
 template <class P, class T, int CV, int D>
 __global__ void __launch_bounds__(kMaxBlockThreads, 1) paths_coupled(
-    const __grid_constant__ PathArgs a) {
+    const __grid_constant__ PathArgsN<2> a) {
   using S = CoupledShape<D>;
   const PairRing<T> ring = pair_ring_of_warp<T>(a);
   RingCursor rc;
@@ -1424,7 +1430,8 @@ static bool use_cache(const PathArgs& a, unsigned long long records, bool spread
 }
 
 // Shared-memory record slots of a launch: the segments' nodes in segment order.
-static void place_records(PathArgs& b) {
+template <class A>
+static void place_records(A& b) {
   uint32_t base = 0;
   for (int i = 0; i < b.n_segs; ++i) {
     b.seg[i].cache_base = base;
@@ -1546,13 +1553,16 @@ static int target_warps(const PathArgs& a, int num_sms) {
   return few(24) ? 24 : 0;
 }
 
-template <class K>
-static cudaError_t launch_persistent(K kern, const PathArgs& a, int num_sms, cudaStream_t st,
+template <int N>
+static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs& a, int num_sms, cudaStream_t st,
                                      int* blocks, size_t ring_per_warp, int spread, int warps, int refill, bool l1,
                                      std::atomic<int>* attr_set, std::atomic<int>* occ_cache) {
-  PathArgs b = a;
+  if (a.n_segs > N) return cudaErrorInvalidValue;
+  PathArgsN<N> b;
+  (PathHead&)b = a;
   b.refill_min = refill;
   for (int i = 0; i < a.n_segs; ++i) {
+    b.seg[i] = a.seg[i];
     b.seg[i].h32 = (float)a.seg[i].h;
     b.seg[i].sqrt_h32 = (float)a.seg[i].sqrt_h;
     b.seg[i].thr32 = (float)a.seg[i].thr0;
@@ -1664,7 +1674,7 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, i
 template <class P, class T, int CV, bool MULTI>
 static cudaError_t occupancy_one(int threads, int* occ) {
   if (threads % 32 != 0 || threads < 32 || threads > kMaxBlockThreads) return cudaErrorInvalidValue;
-  void (*kern)(PathArgs);
+  void (*kern)(PathArgsN<kSegs<MULTI>>);
   if constexpr (P::kDim == 3)
     kern = paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>;
   else
