@@ -206,7 +206,8 @@ int pdd_ctx_launch_count(pdd_ctx* ctx, int64_t* launches);
 /* Number of CUDA graphs captured by PDD_FLAG_GRAPH calls on this context. */
 int pdd_ctx_graph_count(pdd_ctx* ctx, int64_t* captures);
 /* Launch shape of the path kernels: block_threads (multiple of 32 in
-   [32, 512]; 0 = 128) and a cap on the grid size (0 = occupancy x SM count).
+   [32, 512]) and a cap on the grid size; 0, the default, lets each launch take
+   the shape that its paths, node records and kernel call for.
    The shape changes only the speed: the results are exact sums keyed by
    (node, path), identical for every shape.                                  */
 int pdd_ctx_set_launch(pdd_ctx* ctx, int block_threads, int max_blocks);
@@ -232,8 +233,9 @@ int pdd_ctx_get_launch(pdd_ctx* ctx, int* block_threads, int* max_blocks, int* i
    then run them one at a time as they finish): 0 (the default) = automatic,
    4 when the launch's paths are short (the segments with time steps of at
    most 2e-3 hold at most 5 % of its expected path-steps) and it has at least
-   4 x 32 paths for every warp that can be resident, 1 otherwise; or a power
-   of two in [1, 64].  Larger claims hit the
+   4 x 32 paths for every warp that can be resident, 1 otherwise, and 1 to 24
+   paths per warp, each warp taking one batch, for launches too small to fill
+   the chip; or a power of two in [1, 64], which every launch then uses.  Larger claims hit the
    cursor less often (it matters for paths of ~10 steps) but leave more
    unstarted paths with one warp at the end of a launch.  Like the launch
    shape, the claim changes only the speed.  PDD_ERR_INVALID for other values.

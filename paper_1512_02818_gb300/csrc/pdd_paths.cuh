@@ -8,21 +8,24 @@
 // different nodes, so the paths in flight at any moment spread their record
 // atomics over all node records instead of queueing on one record's cache
 // line); warps take batches of 32 indices from a global cursor (atomicAdd)
-// and every lane whose path has finished takes the next index of its warp's
-// batch at the next iteration boundary, so lanes stay busy whatever the
-// spread of exit times (paths of one node range over ~12x the mean number of
-// steps).  The grid is persistent (occupancy x SM count blocks).  A finished
-// path parks in its warp's exit ring in shared memory and is scored and
-// recorded later, 32 at a time by the whole warp; launches with at most 512
-// node records add into a per-block shared-memory copy of the records, which
-// the block adds into the global ones at the end.  Per-node sums are exact
-// integers, so which lane, warp or block runs a path changes nothing in the
-// results.
+// and the lanes whose paths have finished take the next indices of their warp's
+// batch at an iteration boundary (short paths: once enough lanes wait, see
+// refill_min), so lanes stay busy whatever the spread of exit times (paths of
+// one node range over ~12x the mean number of steps).  The grid is persistent
+// (occupancy x SM count blocks), smaller where a launch has few paths per lane
+// (target_warps); a launch with fewer paths than lanes gives each warp one
+// smaller batch instead (spread_batch).  A finished path parks in its warp's
+// exit ring in shared memory and is scored and recorded later, 32 at a time by
+// the whole warp, into a per-block shared-memory copy of the records where that
+// pays (use_cache), which the block adds into the global ones at the end.  Once
+// the cursor is exhausted a warp with half its lanes idle takes batches of steps
+// of the paths it still holds (see Drain).  Per-node sums are exact integers, so
+// which lane, warp or block runs a path changes nothing in the results.
 //
-// One iteration takes as many Euler steps as one Philox block has normals
-// for: two steps in 2D (4 normals), four steps in 3D (3 blocks, 12 normals),
-// so no random word is wasted and every path's stream is the one fixed by
-// its (seed, stream_tag, node, path) key.
+// One iteration takes a whole number of Philox blocks' worth of Euler steps (2D:
+// two steps a block; 3D: four steps of three blocks), so no random word is wasted
+// and every path's stream is the one fixed by its (seed, stream_tag, node, path)
+// key.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -1447,15 +1450,7 @@ static void place_records(A& b) {
 // 512; the coupled kernels, above 72, are faster with one).
 static int cache_block_threads(int regs) { return regs > 64 && regs <= 72 ? 448 : 512; }
 
-// Persistent launch of `kern` over the flat index space of `a`: occupancy x
-// SM count blocks (at most one warp per 32 paths), with the record cache
-// when the launch's nodes fit it and `ring_per_warp` bytes of exit ring per
-// warp.  `spread` > 0: that many paths per warp (see spread_batch), in blocks
-// of 128 threads so that the warps cover the SMs evenly.  `warps`: see
-// target_warps; `refill`: see refill_min; `l1`: see use_cache.  `attr_set` /
-// `occ_cache` are the kernel's own (static) state: the
-// dynamic shared memory limit set so far and the occupancy per block size
-// without the cache.
+// Whether a launch takes the long iteration (see kLongPathH).
 static bool long_iterations(const PathArgs& a) {
   double all = 0.0, shorter = 0.0;
   for (int i = 0; i < a.n_segs; ++i) {
@@ -1553,10 +1548,20 @@ static int target_warps(const PathArgs& a, int num_sms) {
   return few(24) ? 24 : 0;
 }
 
+// Persistent launch of `kern` over the flat index space of `a`: occupancy x
+// SM count blocks (at most one warp per 32 paths), with the record cache
+// when the launch's nodes fit it and `ring_per_warp` bytes of exit ring per
+// warp.  `spread` > 0: that many paths per warp (see spread_batch), in blocks
+// of 128 threads so that the warps cover the SMs evenly.  `warps`: see
+// target_warps; `refill`: see refill_min; `l1`: see use_cache.  `attr_set` /
+// `occ_cache` are the kernel's own (static) state: the
+// dynamic shared memory limit set so far and the occupancy per block size
+// without the cache.
 template <int N>
-static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs& a, int num_sms, cudaStream_t st,
-                                     int* blocks, size_t ring_per_warp, int spread, int warps, int refill, bool l1,
-                                     std::atomic<int>* attr_set, std::atomic<int>* occ_cache) {
+static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs& a, int num_sms,
+                                     cudaStream_t st, int* blocks, size_t ring_per_warp, int spread,
+                                     int warps, int refill, bool l1, std::atomic<int>* attr_set,
+                                     std::atomic<int>* occ_cache) {
   if (a.n_segs > N) return cudaErrorInvalidValue;
   PathArgsN<N> b;
   (PathHead&)b = a;
@@ -1651,23 +1656,27 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, i
     if (longer) {
       static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
       static std::atomic<int> attr{0};
-      return launch_persistent(paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>, a, num_sms,
-                               st, blocks, ExitRing<T, 3>::kBytes, spread, warps, refill, CV == kCvGrid, &attr, per_sm);
+      return launch_persistent(paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>, a, num_sms, st,
+                               blocks, ExitRing<T, 3>::kBytes, spread, warps, refill,
+                               CV == kCvGrid, &attr, per_sm);
     }
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_3d<P, T, CV, MULTI, 4>, a, num_sms, st, blocks,
-                             ExitRing<T, 3>::kBytes, spread, warps, refill, CV == kCvGrid, &attr, per_sm);
+                             ExitRing<T, 3>::kBytes, spread, warps, refill, CV == kCvGrid, &attr,
+                             per_sm);
   } else if (longer) {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, LongSteps2D<T, CV>::value>, a, num_sms, st,
-                             blocks, ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid, &attr, per_sm);
+                             blocks, ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid,
+                             &attr, per_sm);
   } else {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, 2>, a, num_sms, st, blocks,
-                             ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid, &attr, per_sm);
+                             ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid, &attr,
+                             per_sm);
   }
 }
 
