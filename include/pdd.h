@@ -207,7 +207,8 @@ int pdd_ctx_launch_count(pdd_ctx* ctx, int64_t* launches);
 int pdd_ctx_graph_count(pdd_ctx* ctx, int64_t* captures);
 /* Launch shape of the path kernels: block_threads (multiple of 32 in
    [32, 512]) and a cap on the grid size; 0, the default, lets each launch take
-   the shape that its paths, node records and kernel call for.
+   the shape that its paths, node records and kernel call for.  Kernels that
+   fit an SM twice at 448 threads but once above it take 448 at most.
    The shape changes only the speed: the results are exact sums keyed by
    (node, path), identical for every shape.                                  */
 int pdd_ctx_set_launch(pdd_ctx* ctx, int block_threads, int max_blocks);

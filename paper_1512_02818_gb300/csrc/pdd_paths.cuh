@@ -944,17 +944,8 @@ __device__ __forceinline__ void drain(const A& a, const ExitRing<T, D> ring, Rin
   if (held > 0u) ring_drain<P, T, D, MULTI>(a, ring, 0u, held);
 }
 
-// The segment-table build keeps per-lane segment parameters in registers, 72
-// with the control variate (28 warps an SM).  A cap at 64 makes ptxas trade the
-// whole loop's schedule for registers: 2 x 256 nodes x 50,000 paths with the
-// control variate take 124 ms at 72 and 131 ms at 64.  Short paths want the
-// warps more (130 segments x 217 nodes x 4,942 paths of 10 to 100 steps:
-// 48.4 ms at 72, 47.3 ms at 64), so the short iteration is capped.
-template <class T, bool MULTI, int STEPS>
-constexpr int kMinBlocks2D = MULTI && sizeof(T) == 4 && STEPS == 2 ? 2 : PDD_MIN_BLOCKS_2D;
-template <class P, class T, int CV, bool MULTI, int STEPS>
-__global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEPS>))
-    paths_2d(const __grid_constant__ PathArgsN<kSegs<MULTI>> a) {
+template <class P, class T, int CV, bool MULTI, int STEPS, class A>
+__device__ __forceinline__ void run_2d(const A& a) {
   PathState<T> s;
   LaneSeg<T> ls;
   init_lane<T, 2>(a, s, ls);
@@ -974,7 +965,7 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEP
     // path still runs (a region, its join and a flag per step and half-step) the
     // plain 256 x 20,000 launch took 16.9 ms, now 15.3; with the control variate
     // 256 x 100,000 107.7 and 102.  Unrolled, the segment-table build takes 94
-    // registers instead of 72 (fixed-error run 3.24 and 3.00 ms).
+    // registers instead of 76 (fixed-error run 3.24 and 3.00 ms).
     if (active) {
 #pragma unroll (MULTI ? 1 : STEPS / 2)
       for (int half = 0; half < STEPS / 2; ++half) {
@@ -1008,6 +999,39 @@ __global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEP
   }
   drain<P, T, 2, CV, MULTI>(a, ring, rc, s, ls, active);
   cache_flush(a);
+}
+
+// The segment-table build keeps per-lane segment parameters in registers.  Its
+// short iteration is held to 64 of them: short paths want the warps (130
+// segments x 217 nodes x 4,942 paths of 10 to 100 steps: 48.4 ms at 72
+// registers, 47.3 at 64).
+template <class T, bool MULTI, int STEPS>
+constexpr int kMinBlocks2D = MULTI && sizeof(T) == 4 && STEPS == 2 ? 2 : PDD_MIN_BLOCKS_2D;
+template <class P, class T, int CV, bool MULTI, int STEPS>
+__global__ void __launch_bounds__(kMaxBlockThreads, (kMinBlocks2D<T, MULTI, STEPS>))
+    paths_2d(const __grid_constant__ PathArgsN<kSegs<MULTI>> a) {
+  run_2d<P, T, CV, MULTI, STEPS>(a);
+}
+
+// The segment-table build with the long iteration (FP32).  Left to itself it
+// takes 76 registers and one block of 512 threads an SM; asked for two such
+// blocks it fits 64 by trading the whole loop's schedule for them; under a limit
+// on the registers alone ptxas finds a schedule of 64 that is faster than both.
+// 128 segments x 2 nodes x 48,000 paths at h = 1e-4 with the control variate:
+// 81.7 ms, 65.6 and 61.0 (plain 43.4, 45.7 and 43.4); 8 segments x 32 nodes x
+// 8,000 paths 14.2 ms and 11.3; 128 x 2 x 1,387, where the drain weighs, 3.03 and
+// 3.10.  (Bounds of 1,024 threads, 57 registers: 61.0, 42.8, 11.2, 3.15.)
+template <class P, int CV>
+__global__ void __maxnreg__(72)
+    paths_2d_table(const __grid_constant__ PathArgs a) {
+  run_2d<P, float, CV, true, LongSteps2D<float, CV>::value>(a);
+}
+
+// The long-iteration kernel of a build.
+template <class P, class T, int CV, bool MULTI>
+constexpr auto long_kernel_2d() {
+  if constexpr (MULTI && sizeof(T) == 4) return paths_2d_table<P, CV>;
+  else return paths_2d<P, T, CV, MULTI, LongSteps2D<T, CV>::value>;
 }
 
 // 3D: steps 4j .. 4j+3 use normals 12j .. 12j+11, i.e. Philox blocks 3j,
@@ -1447,8 +1471,11 @@ static void place_records(A& b) {
 // warps share one copy of the records, and two blocks to an SM where that
 // costs few warps (up to 64 registers a thread: 512 threads, 72: 448, which
 // measured 23.0 -> 16.6 ms on 512 nodes x 10-step paths against one block of
-// 512; the coupled kernels, above 72, are faster with one).
-static int cache_block_threads(int regs) { return regs > 64 && regs <= 72 ? 448 : 512; }
+// 512; the coupled kernels, above 72, are faster with one).  A caller's choice
+// of more threads, made for another kernel, is cut to it (31,744 nodes of the
+// anisotropic problem, 69 registers: 75.3 ms with 512 threads, 62.3 with 448).
+constexpr int kTwoBlocks72 = 448;
+static int cache_block_threads(int regs) { return regs > 64 && regs <= 72 ? kTwoBlocks72 : 512; }
 
 // Whether a launch takes the long iteration (see kLongPathH).
 static bool long_iterations(const PathArgs& a) {
@@ -1577,7 +1604,9 @@ static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs&
   unsigned long long records = 0;
   for (int i = 0; i < a.n_segs; ++i) records += a.seg[i].n_nodes;
   int threads = a.block_threads > 0 ? a.block_threads : kBlockThreads;
-  if (a.block_threads <= 0 && spread == 0 && records <= kCacheMaxNodes) {
+  if (threads % 32 != 0 || threads > kMaxBlockThreads) return cudaErrorInvalidValue;
+  const bool sized = a.block_threads <= 0 && spread == 0 && records <= kCacheMaxNodes;
+  if (sized || threads > kTwoBlocks72) {
     // occ_cache[0] keeps the kernel's register count (block sizes start at 32)
     int regs = occ_cache[0].load(std::memory_order_relaxed);
     if (regs == 0) {
@@ -1587,7 +1616,10 @@ static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs&
       regs = fa.numRegs > 0 ? fa.numRegs : 1;
       occ_cache[0].store(regs, std::memory_order_relaxed);
     }
-    threads = cache_block_threads(regs);
+    const int most = cache_block_threads(regs);
+    if (sized || threads > most) threads = most;
+  }
+  if (sized) {
     // a launch that does not fill the chip: as many warps on every SM
     unsigned long long per_sm =
         ((a.total + b.warp_batch - 1ull) / b.warp_batch + num_sms - 1) / num_sms;
@@ -1605,7 +1637,6 @@ static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs&
   } else if (a.block_threads <= 0) {
     threads = kBlockThreads;
   }
-  if (threads % 32 != 0 || threads > kMaxBlockThreads) return cudaErrorInvalidValue;
   const size_t smem = cache + (size_t)(threads / 32) * ring_per_warp;
   if (smem > 48u * 1024u && (int)smem > attr_set->load(std::memory_order_relaxed)) {
     const int lim = (int)(cache_bytes(kCacheMaxNodes) + (kMaxBlockThreads / 32) * ring_per_warp);
@@ -1668,8 +1699,8 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, i
   } else if (longer) {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
-    return launch_persistent(paths_2d<P, T, CV, MULTI, LongSteps2D<T, CV>::value>, a, num_sms, st,
-                             blocks, ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid,
+    return launch_persistent(long_kernel_2d<P, T, CV, MULTI>(), a, num_sms, st, blocks,
+                             ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid,
                              &attr, per_sm);
   } else {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
@@ -1687,7 +1718,7 @@ static cudaError_t occupancy_one(int threads, int* occ) {
   if constexpr (P::kDim == 3)
     kern = paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>;
   else
-    kern = paths_2d<P, T, CV, MULTI, LongSteps2D<T, CV>::value>;
+    kern = long_kernel_2d<P, T, CV, MULTI>();
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       occ, kern, threads, (size_t)(threads / 32) * ExitRing<T, P::kDim>::kBytes);
 }
