@@ -47,19 +47,19 @@ TARGET_RMSE = 1e-3
 # Box-Muller, coefficients, updates, exit test, and for the control variate
 # the cell record, bilinear gradient and xi update), as executed: ncu's
 # smsp__thread_inst_executed.sum over the path-steps of the full-size launches
-# of this benchmark (a one-pass capture of the 4-steps-per-iteration kernels;
-# the planning estimates were 110 and 150).
-ALGO_INSTR = {"plain": 93.7, "cv": 126.4}
+# of this benchmark (a one-pass capture; the planning estimates were 110 and
+# 150).
+ALGO_INSTR = {"plain": 84.9, "cv": 120.0}
 # DRAM bytes (read + write) per launch of the dominant kernel (the eps = 1e-2
 # pass) from the same full-size capture; None whenever the kernel has changed
 # since that capture.
-NCU_TRAFFIC_BYTES = 1364224
+NCU_TRAFFIC_BYTES = 1266176
 # Thread-instructions per path-step of the 3D control-variate kernel over the
 # full-size cascade launch of --workload c2 (ncu smsp__thread_inst_executed.sum
 # over its path-steps, a one-pass capture; the planning estimate was 190), for
 # the short (4 steps per iteration) and the long (8) iteration the autotuner
 # may pick.
-INSTR_3D = {"short": 222.7, "long": 217.0}
+INSTR_3D = {"short": 212.7, "long": 205.9}
 WORKLOAD = ("2D CFG0 (b=(sin y/2, cos x/2), c=1+x^2+y^2, u=e^{x+y}cos(x-y)), 2x2 subdomains, "
             "256 interfacial nodes x 1e5 paths, dt=1e-4, Gobet-Menozzi; plain + control "
             "variate on 129^2 grids eps in {1e-1,1e-2,1e-3}")
@@ -671,9 +671,9 @@ def run_c2(args):
                          "algorithmic": f"{instr_3d} thread-instr per 3D control-variate "
                                         f"path-step ({iter_run} iteration; ncu, executed, "
                                         "full-size cascade launch)",
-                         "second_limit": "L1 data pipe: 78 % of its peak in the ncu capture of "
-                                         "the profiling case (two 256-bit cell-record gathers "
-                                         "per step), issue 75 %"}}
+                         "second_limit": "L1 data pipe: 64 wavefronts per warp step (two 256-bit "
+                                         "cell-record gathers), 0.83 of its cycles at 1.30e11 "
+                                         "path-steps/s"}}
     line["roofline"]["frac"] = (line["roofline"]["achieved"] / line["roofline"]["peak"]
                                 if instr_3d else None)
     prob.close()

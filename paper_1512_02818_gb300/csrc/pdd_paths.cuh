@@ -666,7 +666,8 @@ __device__ __forceinline__ int nth_set_bit(unsigned m, int q) {
 // with all of a chip's warps in it, the issue slots, most of which go to the
 // two chains' few lanes.  256 nodes x 1,387 paths at h = 1e-4: 2.95 -> 2.24 ms
 // plain, 4.79 -> 2.96 ms with the control variate; 10 paths per node in 3D,
-// 2.67 -> 1.40 ms.
+// 2.67 -> 1.40 ms (with fewer warps, and spread, 1.74, 2.65 and 0.46: see
+// target_warps and spread_batch).
 template <class T, int D>
 struct Drain {
   static constexpr int kMaxRun = D == 2 ? PDD_DRAIN_RUN_2D : PDD_DRAIN_RUN_3D;
