@@ -90,6 +90,7 @@ struct pdd_ctx {
   int claim = 0;  // paths per lane per cursor claim, 0 = automatic (pdd_ctx_set_claim)
   cudaGraphExec_t gexec = nullptr;  // cached graph of the last PDD_FLAG_GRAPH call
   uint64_t gkey = 0;
+  unsigned long long gend = 0;  // cursor_end of the graph's launch
   int64_t graph_captures = 0;
   // pdd_ctx_abort: copies into the workspace header on a stream of its own
   // (created at the first abort), ordered before the next call's header reset
@@ -501,11 +502,11 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   // The launch sequence: clear the header and records, run every path, finalise
   // every level.  With PDD_FLAG_GRAPH it is captured once into a CUDA graph and
   // replayed while the arguments stay the same.
+  LaunchInfo info{};
   auto enqueue = [&](cudaStream_t st) -> cudaError_t {
     cudaError_t e = cudaMemsetAsync(ws, 0, off_acc + copies * rec_bytes, st);
     if (e != cudaSuccess) return e;
-    int blocks = 0;
-    e = launch_paths(p->desc.kind, p->desc.precision, cv, pa, c->num_sms, st, &blocks);
+    e = launch_paths(p->desc.kind, p->desc.precision, cv, pa, c->num_sms, st, &info);
     if (e == cudaSuccess && copies > 1)
       e = launch_merge_records(acc, (unsigned)total_nodes, copies, pa.copy_words, st);
     if (e != cudaSuccess) return e;
@@ -565,8 +566,10 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
         return cuda_fail(e, "cudaGraphInstantiate");
       }
       c->gkey = key;
+      c->gend = info.cursor_end;
       c->graph_captures += 1;
     }
+    info.cursor_end = c->gend;
     wait_abort(c);
     if (c->timing) PDD_CUDA(cudaEventRecord(ev0, c->stream), "cudaEventRecord");
     PDD_CUDA(cudaGraphLaunch(c->gexec, c->stream), "cudaGraphLaunch");
@@ -582,8 +585,7 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
       PDD_CUDA(cudaMemsetAsync(ws, 0, clear, c->stream), "cudaMemsetAsync");
     }
     if (c->timing) PDD_CUDA(cudaEventRecord(ev0, c->stream), "cudaEventRecord");
-    int blocks = 0;
-    PDD_CUDA(launch_paths(p->desc.kind, p->desc.precision, cv, pa, c->num_sms, c->stream, &blocks),
+    PDD_CUDA(launch_paths(p->desc.kind, p->desc.precision, cv, pa, c->num_sms, c->stream, &info),
              "path kernel launch");
     if (c->timing) PDD_CUDA(cudaEventRecord(ev1, c->stream), "cudaEventRecord");
     if (copies > 1)
@@ -630,8 +632,9 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   memcpy(&h, host_hdr, sizeof(h));
   if (h.aborted) return aborted_status(who);
   if (h.err != 0u) return error_word_status(h.err, who);
-  if (h.cursor < pa.total) {
-    set_error("%s: internal error, %llu of %llu paths scheduled", who, h.cursor, pa.total);
+  if (h.cursor < info.cursor_end) {
+    set_error("%s: internal error, launch of %llu paths incomplete (cursor %llu of %llu)", who,
+              pa.total, h.cursor, info.cursor_end);
     return PDD_ERR_CUDA;
   }
   if (h.trunc_total > 0) {
@@ -685,7 +688,7 @@ int pdd_ctx_create(int device, void* cuda_stream, size_t mem_budget, pdd_ctx** o
     return cuda_fail(ea, "pdd_ctx_create: abort resources");
   }
   c->pinned = (char*)c->abort_src + 256;
-  c->abort_src[0] = 1ull << 62;  // past the index space of any launch (< 2^62 paths)
+  c->abort_src[0] = kAborted;  // past the index space of any launch (< 2^62 paths)
   c->abort_src[1] = 1ull;        // low word: the header's `aborted`
   if (cuda_stream) {
     c->stream = (cudaStream_t)cuda_stream;
@@ -1063,8 +1066,8 @@ int pdd_accumulate(pdd_problem* p, const pdd_estimate_args* a, uint64_t path_off
   pa.total = sg.total;
   wait_abort(c);
   PDD_CUDA(cudaMemsetAsync(hdr, 0, 256, c->stream), "cudaMemsetAsync");
-  int blocks = 0;
-  PDD_CUDA(launch_paths(p->desc.kind, p->desc.precision, lp.cv, pa, c->num_sms, c->stream, &blocks),
+  LaunchInfo info{};
+  PDD_CUDA(launch_paths(p->desc.kind, p->desc.precision, lp.cv, pa, c->num_sms, c->stream, &info),
            "path kernel launch");
   c->launches += 1;
   if (a->flags & PDD_FLAG_ASYNC) return PDD_OK;
@@ -1204,10 +1207,10 @@ static int coupled_launch(pdd_problem* p, const pdd_estimate_args* a, const Leve
   }
   wait_abort(c);
   PDD_CUDA(cudaMemsetAsync(hdr, 0, 256, c->stream), "cudaMemsetAsync");
-  int blocks = 0;
+  LaunchInfo info{};
   char what[96];
   snprintf(what, sizeof(what), "%s: coupled kernel launch", who);
-  PDD_CUDA(launch_coupled(p->desc.kind, lp.cv, pa, c->num_sms, c->stream, &blocks), what);
+  PDD_CUDA(launch_coupled(p->desc.kind, lp.cv, pa, c->num_sms, c->stream, &info), what);
   c->launches += 1;
   return PDD_OK;
 }

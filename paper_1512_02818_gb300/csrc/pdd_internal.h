@@ -79,6 +79,10 @@ cudaError_t f64_tables(const F64Tables** tables);
 // a launch's cost grows with its parameters (an empty kernel and its wait on
 // GB300: 11.1 us with 24 KB, 8.6 us with 256 B; a whole call of one node x 1,000
 // paths: 66 -> 61 us).
+constexpr unsigned long long kAborted = 1ull << 62;  // cursor of an aborted launch: past any path
+// What a warp of a spread launch adds to the cursor: past the last path of any
+// such launch, and a count of the warps in the upper half.
+constexpr unsigned long long kSpreadClaim = 1ull << 32;
 struct PathHead {
   unsigned long long total;    // sum of the segments' totals
   unsigned long long* cursor;  // flat path cursor, zeroed before the launch
@@ -102,6 +106,11 @@ struct PathHead {
   // (copy_mask = copies - 1), copy_words words apart; 0: the records themselves.
   unsigned copy_mask;
   unsigned long long copy_words;
+};
+// What a launcher chose.
+struct LaunchInfo {
+  int blocks;
+  unsigned long long cursor_end;  // the cursor reaches this once every path has been handed out
 };
 template <int N>
 struct PathArgsN : PathHead {
@@ -170,13 +179,13 @@ int ctx_claim(pdd_ctx* c);      // the context's paths-per-lane claim (0: automa
 pdd_ctx* problem_ctx(pdd_problem* p);
 
 cudaError_t launch_paths(int kind, int precision, int cv, const PathArgs& a, int num_sms,
-                         cudaStream_t st, int* blocks);
+                         cudaStream_t st, LaunchInfo* info);
 // Resident blocks per SM of the path kernel of (kind, precision, cv, multi) at
 // `threads` threads per block.
 cudaError_t occupancy_paths(int kind, int precision, int cv, bool multi, int threads, int* occ);
 // Coupled fine (seg[0]) / coarse (seg[1]) pairs, FP32 paths (2D and 3D problems).
 cudaError_t launch_coupled(int kind, int cv, const PathArgs& a, int num_sms, cudaStream_t st,
-                           int* blocks);
+                           LaunchInfo* info);
 cudaError_t launch_finalize(const unsigned long long* acc, uint32_t n_nodes, double kappa,
                             const StatPtrs& out, cudaStream_t st);
 // One launch for the records of up to kMaxSegments levels (empty ones skipped;

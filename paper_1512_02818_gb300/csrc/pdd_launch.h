@@ -17,9 +17,9 @@ struct PaperEx;
 template <class P>
 struct PathLaunch {
   static cudaError_t paths(int precision, int cv, bool multi, const PathArgs& a, int num_sms,
-                           cudaStream_t st, int* blocks);
+                           cudaStream_t st, LaunchInfo* info);
   static cudaError_t occupancy(int precision, int cv, bool multi, int threads, int* occ);
-  static cudaError_t coupled(int cv, const PathArgs& a, int num_sms, cudaStream_t st, int* blocks);
+  static cudaError_t coupled(int cv, const PathArgs& a, int num_sms, cudaStream_t st, LaunchInfo* info);
 };
 
 }  // namespace pdd

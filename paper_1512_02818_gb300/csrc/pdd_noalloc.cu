@@ -191,8 +191,8 @@ extern "C" int pdd_estimate_nodes_noalloc(pdd_problem* problem, const pdd_estima
   sg.seed_hi = (uint32_t)(a->seed >> 32);
   sg.grid_n = grid_n;
   sg.max_steps = (int)max_steps;
-  int blocks = 0;
-  e = launch_paths(pv.kind, pv.precision, cv, pa, pv.num_sms, pv.stream, &blocks);
+  LaunchInfo info{};
+  e = launch_paths(pv.kind, pv.precision, cv, pa, pv.num_sms, pv.stream, &info);
   if (e != cudaSuccess) return fail(e, "path kernel launch");
   StatPtrs sp{};
   sp.mean_phi = out->mean_phi;
@@ -218,9 +218,10 @@ extern "C" int pdd_estimate_nodes_noalloc(pdd_problem* problem, const pdd_estima
   if (e == cudaSuccess) e = cudaStreamSynchronize(pv.stream);
   if (e != cudaSuccess) return fail(e, "cudaStreamSynchronize");
   if (h.err != 0u) return error_word_status(h.err, "pdd_estimate_nodes_noalloc");
-  if (h.cursor < pa.total) {
-    set_error("pdd_estimate_nodes_noalloc: internal error, %llu of %llu paths scheduled",
-              h.cursor, pa.total);
+  if (h.cursor < info.cursor_end) {
+    set_error("pdd_estimate_nodes_noalloc: internal error, launch of %llu paths incomplete (cursor "
+              "%llu of %llu)",
+              pa.total, h.cursor, info.cursor_end);
     return PDD_ERR_CUDA;
   }
   if (h.trunc_total > 0) {

@@ -179,7 +179,7 @@ cudaError_t launch_stage_requests(const StageRequest* req, int n, cudaStream_t s
 // Dispatch by problem.
 // ---------------------------------------------------------------------------
 cudaError_t launch_paths(int kind, int precision, int cv, const PathArgs& args, int num_sms,
-                         cudaStream_t st, int* blocks) {
+                         cudaStream_t st, LaunchInfo* info) {
   PathArgs a = args;
   if (precision == 1) {
     cudaError_t e = f64_tables(&a.f64);
@@ -189,11 +189,11 @@ cudaError_t launch_paths(int kind, int precision, int cv, const PathArgs& args, 
   // the single-segment build follows the Euler Y rule only (see euler_step)
   const bool multi = a.n_segs > 1 || a.y_exp != 0;
   switch (kind) {
-    case 0: return PathLaunch<Cfg0>::paths(precision, cv, multi, a, num_sms, st, blocks);
-    case 1: return PathLaunch<Aniso>::paths(precision, cv, multi, a, num_sms, st, blocks);
-    case 2: return PathLaunch<Cube3>::paths(precision, cv, multi, a, num_sms, st, blocks);
-    case 4: return PathLaunch<PaperEx>::paths(precision, cv, multi, a, num_sms, st, blocks);
-    default: return PathLaunch<Harmonic>::paths(precision, cv, multi, a, num_sms, st, blocks);
+    case 0: return PathLaunch<Cfg0>::paths(precision, cv, multi, a, num_sms, st, info);
+    case 1: return PathLaunch<Aniso>::paths(precision, cv, multi, a, num_sms, st, info);
+    case 2: return PathLaunch<Cube3>::paths(precision, cv, multi, a, num_sms, st, info);
+    case 4: return PathLaunch<PaperEx>::paths(precision, cv, multi, a, num_sms, st, info);
+    default: return PathLaunch<Harmonic>::paths(precision, cv, multi, a, num_sms, st, info);
   }
 }
 
@@ -208,13 +208,13 @@ cudaError_t occupancy_paths(int kind, int precision, int cv, bool multi, int thr
 }
 
 cudaError_t launch_coupled(int kind, int cv, const PathArgs& a, int num_sms, cudaStream_t st,
-                           int* blocks) {
+                           LaunchInfo* info) {
   switch (kind) {
-    case 0: return PathLaunch<Cfg0>::coupled(cv, a, num_sms, st, blocks);
-    case 1: return PathLaunch<Aniso>::coupled(cv, a, num_sms, st, blocks);
-    case 2: return PathLaunch<Cube3>::coupled(cv, a, num_sms, st, blocks);
-    case 3: return PathLaunch<Harmonic>::coupled(cv, a, num_sms, st, blocks);
-    case 4: return PathLaunch<PaperEx>::coupled(cv, a, num_sms, st, blocks);
+    case 0: return PathLaunch<Cfg0>::coupled(cv, a, num_sms, st, info);
+    case 1: return PathLaunch<Aniso>::coupled(cv, a, num_sms, st, info);
+    case 2: return PathLaunch<Cube3>::coupled(cv, a, num_sms, st, info);
+    case 3: return PathLaunch<Harmonic>::coupled(cv, a, num_sms, st, info);
+    case 4: return PathLaunch<PaperEx>::coupled(cv, a, num_sms, st, info);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -468,7 +468,8 @@ __device__ __forceinline__ bool refill(const A& a, PathState<T>& s, LaneSeg<T>& 
 }
 
 // Spread launches (see spread_batch): every warp has a batch of its own, and
-// the cursor is past the last path when the warp asks it for more.
+// the cursor is past the last path when the warp asks it for more (and counts
+// the warps).  A warp that finds the launch aborted takes no batch.
 template <bool MULTI, class A>
 __device__ __forceinline__ void spread_claim(const A& a, unsigned long long& bnext,
                                              unsigned long long& bend, uint32_t& bseg) {
@@ -476,10 +477,12 @@ __device__ __forceinline__ void spread_claim(const A& a, unsigned long long& bne
   // (the shuffle tells the compiler that the batch is the warp's: without it
   // the kernels take 20 registers more)
   const unsigned warp = __shfl_sync(kFull, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, 0);
-  bnext = min(warp * a.warp_batch, a.total);
-  bend = min(bnext + a.warp_batch, a.total);
+  unsigned long long before = 0;
+  if ((threadIdx.x & 31u) == 0u) before = atomicAdd(a.cursor, kSpreadClaim);
+  const unsigned long long end = __any_sync(kFull, before >= kAborted) ? 0ull : a.total;
+  bnext = min(warp * a.warp_batch, end);
+  bend = min(bnext + a.warp_batch, end);
   if (MULTI) bseg = segment_of(a, bnext);
-  if ((threadIdx.x & 31u) == 0u) atomicAdd(a.cursor, a.total);
 }
 
 // Per-warp exit ring.  A lane whose path has ended parks the path's final
@@ -1587,7 +1590,7 @@ static int target_warps(const PathArgs& a, int num_sms) {
 // without the cache.
 template <int N>
 static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs& a, int num_sms,
-                                     cudaStream_t st, int* blocks, size_t ring_per_warp, int spread,
+                                     cudaStream_t st, LaunchInfo* info, size_t ring_per_warp, int spread,
                                      int warps, int refill, bool l1, std::atomic<int>* attr_set,
                                      std::atomic<int>* occ_cache) {
   if (a.n_segs > N) return cudaErrorInvalidValue;
@@ -1670,14 +1673,15 @@ static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs&
   if (nb > blocks_needed) nb = blocks_needed;
   if (nb < 1) nb = 1;
   b.one_claim = spread > 0 && nb == blocks_needed;  // the warps' single batches cover every path
-  *blocks = (int)nb;
+  info->blocks = (int)nb;
+  info->cursor_end = b.one_claim ? (nb * (threads / 32)) * kSpreadClaim : a.total;
   kern<<<(unsigned)nb, (unsigned)threads, smem, st>>>(b);
   return cudaGetLastError();
 }
 
 
 template <class P, class T, int CV, bool MULTI>
-static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, int* blocks) {
+static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, LaunchInfo* info) {
   // FP64 paths: the step dominates, they always take the short iteration
   const bool longer = sizeof(T) == 4 && (a.iter_mode == PDD_ITER_LONG ||
                                          (a.iter_mode == PDD_ITER_AUTO && long_iterations(a)));
@@ -1689,24 +1693,24 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, i
       static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
       static std::atomic<int> attr{0};
       return launch_persistent(paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>, a, num_sms, st,
-                               blocks, ExitRing<T, 3>::kBytes, spread, warps, refill,
+                               info, ExitRing<T, 3>::kBytes, spread, warps, refill,
                                CV == kCvGrid, &attr, per_sm);
     }
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
-    return launch_persistent(paths_3d<P, T, CV, MULTI, 4>, a, num_sms, st, blocks,
+    return launch_persistent(paths_3d<P, T, CV, MULTI, 4>, a, num_sms, st, info,
                              ExitRing<T, 3>::kBytes, spread, warps, refill, CV == kCvGrid, &attr,
                              per_sm);
   } else if (longer) {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
-    return launch_persistent(long_kernel_2d<P, T, CV, MULTI>(), a, num_sms, st, blocks,
+    return launch_persistent(long_kernel_2d<P, T, CV, MULTI>(), a, num_sms, st, info,
                              ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid,
                              &attr, per_sm);
   } else {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
     static std::atomic<int> attr{0};
-    return launch_persistent(paths_2d<P, T, CV, MULTI, 2>, a, num_sms, st, blocks,
+    return launch_persistent(paths_2d<P, T, CV, MULTI, 2>, a, num_sms, st, info,
                              ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid, &attr,
                              per_sm);
   }
@@ -1734,31 +1738,31 @@ static cudaError_t occupancy_cv(int cv, int threads, int* occ) {
 }
 
 template <class P, class T, bool MULTI>
-static cudaError_t launch_cv(int cv, const PathArgs& a, int sms, cudaStream_t st, int* blocks) {
+static cudaError_t launch_cv(int cv, const PathArgs& a, int sms, cudaStream_t st, LaunchInfo* info) {
   switch (cv) {
-    case kCvNone: return launch_one<P, T, kCvNone, MULTI>(a, sms, st, blocks);
-    case kCvGrid: return launch_one<P, T, kCvGrid, MULTI>(a, sms, st, blocks);
-    default: return launch_one<P, T, kCvExact, MULTI>(a, sms, st, blocks);
+    case kCvNone: return launch_one<P, T, kCvNone, MULTI>(a, sms, st, info);
+    case kCvGrid: return launch_one<P, T, kCvGrid, MULTI>(a, sms, st, info);
+    default: return launch_one<P, T, kCvExact, MULTI>(a, sms, st, info);
   }
 }
 
 template <class P, class T, int CV, int D>
 static cudaError_t launch_coupled_one(const PathArgs& a, int num_sms, cudaStream_t st,
-                                      int* blocks) {
+                                      LaunchInfo* info) {
   static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
   static std::atomic<int> attr{0};
-  return launch_persistent(paths_coupled<P, T, CV, D>, a, num_sms, st, blocks,
+  return launch_persistent(paths_coupled<P, T, CV, D>, a, num_sms, st, info,
                            PairRing<T>::kBytes, spread_batch<T>(a, num_sms), 0, 1, true,
                            &attr, per_sm);
 }
 
 template <class P, class T, int D>
 static cudaError_t launch_coupled_cv(int cv, const PathArgs& a, int sms, cudaStream_t st,
-                                     int* blocks) {
+                                     LaunchInfo* info) {
   switch (cv) {
-    case kCvNone: return launch_coupled_one<P, T, kCvNone, D>(a, sms, st, blocks);
-    case kCvGrid: return launch_coupled_one<P, T, kCvGrid, D>(a, sms, st, blocks);
-    default: return launch_coupled_one<P, T, kCvExact, D>(a, sms, st, blocks);
+    case kCvNone: return launch_coupled_one<P, T, kCvNone, D>(a, sms, st, info);
+    case kCvGrid: return launch_coupled_one<P, T, kCvGrid, D>(a, sms, st, info);
+    default: return launch_coupled_one<P, T, kCvExact, D>(a, sms, st, info);
   }
 }
 
@@ -1768,13 +1772,13 @@ static cudaError_t launch_coupled_cv(int cv, const PathArgs& a, int sms, cudaStr
 // stalled on the texture/MIO queues), so the latter is not instantiated.
 template <class P>
 cudaError_t PathLaunch<P>::paths(int precision, int cv, bool multi, const PathArgs& a, int num_sms,
-                                 cudaStream_t st, int* blocks) {
+                                 cudaStream_t st, LaunchInfo* info) {
   constexpr bool kTable = P::kDim == 3;
   if (precision == 1)
-    return multi ? launch_cv<P, double, true>(cv, a, num_sms, st, blocks)
-                 : launch_cv<P, double, kTable>(cv, a, num_sms, st, blocks);
-  return multi ? launch_cv<P, float, true>(cv, a, num_sms, st, blocks)
-               : launch_cv<P, float, kTable>(cv, a, num_sms, st, blocks);
+    return multi ? launch_cv<P, double, true>(cv, a, num_sms, st, info)
+                 : launch_cv<P, double, kTable>(cv, a, num_sms, st, info);
+  return multi ? launch_cv<P, float, true>(cv, a, num_sms, st, info)
+               : launch_cv<P, float, kTable>(cv, a, num_sms, st, info);
 }
 
 template <class P>
@@ -1789,8 +1793,8 @@ cudaError_t PathLaunch<P>::occupancy(int precision, int cv, bool multi, int thre
 
 template <class P>
 cudaError_t PathLaunch<P>::coupled(int cv, const PathArgs& a, int num_sms, cudaStream_t st,
-                                   int* blocks) {
-  return launch_coupled_cv<P, float, P::kDim>(cv, a, num_sms, st, blocks);
+                                   LaunchInfo* info) {
+  return launch_coupled_cv<P, float, P::kDim>(cv, a, num_sms, st, info);
 }
 
 }  // namespace pdd

@@ -323,8 +323,8 @@ int run_pilot(pdd_server* s, const Request& r, double* steps) {
   sg.key1 = 0xFFFFFFF0u;
   sg.max_steps = r.max_steps;
   pa.total = sg.total;
-  int blocks = 0;
-  if (e == cudaSuccess) e = launch_paths(r.pv.kind, r.pv.precision, 0, pa, s->num_sms, st, &blocks);
+  LaunchInfo info{};
+  if (e == cudaSuccess) e = launch_paths(r.pv.kind, r.pv.precision, 0, pa, s->num_sms, st, &info);
   StatPtrs sp{};
   sp.mean_steps = mean_steps;
   if (e == cudaSuccess) e = launch_finalize(acc, (uint32_t)n, 1.0, sp, st);
@@ -534,8 +534,8 @@ bool issue_launch(pdd_server* s) {
   }
   pa.n_segs = ns;
   pa.total = begin;
-  int blocks = 0;
-  if (e == cudaSuccess) e = launch_paths(pv.kind, pv.precision, cv, pa, s->num_sms, st, &blocks);
+  LaunchInfo info{};
+  if (e == cudaSuccess) e = launch_paths(pv.kind, pv.precision, cv, pa, s->num_sms, st, &info);
   // the launch's header (error word, executed path-steps), read when its event
   // has completed; the slot is not reused before then (the next launch on this
   // stream is issued after this one retires)
