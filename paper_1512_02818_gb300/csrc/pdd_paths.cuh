@@ -1584,15 +1584,14 @@ static int target_warps(const PathArgs& a, int num_sms) {
 // when the launch's nodes fit it and `ring_per_warp` bytes of exit ring per
 // warp.  `spread` > 0: that many paths per warp (see spread_batch), in blocks
 // of 128 threads so that the warps cover the SMs evenly.  `warps`: see
-// target_warps; `refill`: see refill_min; `l1`: see use_cache.  `attr_set` /
-// `occ_cache` are the kernel's own (static) state: the
-// dynamic shared memory limit set so far and the occupancy per block size
-// without the cache.
+// target_warps; `refill`: see refill_min; `l1`: see use_cache.  `occ_cache` is
+// the kernel's own (static) state: its registers and the occupancy per block
+// size without the cache, the same on every device that runs this code (it is
+// compiled for one architecture).
 template <int N>
 static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs& a, int num_sms,
                                      cudaStream_t st, LaunchInfo* info, size_t ring_per_warp, int spread,
-                                     int warps, int refill, bool l1, std::atomic<int>* attr_set,
-                                     std::atomic<int>* occ_cache) {
+                                     int warps, int refill, bool l1, std::atomic<int>* occ_cache) {
   if (a.n_segs > N) return cudaErrorInvalidValue;
   PathArgsN<N> b;
   (PathHead&)b = a;
@@ -1642,11 +1641,11 @@ static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs&
     threads = kBlockThreads;
   }
   const size_t smem = cache + (size_t)(threads / 32) * ring_per_warp;
-  if (smem > 48u * 1024u && (int)smem > attr_set->load(std::memory_order_relaxed)) {
+  if (smem > 48u * 1024u) {
+    // for the current device alone, so at every such launch (0.2 us)
     const int lim = (int)(cache_bytes(kCacheMaxNodes) + (kMaxBlockThreads / 32) * ring_per_warp);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     if (e != cudaSuccess) return e;
-    attr_set->store(lim, std::memory_order_relaxed);
   }
   int occ = 0;
   const int known = occ_cache[threads / 32].load(std::memory_order_relaxed);
@@ -1691,28 +1690,22 @@ static cudaError_t launch_one(const PathArgs& a, int num_sms, cudaStream_t st, L
   if constexpr (P::kDim == 3) {
     if (longer) {
       static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
-      static std::atomic<int> attr{0};
       return launch_persistent(paths_3d<P, T, CV, MULTI, sizeof(T) == 4 ? 8 : 4>, a, num_sms, st,
                                info, ExitRing<T, 3>::kBytes, spread, warps, refill,
-                               CV == kCvGrid, &attr, per_sm);
+                               CV == kCvGrid, per_sm);
     }
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
-    static std::atomic<int> attr{0};
     return launch_persistent(paths_3d<P, T, CV, MULTI, 4>, a, num_sms, st, info,
-                             ExitRing<T, 3>::kBytes, spread, warps, refill, CV == kCvGrid, &attr,
-                             per_sm);
+                             ExitRing<T, 3>::kBytes, spread, warps, refill, CV == kCvGrid, per_sm);
   } else if (longer) {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
-    static std::atomic<int> attr{0};
     return launch_persistent(long_kernel_2d<P, T, CV, MULTI>(), a, num_sms, st, info,
                              ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid,
-                             &attr, per_sm);
+                             per_sm);
   } else {
     static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
-    static std::atomic<int> attr{0};
     return launch_persistent(paths_2d<P, T, CV, MULTI, 2>, a, num_sms, st, info,
-                             ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid, &attr,
-                             per_sm);
+                             ExitRing<T, 2>::kBytes, spread, warps, refill, CV == kCvGrid, per_sm);
   }
 }
 
@@ -1750,10 +1743,9 @@ template <class P, class T, int CV, int D>
 static cudaError_t launch_coupled_one(const PathArgs& a, int num_sms, cudaStream_t st,
                                       LaunchInfo* info) {
   static std::atomic<int> per_sm[kMaxBlockThreads / 32 + 1];
-  static std::atomic<int> attr{0};
   return launch_persistent(paths_coupled<P, T, CV, D>, a, num_sms, st, info,
                            PairRing<T>::kBytes, spread_batch<T>(a, num_sms), 0, 1, true,
-                           &attr, per_sm);
+                           per_sm);
 }
 
 template <class P, class T, int D>
