@@ -748,7 +748,9 @@ __device__ __forceinline__ void batch_normals(const BatchLane& b, uint32_t blk, 
   }
 }
 
-// Increment of step i; PAIR: the sum of those of steps 2i and 2i + 1.
+// Increment of step i; PAIR: the sum of those of steps 2i and 2i + 1, rounded by
+// itself here and in the ordinary iterations (there each is a product in the
+// same function, with which a plain sum may be fused).
 template <class T, int D, bool PAIR>
 __device__ __forceinline__ void batch_noise(const T* nrm, int i, const BatchLane& b, T* dW) {
   get_vec<T, D>(nrm, PAIR ? 2 * i : i, b.q, b.A, dW);
@@ -756,7 +758,7 @@ __device__ __forceinline__ void batch_noise(const T* nrm, int i, const BatchLane
     T e[3];
     get_vec<T, D>(nrm, 2 * i + 1, b.q, b.A, e);
 #pragma unroll
-    for (int d = 0; d < D; ++d) dW[d] = dW[d] + e[d];
+    for (int d = 0; d < D; ++d) dW[d] = add_rn(dW[d], e[d]);
   }
 }
 
@@ -1388,8 +1390,8 @@ __global__ void __launch_bounds__(kMaxBlockThreads, 1) paths_coupled(
               p.ac = false;
             } else {
               const int o = 2 * D * q;  // fine steps 2q and 2q+1 of this iteration
-              T d[3] = {n[o] + n[o + D], n[o + 1] + n[o + D + 1],
-                        D == 3 ? n[o + 2] + n[o + D + 2] : T(0)};
+              T d[3] = {add_rn(n[o], n[o + D]), add_rn(n[o + 1], n[o + D + 1]),
+                        D == 3 ? add_rn(n[o + 2], n[o + D + 2]) : T(0)};
               euler_step<P, T, D, CV, false, true>(a, c, lc, d);
               if (c.k >= lc.max_steps) {
                 p.ac = false;
