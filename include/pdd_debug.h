@@ -1,14 +1,17 @@
 /*
  * pdd_debug.h -- test hooks of libpdd.so.  They expose the device random
  * number stages on their own so that tests can compare them with the oracle
- * and with cuRAND's Philox4_32_10 generator; they are not part of the
- * estimation path.  All pointers are device pointers; calls are synchronous;
- * return a pdd_status (see pdd.h).
+ * and with cuRAND's Philox4_32_10 generator, and tell which route a launch
+ * took; they are not part of the estimation path.  Pointers are device pointers
+ * where nothing else is said; calls are synchronous; return a pdd_status (see
+ * pdd.h).
  */
 #ifndef PDD_DEBUG_H
 #define PDD_DEBUG_H
 
 #include <stdint.h>
+
+#include "pdd.h"
 
 #ifdef __cplusplus
 extern "C" {
@@ -48,6 +51,14 @@ int pdd_debug_issue_rate(int kind, int iters, double* ops_per_s, double* ms);
    release build, whose checks compile to nothing.  Synchronous; allocates
    and frees one device word.                                                */
 int pdd_debug_bounds_selftest(uint32_t* bits);
+
+/* The shape of the context's last path launch (estimates, accumulations and
+   coupled calls; no counterpart in the paper): blocks, threads per block, node
+   records kept in every block's shared memory (0: none), and paths per warp of
+   a launch whose warps take one batch each (0: the others).  Zeros before the
+   first launch; any output may be NULL.                                      */
+int pdd_debug_last_launch(pdd_ctx* ctx, int* blocks, int* block_threads, int* cached_records,
+                          int* paths_per_warp);
 
 #ifdef __cplusplus
 }

@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/pdd.h"
+#include "../../include/pdd_debug.h"
 #include "pdd_device.cuh"
 #include "pdd_internal.h"
 
@@ -90,7 +91,8 @@ struct pdd_ctx {
   int claim = 0;  // paths per lane per cursor claim, 0 = automatic (pdd_ctx_set_claim)
   cudaGraphExec_t gexec = nullptr;  // cached graph of the last PDD_FLAG_GRAPH call
   uint64_t gkey = 0;
-  unsigned long long gend = 0;  // cursor_end of the graph's launch
+  LaunchInfo glaunch{};  // of the cached graph's path launch
+  LaunchInfo last{};     // of the last path launch (mu)
   int64_t graph_captures = 0;
   // pdd_ctx_abort: copies into the workspace header on a stream of its own
   // (created at the first abort), ordered before the next call's header reset
@@ -502,7 +504,7 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   // The launch sequence: clear the header and records, run every path, finalise
   // every level.  With PDD_FLAG_GRAPH it is captured once into a CUDA graph and
   // replayed while the arguments stay the same.
-  LaunchInfo info{};
+  LaunchInfo& info = c->last;
   auto enqueue = [&](cudaStream_t st) -> cudaError_t {
     cudaError_t e = cudaMemsetAsync(ws, 0, off_acc + copies * rec_bytes, st);
     if (e != cudaSuccess) return e;
@@ -566,10 +568,10 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
         return cuda_fail(e, "cudaGraphInstantiate");
       }
       c->gkey = key;
-      c->gend = info.cursor_end;
+      c->glaunch = info;
       c->graph_captures += 1;
     }
-    info.cursor_end = c->gend;
+    info = c->glaunch;
     wait_abort(c);
     if (c->timing) PDD_CUDA(cudaEventRecord(ev0, c->stream), "cudaEventRecord");
     PDD_CUDA(cudaGraphLaunch(c->gexec, c->stream), "cudaGraphLaunch");
@@ -1066,8 +1068,7 @@ int pdd_accumulate(pdd_problem* p, const pdd_estimate_args* a, uint64_t path_off
   pa.total = sg.total;
   wait_abort(c);
   PDD_CUDA(cudaMemsetAsync(hdr, 0, 256, c->stream), "cudaMemsetAsync");
-  LaunchInfo info{};
-  PDD_CUDA(launch_paths(p->desc.kind, p->desc.precision, lp.cv, pa, c->num_sms, c->stream, &info),
+  PDD_CUDA(launch_paths(p->desc.kind, p->desc.precision, lp.cv, pa, c->num_sms, c->stream, &c->last),
            "path kernel launch");
   c->launches += 1;
   if (a->flags & PDD_FLAG_ASYNC) return PDD_OK;
@@ -1207,10 +1208,9 @@ static int coupled_launch(pdd_problem* p, const pdd_estimate_args* a, const Leve
   }
   wait_abort(c);
   PDD_CUDA(cudaMemsetAsync(hdr, 0, 256, c->stream), "cudaMemsetAsync");
-  LaunchInfo info{};
   char what[96];
   snprintf(what, sizeof(what), "%s: coupled kernel launch", who);
-  PDD_CUDA(launch_coupled(p->desc.kind, lp.cv, pa, c->num_sms, c->stream, &info), what);
+  PDD_CUDA(launch_coupled(p->desc.kind, lp.cv, pa, c->num_sms, c->stream, &c->last), what);
   c->launches += 1;
   return PDD_OK;
 }
@@ -1380,6 +1380,20 @@ int pdd_ctx_get_launch(pdd_ctx* c, int* block_threads, int* max_blocks, int* ite
   if (block_threads) *block_threads = c->block_threads;
   if (max_blocks) *max_blocks = c->max_blocks;
   if (iteration) *iteration = c->iter_mode;
+  return PDD_OK;
+}
+
+int pdd_debug_last_launch(pdd_ctx* c, int* blocks, int* block_threads, int* cached_records,
+                          int* paths_per_warp) {
+  if (!c) {
+    set_error("pdd_debug_last_launch: NULL context");
+    return PDD_ERR_INVALID;
+  }
+  std::lock_guard<std::mutex> lk(c->mu);
+  if (blocks) *blocks = c->last.blocks;
+  if (block_threads) *block_threads = c->last.threads;
+  if (cached_records) *cached_records = (int)c->last.cached_records;
+  if (paths_per_warp) *paths_per_warp = c->last.paths_per_warp;
   return PDD_OK;
 }
 

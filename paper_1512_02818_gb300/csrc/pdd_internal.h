@@ -109,7 +109,9 @@ struct PathHead {
 };
 // What a launcher chose.
 struct LaunchInfo {
-  int blocks;
+  int blocks, threads;
+  uint32_t cached_records;        // records kept in every block's shared memory (0: none)
+  int paths_per_warp;             // spread launches: the batch of every warp (0: the others)
   unsigned long long cursor_end;  // the cursor reaches this once every path has been handed out
 };
 template <int N>

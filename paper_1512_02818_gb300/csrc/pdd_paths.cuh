@@ -1675,6 +1675,9 @@ static cudaError_t launch_persistent(void (*kern)(PathArgsN<N>), const PathArgs&
   if (nb < 1) nb = 1;
   b.one_claim = spread > 0 && nb == blocks_needed;  // the warps' single batches cover every path
   info->blocks = (int)nb;
+  info->threads = threads;
+  info->cached_records = b.cache_nodes;
+  info->paths_per_warp = b.one_claim ? spread : 0;
   info->cursor_end = b.one_claim ? (nb * (threads / 32)) * kSpreadClaim : a.total;
   kern<<<(unsigned)nb, (unsigned)threads, smem, st>>>(b);
   return cudaGetLastError();

@@ -219,6 +219,7 @@ _SIGS = [
     ("pdd_debug_normals", ctypes.c_int, [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint32,
                                          ctypes.c_uint32, ctypes.c_uint64, ctypes.c_int64,
                                          ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]),
+    ("pdd_debug_last_launch", ctypes.c_int, [ctypes.c_void_p] + 4 * [ctypes.POINTER(ctypes.c_int)]),
     ("pdd_debug_issue_rate", ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_double),
                                             ctypes.POINTER(ctypes.c_double)]),
 ]
@@ -493,6 +494,14 @@ def pdd_debug_normals(seed: int, tag: int, node: int, path: int, first: int, cou
                       precision: int, out_f32: int | None, out_f64: int | None) -> None:
     _check(lib().pdd_debug_normals(seed, tag, node, path, first, count, precision, out_f32,
                                    out_f64))
+
+
+def pdd_debug_last_launch(ctx: int) -> dict:
+    """Shape of the context's last path launch."""
+    names = ("blocks", "block_threads", "cached_records", "paths_per_warp")
+    v = [ctypes.c_int(0) for _ in names]
+    _check(lib().pdd_debug_last_launch(ctx, *[ctypes.byref(x) for x in v]))
+    return {k: x.value for k, x in zip(names, v)}
 
 
 # ---- torch conveniences ------------------------------------------------------
