@@ -31,6 +31,12 @@ int pdd_debug_philox_curand(const uint32_t* ctr, const uint32_t* key, uint32_t* 
 int pdd_debug_normals(uint64_t seed, uint32_t tag, uint32_t node, uint32_t path, uint64_t first,
                       int64_t count, int precision, float* out_f32, double* out_f64);
 
+/* The FP64 paths' elementary functions of x in [0, 2] (sin, cos, exp by table),
+   and the control grid's cell index and offset of x for n points per axis
+   (no counterpart in the paper).  Device arrays of `count` elements.         */
+int pdd_debug_f64_functions(const double* x, int64_t count, int n, double* sin_x, double* cos_x,
+                            double* exp_x, int* cell, double* frac);
+
 /* Issue-rate probe (no counterpart in the paper): thread-operations per second
    of one instruction class, run by 4 x SM-count blocks of 512 threads on the
    current device, each thread `iters` x 32 operations in 8 independent

@@ -61,6 +61,18 @@ __global__ void normals_kernel(uint64_t seed, uint32_t tag, uint32_t node, uint3
   out[j] = (i % 2 == 0) ? a : b;
 }
 
+__global__ void f64_functions_kernel(const double* x, int64_t count, int n, double* s, double* c,
+                                     double* e, int* cell, double* frac,
+                                     const pdd::F64Tables* tb) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= count) return;
+  const pdd::UnitPoint p(x[j], tb);
+  s[j] = p.sin();
+  c[j] = p.cos();
+  e[j] = p.exp();
+  cell[j] = pdd::cell_of(x[j], (double)(n - 1), n, frac[j]);
+}
+
 int finish(cudaError_t e) {
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
@@ -112,6 +124,21 @@ extern "C" int pdd_debug_normals(uint64_t seed, uint32_t tag, uint32_t node, uin
     if (e != cudaSuccess) return finish(e);
     normals_kernel<double><<<blocks, 256>>>(seed, tag, node, path, first, count, out_f64, tb);
   }
+  return finish(cudaGetLastError());
+}
+
+extern "C" int pdd_debug_f64_functions(const double* x, int64_t count, int n, double* sin_x,
+                                       double* cos_x, double* exp_x, int* cell, double* frac) {
+  if (count < 0 || n < 3 || (count > 0 && (!x || !sin_x || !cos_x || !exp_x || !cell || !frac))) {
+    pdd::set_error("pdd_debug_f64_functions: bad arguments");
+    return PDD_ERR_INVALID;
+  }
+  if (count == 0) return PDD_OK;
+  const pdd::F64Tables* tb = nullptr;
+  cudaError_t e = pdd::f64_tables(&tb);
+  if (e != cudaSuccess) return finish(e);
+  f64_functions_kernel<<<(unsigned)((count + 255) / 256), 256>>>(x, count, n, sin_x, cos_x, exp_x,
+                                                                 cell, frac, tb);
   return finish(cudaGetLastError());
 }
 

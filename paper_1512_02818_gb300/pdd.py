@@ -219,6 +219,8 @@ _SIGS = [
     ("pdd_debug_normals", ctypes.c_int, [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint32,
                                          ctypes.c_uint32, ctypes.c_uint64, ctypes.c_int64,
                                          ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]),
+    ("pdd_debug_f64_functions", ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int]
+     + 5 * [ctypes.c_void_p]),
     ("pdd_debug_last_launch", ctypes.c_int, [ctypes.c_void_p] + 4 * [ctypes.POINTER(ctypes.c_int)]),
     ("pdd_debug_issue_rate", ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_double),
                                             ctypes.POINTER(ctypes.c_double)]),
@@ -494,6 +496,12 @@ def pdd_debug_normals(seed: int, tag: int, node: int, path: int, first: int, cou
                       precision: int, out_f32: int | None, out_f64: int | None) -> None:
     _check(lib().pdd_debug_normals(seed, tag, node, path, first, count, precision, out_f32,
                                    out_f64))
+
+
+def pdd_debug_f64_functions(x_ptr: int, count: int, n: int, sin_ptr: int, cos_ptr: int,
+                            exp_ptr: int, cell_ptr: int, frac_ptr: int) -> None:
+    _check(lib().pdd_debug_f64_functions(x_ptr, count, n, sin_ptr, cos_ptr, exp_ptr, cell_ptr,
+                                         frac_ptr))
 
 
 def pdd_debug_last_launch(ctx: int) -> dict:
