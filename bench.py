@@ -403,6 +403,7 @@ def run_ours(args, rank, world, local):
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
+    launched = pdd.pdd_debug_last_launch(ctx.handle)
     ctx.set_timing(True)
     ctx.kernel_time()  # drop warm-up events
     launches0 = ctx.launch_count()
@@ -511,8 +512,8 @@ def run_ours(args, rank, world, local):
         "pass_rate_path_steps_per_s": rate,
         "clocks": clk,
         "timed_kernel_launches": n_timed,
-        "launch_shape": {"block_threads": tuned[0] or (512 if n_nodes <= 512 else 128),
-                         "max_blocks": tuned[1],
+        "launch_shape": {"block_threads": launched["block_threads"],
+                         "blocks": launched["blocks"],
                          "iteration": ["auto", "short", "long"][launch_iter],
                          "paths_per_lane_claim": launch_claim or "auto",
                          "chosen_by": "pdd_autotune on the eps=1e-2 pass" if tuned[2]
@@ -627,6 +628,7 @@ def run_c2(args):
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
+    launched = pdd.pdd_debug_last_launch(ctx.handle)
     launches0 = ctx.launch_count()
     clocks = ClockSampler(smi_id(0))
     ms = _timed_steps(torch, ctx.stream, args.steps, step, flush)
@@ -657,7 +659,7 @@ def run_c2(args):
                                    "persistent launch replayed from a CUDA graph",
                        "l2": "flushed between steps (256 MB)"},
             "nodes_per_s": len(nodes) * args.steps / (total_ms / 1e3),
-            "launch_shape": {"block_threads": tuned[0] or 128, "max_blocks": tuned[1],
+            "launch_shape": {"block_threads": launched["block_threads"], "blocks": launched["blocks"],
                              "iteration": ["auto", "short", "long"][ctx.get_launch()[2]],
                              "paths_per_lane_claim": ctx.get_claim() or "auto",
                              "chosen_by": "pdd_autotune on 1/8 of the finest level" if tuned[2]

@@ -487,15 +487,19 @@ int pdd_balanced_plan(int64_t n_nodes, double a, double q, double delta, const d
 int pdd_schedule_predict(const pdd_schedule_args* s, double a, double aj, double* rho2,
                          double* cost);
 
-/* Autotuner: runs `sample` (device coordinates) under candidate launch shapes
-   (128/256/512 threads per block, full and half occupancy) with the automatic
-   iteration and claim, then the fastest shape with the short and the long
-   iteration (pdd_ctx_set_iteration; FP32 paths), then with claims of 1, 4 and
-   16 paths per lane (pdd_ctx_set_claim), times each with CUDA events on the
-   context's stream, and keeps the fastest as the context's launch shape,
-   iteration and claim.  Outputs (nullable): the chosen shape and its time
-   (pdd_ctx_get_launch gives the iteration, pdd_ctx_get_claim the claim).
-   Results of later calls do not depend on the choice.                       */
+/* Autotuner: runs `sample` (device coordinates) with the automatic settings
+   and under candidate launch shapes (128/256/512 threads per block, full and
+   half occupancy) with the automatic iteration and claim, then the fastest of
+   these with the short and the long iteration (pdd_ctx_set_iteration; FP32
+   paths), then with claims of 1, 4 and 16 paths per lane (pdd_ctx_set_claim),
+   times each with CUDA events on the context's stream, and keeps the fastest;
+   an automatic setting is left only for one that is at least 1 % faster.
+   Outputs (nullable): the fastest explicit shape, and the time of what was kept
+   (pdd_ctx_get_launch gives the iteration, pdd_ctx_get_claim the claim).  Where
+   the automatic shape is kept the context goes on with it, while the output and
+   pdd_ctx_get_launch report the fastest explicit one; passing that one to
+   pdd_ctx_set_launch makes the context use it.  Results of later calls do not
+   depend on the choice.                                                       */
 int pdd_autotune(pdd_problem* problem, const pdd_estimate_args* sample, int* best_threads,
                  int* best_max_blocks, double* best_ms);
 

@@ -85,8 +85,13 @@ struct pdd_ctx {
   bool timing = false;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> events;
   int64_t launches = 0;
-  int block_threads = 0;  // launch shape (0: defaults), set by pdd_ctx_set_launch / pdd_autotune
+  int block_threads = 0;  // launch shape (0: by each launch), set by pdd_ctx_set_launch / pdd_autotune
   int max_blocks = 0;
+  // pdd_autotune found no explicit shape faster than the one by each launch:
+  // that one runs, and the two above report the fastest explicit one
+  bool auto_shape = false;
+  int run_threads() const { return auto_shape ? 0 : block_threads; }
+  int run_blocks() const { return auto_shape ? 0 : max_blocks; }
   int iter_mode = PDD_ITER_AUTO;  // steps per iteration (pdd_ctx_set_iteration / pdd_autotune)
   int claim = 0;  // paths per lane per cursor claim, 0 = automatic (pdd_ctx_set_claim)
   cudaGraphExec_t gexec = nullptr;  // cached graph of the last PDD_FLAG_GRAPH call
@@ -150,8 +155,8 @@ bool ctx_view(pdd_ctx* c, int* device, int* num_sms, int* block_threads, int* ma
   if (!c) return false;
   *device = c->device;
   *num_sms = c->num_sms;
-  *block_threads = c->block_threads;
-  *max_blocks = c->max_blocks;
+  *block_threads = c->run_threads();
+  *max_blocks = c->run_blocks();
   return true;
 }
 pdd_ctx* problem_ctx(pdd_problem* p) { return p ? p->ctx : nullptr; }
@@ -410,8 +415,8 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   pa.err = &hdr->err;
   pa.trunc_total = &hdr->trunc_total;
   pa.y_exp = p->desc.y_rule == PDD_Y_EXP;
-  pa.max_blocks = c->max_blocks;
-  pa.block_threads = c->block_threads;
+  pa.max_blocks = c->run_blocks();
+  pa.block_threads = c->run_threads();
   pa.iter_mode = c->iter_mode;
   pa.claim = c->claim;
   pa.copy_mask = copies - 1;
@@ -1038,8 +1043,8 @@ int pdd_accumulate(pdd_problem* p, const pdd_estimate_args* a, uint64_t path_off
   pa.err = &hdr->err;
   pa.trunc_total = &hdr->trunc_total;
   pa.y_exp = p->desc.y_rule == PDD_Y_EXP;
-  pa.max_blocks = c->max_blocks;
-  pa.block_threads = c->block_threads;
+  pa.max_blocks = c->run_blocks();
+  pa.block_threads = c->run_threads();
   pa.iter_mode = c->iter_mode;
   pa.claim = c->claim;
   pa.n_segs = 1;
@@ -1171,8 +1176,8 @@ static int coupled_launch(pdd_problem* p, const pdd_estimate_args* a, const Leve
   pa.err = &hdr->err;
   pa.trunc_total = &hdr->trunc_total;
   pa.y_exp = p->desc.y_rule == PDD_Y_EXP;
-  pa.max_blocks = c->max_blocks;
-  pa.block_threads = c->block_threads;
+  pa.max_blocks = c->run_blocks();
+  pa.block_threads = c->run_threads();
   pa.iter_mode = c->iter_mode;
   pa.claim = c->claim;
   pa.n_segs = 2;
@@ -1337,6 +1342,7 @@ int pdd_ctx_set_launch(pdd_ctx* c, int block_threads, int max_blocks) {
   std::lock_guard<std::mutex> lk(c->mu);
   c->block_threads = block_threads;
   c->max_blocks = max_blocks;
+  c->auto_shape = false;
   return PDD_OK;
 }
 
@@ -1409,6 +1415,7 @@ int pdd_autotune(pdd_problem* p, const pdd_estimate_args* sample, int* best_thre
   }
   pdd_ctx* c = p->ctx;
   const int old_threads = c->block_threads, old_blocks = c->max_blocks;
+  const bool old_auto = c->auto_shape;
   const size_t n = (size_t)sample->n_nodes;
   if (n == 0) {
     set_error("pdd_autotune: empty sample");
@@ -1427,11 +1434,11 @@ int pdd_autotune(pdd_problem* p, const pdd_estimate_args* sample, int* best_thre
   a.flags &= ~(PDD_FLAG_EMIT_PATHS | PDD_FLAG_ASYNC);
   const int old_iter = c->iter_mode, old_claim = c->claim;
   int rc = PDD_OK;
-  // CUDA-event time of the sample under the context's current settings (the
-  // first of two runs warms up)
+  // CUDA-event time of the sample under the context's current settings: the
+  // faster of two runs after one that warms up
   auto time_one = [&]() -> double {
-    double ms = 0.0;
-    for (int rep = 0; rep < 2 && rc >= 0; ++rep) {
+    double ms = 1e300;
+    for (int rep = 0; rep < 3 && rc >= 0; ++rep) {
       cudaEvent_t e0, e1;
       {
         DeviceGuard g(c->device);
@@ -1446,7 +1453,7 @@ int pdd_autotune(pdd_problem* p, const pdd_estimate_args* sample, int* best_thre
         cudaEventSynchronize(e1);
         float f = 0.f;
         cudaEventElapsedTime(&f, e0, e1);
-        ms = f;
+        if (rep > 0 && f < ms) ms = f;
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
       }
@@ -1454,10 +1461,16 @@ int pdd_autotune(pdd_problem* p, const pdd_estimate_args* sample, int* best_thre
     return ms;
   };
   const int threads_c[3] = {128, 256, 512};
-  int bt = 0, bb = 0, bi = PDD_ITER_AUTO;
+  int bt = 0, bb = 0, bi = PDD_ITER_AUTO, bc = 0;
   double bms = 1e300;
+  // The automatic settings, which follow every later launch's own size, are left
+  // only for a gain above the noise of two runs (64 FP64 nodes x 1,000 paths: 3.2
+  // ms by the launch's size, 3.4 to 3.5 with the fastest explicit shape).
+  constexpr double kGain = 0.99;
   pdd_ctx_set_iteration(c, PDD_ITER_AUTO);
   pdd_ctx_set_claim(c, 0);
+  pdd_ctx_set_launch(c, 0, 0);
+  const double auto_ms = time_one();
   for (int ti = 0; ti < 3 && rc >= 0; ++ti) {
     // full occupancy, and half of it (fewer resident warps, less L1 pressure)
     for (int frac = 0; frac < 2 && rc >= 0; ++frac) {
@@ -1477,27 +1490,34 @@ int pdd_autotune(pdd_problem* p, const pdd_estimate_args* sample, int* best_thre
       }
     }
   }
+  const bool by_launch = !(bms < kGain * auto_ms);
+  if (by_launch) bms = auto_ms;
+  auto set_shape = [&](int threads, int blocks, bool automatic) {
+    pdd_ctx_set_launch(c, threads, blocks);
+    std::lock_guard<std::mutex> lk(c->mu);
+    c->auto_shape = automatic;
+  };
+  set_shape(bt, bb, by_launch);
   // the scheduling quantum (steps per iteration) at the fastest shape
   if (rc >= 0 && p->desc.precision == PDD_PATH_FP32) {
-    pdd_ctx_set_launch(c, bt, bb);
+    const double base = bms;
     for (int mode : {PDD_ITER_SHORT, PDD_ITER_LONG}) {
       pdd_ctx_set_iteration(c, mode);
       const double ms = time_one();
-      if (rc >= 0 && ms < bms) {
+      if (rc >= 0 && ms < bms && ms < kGain * base) {
         bms = ms;
         bi = mode;
       }
     }
   }
   // paths per lane per cursor claim (the automatic choice was timed above)
-  int bc = 0;
   if (rc >= 0) {
-    pdd_ctx_set_launch(c, bt, bb);
     pdd_ctx_set_iteration(c, bi);
+    const double base = bms;
     for (int claim : {1, 4, 16}) {
       pdd_ctx_set_claim(c, claim);
       const double ms = time_one();
-      if (rc >= 0 && ms < bms) {
+      if (rc >= 0 && ms < bms && ms < kGain * base) {
         bms = ms;
         bc = claim;
       }
@@ -1508,12 +1528,11 @@ int pdd_autotune(pdd_problem* p, const pdd_estimate_args* sample, int* best_thre
     cudaFree(dmean);
   }
   if (rc < 0) {
-    pdd_ctx_set_launch(c, old_threads, old_blocks);
+    set_shape(old_threads, old_blocks, old_auto);
     pdd_ctx_set_iteration(c, old_iter);
     pdd_ctx_set_claim(c, old_claim);
     return rc;
   }
-  pdd_ctx_set_launch(c, bt, bb);
   pdd_ctx_set_iteration(c, bi);
   pdd_ctx_set_claim(c, bc);
   if (best_threads) *best_threads = bt;
