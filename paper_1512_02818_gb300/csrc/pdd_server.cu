@@ -104,6 +104,14 @@ class Arena {
 
 enum class RState { kPending, kActive, kFinishing, kDone, kFailed, kCancelled };
 
+// The inputs of the requests of one admission are in place.
+struct Staged {
+  cudaEvent_t ev = nullptr;
+  ~Staged() {
+    if (ev) cudaEventDestroy(ev);
+  }
+};
+
 struct Request {
   uint64_t ticket = 0;
   pdd_problem* prob = nullptr;
@@ -126,6 +134,7 @@ struct Request {
   bool has_mem = false;
   int inflight = 0;  // in-flight launches that reference this request
   bool in_active = false;  // in the running batch (until the scheduler drops it)
+  std::shared_ptr<Staged> staged;  // inputs and cleared records; null once known to be there
   cudaEvent_t done = nullptr;  // results in host memory
   Clock::time_point t_submit, t_done;
   double est_steps = 0;  // expected steps per path (for slicing)
@@ -159,7 +168,6 @@ struct pdd_server {
   pdd_server_desc desc{};
   cudaStream_t stream[2] = {nullptr, nullptr};
   cudaStream_t copy_stream = nullptr;
-  cudaEvent_t staged = nullptr;  // inputs of every request admitted so far
   int next_stream = 0;
   char* dev_arena = nullptr;
   char* host_arena = nullptr;  // page-locked: a request's coordinates, later its results
@@ -402,13 +410,18 @@ void admit(pdd_server* s) {
     s->st.admitted++;
   }
   if (entered.empty()) return;
-  // cleared records and inputs of the small ones in one launch, before every path
-  // launch by `staged` (memset, copies and event of eleven small requests held
-  // their launch up by 54 us)
+  // cleared records and inputs of the small ones in one launch, before the
+  // requests' path launches by `staged` (memset, copies and event of eleven small
+  // requests held their launch up by 54 us)
   cudaError_t e = cudaSuccess;
+  const auto staged = std::make_shared<Staged>();
   if (n_stage > 0) e = launch_stage_requests(stage, n_stage, s->copy_stream);
-  if (e == cudaSuccess) e = cudaEventRecord(s->staged, s->copy_stream);
-  if (e == cudaSuccess) return;
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&staged->ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(staged->ev, s->copy_stream);
+  if (e == cudaSuccess) {
+    for (Request* r : entered) r->staged = staged;
+    return;
+  }
   for (Request* r : entered) {
     r->next_path = r->n_paths;  // dropped from the batch by the next retirement
     s->st.admitted--;
@@ -498,9 +511,19 @@ bool issue_launch(pdd_server* s) {
   unsigned long long begin = 0;
   int ns = 0;
   Launch L;
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->staged, 0);
+  const Staged* waited = nullptr;
   for (size_t bi = 0; bi < batch.size(); ++bi) {
     Request* r = batch[bi];
+    // after the staging of its own requests (one event an admission), not of others
+    if (r->staged && r->staged.get() != waited) {
+      if (cudaEventQuery(r->staged->ev) == cudaSuccess) {
+        r->staged.reset();
+      } else {
+        (void)cudaGetLastError();  // not ready is no error
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, r->staged->ev, 0);
+        waited = r->staged.get();
+      }
+    }
     const uint64_t m = take[bi];
     SegArgs& sg = pa.seg[ns++];
     sg.cx = req_coord(s, *r, 0);
@@ -743,7 +766,6 @@ int pdd_server_create(pdd_ctx* ctx, const pdd_server_desc* desc, pdd_server** ou
   for (int i = 0; i < 2 && e == cudaSuccess; ++i)
     e = cudaStreamCreateWithFlags(&s->stream[i], cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->staged, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->pilot_stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
     set_error("pdd_server_create: %s", cudaGetErrorString(e));
@@ -756,7 +778,6 @@ int pdd_server_create(pdd_ctx* ctx, const pdd_server_desc* desc, pdd_server** ou
     for (auto& x : s->stream)
       if (x) cudaStreamDestroy(x);
     if (s->copy_stream) cudaStreamDestroy(s->copy_stream);
-    if (s->staged) cudaEventDestroy(s->staged);
     if (s->pilot_stream) cudaStreamDestroy(s->pilot_stream);
     return e == cudaErrorMemoryAllocation ? PDD_ERR_NOMEM : PDD_ERR_CUDA;
   }
@@ -1030,7 +1051,6 @@ void pdd_server_destroy(pdd_server* s) {
   cudaFreeHost(s->pilot_host);
   for (auto& x : s->stream) cudaStreamDestroy(x);
   cudaStreamDestroy(s->copy_stream);
-  cudaEventDestroy(s->staged);
   cudaStreamDestroy(s->pilot_stream);
   delete s;
 }
