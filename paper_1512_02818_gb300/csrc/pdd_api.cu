@@ -81,6 +81,7 @@ struct pdd_ctx {
   int num_sms = 0;
   void* ws = nullptr;  // workspace: header | node records | coords | staged outputs
   size_t ws_size = 0;
+  size_t ws_refused = SIZE_MAX;  // with record copies: a size that the device had no room for
   std::mutex mu;
   bool timing = false;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> events;
@@ -381,18 +382,26 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
               (outs[l].on_device ? 0 : 14 * align_up((size_t)levels[l].n_nodes * 8, 256));
     while (copies > 1 && rest + copies * rec_bytes > c->budget) copies /= 2;
   }
-  size_t off = align_up(off_acc + copies * rec_bytes, 256);
+  size_t off = 0, coords_at = 0, outs_at = 0;
   size_t coord_off[PDD_MAX_LEVELS], out_off[PDD_MAX_LEVELS];
-  const size_t coords_at = off;
-  for (int l = 0; l < n_levels; ++l) {
-    coord_off[l] = off;
-    if (!levels[l].coords_on_device) off += align_up((size_t)levels[l].n_nodes * 4, 256) * dim;
-  }
-  const size_t outs_at = off;
-  for (int l = 0; l < n_levels; ++l) {
-    out_off[l] = off;
-    if (!outs[l].on_device) off += 14 * align_up((size_t)levels[l].n_nodes * 8, 256);
-  }
+  auto lay_out = [&] {
+    off = coords_at = align_up(off_acc + copies * rec_bytes, 256);
+    for (int l = 0; l < n_levels; ++l) {
+      coord_off[l] = off;
+      if (!levels[l].coords_on_device) off += align_up((size_t)levels[l].n_nodes * 4, 256) * dim;
+    }
+    outs_at = off;
+    for (int l = 0; l < n_levels; ++l) {
+      out_off[l] = off;
+      if (!outs[l].on_device) off += 14 * align_up((size_t)levels[l].n_nodes * 8, 256);
+    }
+  };
+  lay_out();
+  auto without_copies = [&] {
+    copies = 1;
+    lay_out();
+  };
+  if (copies > 1 && off >= c->ws_refused) without_copies();
   // through page-locked memory where they fit (see kPinnedIn)
   const bool pin_in = outs_at - coords_at <= kPinnedIn;
   const bool pin_out = off - outs_at <= kPinnedOut;
@@ -400,6 +409,12 @@ static int estimate_impl(pdd_problem* p, int n_levels, const pdd_estimate_args* 
   char* const host_in = c->pinned + kPinnedHeader;
   char* const host_out = host_in + kPinnedIn;
   int rc = ensure_workspace(c, off);
+  if (rc == PDD_ERR_NOMEM && copies > 1) {  // no room on the device: without the copies
+    (void)cudaGetLastError();
+    c->ws_refused = off;
+    without_copies();
+    rc = ensure_workspace(c, off);
+  }
   if (rc != PDD_OK) return rc;
   char* ws = (char*)c->ws;
   WsHeader* hdr = (WsHeader*)ws;
