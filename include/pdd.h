@@ -222,8 +222,8 @@ int pdd_ctx_set_launch(pdd_ctx* ctx, int block_threads, int max_blocks);
    more steps; a lane whose path ends early in an iteration idles for the rest
    of it.  Like the launch shape, the choice changes only the speed (results
    are exact sums keyed by node and path).  pdd_autotune sets it too.
-   pdd_ctx_get_launch reads the context's shape and iteration choice (any
-   output may be NULL).                                                     */
+   pdd_ctx_get_launch reads the context's shape (after pdd_autotune: see there)
+   and iteration choice (any output may be NULL).                           */
 #define PDD_ITER_AUTO 0
 #define PDD_ITER_SHORT 1
 #define PDD_ITER_LONG 2

@@ -62,7 +62,7 @@ int pdd_debug_bounds_selftest(uint32_t* bits);
    coupled calls; no counterpart in the paper): blocks, threads per block, node
    records kept in every block's shared memory (0: none), and paths per warp of
    a launch whose warps take one batch each (0: the others).  Zeros before the
-   first launch; any output may be NULL.                                      */
+   first launch; host pointers, any of which may be NULL.                     */
 int pdd_debug_last_launch(pdd_ctx* ctx, int* blocks, int* block_threads, int* cached_records,
                           int* paths_per_warp);
 
